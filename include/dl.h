@@ -258,17 +258,19 @@ DL_API dl_status dl_tail_system(dl_ctx *ctx, int32_t n, int32_t m, const dl_tail
  * Sec. 6.3 for a unique solution), else DL_EINVAL.  out_stilde: n x n doubles, row-major
  * (required).  out_bits (optional, NULL allowed): the model, S~ > 0 made exact by the
  * boolean iteration (n * ceil(n/64) words).  mem: where P, B and both outputs live.
- * Paths: DL_PATH_FP64 -- the fixpoint series X <- eps (B + P X P^T) in FP64 until a step
+ * Paths: a P that is acyclic in at most 64 layers of short parent lists is solved in the order of
+ * its layers on DL_PATH_FP64 and DL_PATH_AUTO (every entry once; what the series ends with).
+ * Otherwise DL_PATH_FP64 -- the fixpoint series X <- eps (B + P X P^T) in FP64 until a step
  * changes nothing beyond refine_tol * eps (exact after depth + 1 steps when P is nilpotent);
  * DL_PATH_MIXED -- Smith's doubling on the TF32 tensor cores with FP64 refinement (device
  * workspace about (2K + 4) np^2 FP32 matrices, K the doubling steps, np = n rounded up to 256);
  * DL_PATH_AUTO -- the series, then the refinement if 64 steps did not converge.
  * DL_PATH_BOOL_FP8: DL_EINVAL (no real values).  n is limited to 29000 (a row of S~ in one
  * block's shared memory); DL_ENOTCONV if the series or the refinement does not converge.
- * stats: iters = series steps + refinement steps, final_resid = max|eps (B + P S P^T) - S|/eps
+ * stats: iters = layers, or series steps + refinement steps, final_resid = max|eps (B + P S P^T) - S|/eps
  * (after the series: a power-of-two bound on the last step's largest change, 0 if it changed
  * nothing),
- * path_used = DL_PATH_FP64 when the series alone sufficed, else DL_PATH_MIXED.
+ * path_used = DL_PATH_FP64 when the series (or the layers) alone sufficed, else DL_PATH_MIXED.
  */
 DL_API dl_status dl_sg_real(dl_ctx *ctx, int32_t n, const uint8_t *P, const uint8_t *B, dl_mem mem, double eps,
                      dl_path path, double *out_stilde, uint64_t *out_bits, dl_stats *stats);

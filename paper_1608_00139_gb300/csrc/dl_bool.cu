@@ -13,7 +13,9 @@
 // (the fact with the shortest derivation that is missing has its successor's fact present).
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
+#include <cstring>
 
 #include "dl_internal.h"
 #include "dl_ptx.cuh"
@@ -487,13 +489,125 @@ __global__ void __launch_bounds__(256)
     }
 }
 
-// Ones in rows < n of a bit matrix.
-__global__ void bits_count_kernel(const uint64_t *__restrict__ M, int n, int64_t wp, unsigned long long *ones) {
-    const int64_t t = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-    uint32_t c = t < static_cast<int64_t>(n) * wp ? __popcll(M[t]) : 0u;
+// One level of an acyclic P, a CTA per row i: the OR u of the (final) rows of i's parents goes to
+// shared memory, then lane j looks up whether a parent of j lies in u (one bit from shared memory
+// per parent of j; the first two, nearly always all, come from a coalesced array) and a ballot
+// makes 32 columns' word.  Every row is formed once, where the Iteration forms all of them in
+// every step and the doubling multiplies n x n matrices.  Latency-bound: a level is one launch and
+// a row's chain is its parents' words, a barrier and one look-up; everything that does not depend
+// on the levels below (the parent lists, the first kLevelCols columns' parents of each thread and
+// the row's own words) is loaded before the wait for them, while they still run.
+// REAL: the warp then queues its columns of S_i (few: S is sparse in a forest) and its lanes form
+// their entries of S~ from the parents' rows, so that the FP64 products (two lanes per SM) and the
+// reads are per fact and not per entry; the zeros are a fill before the first level.  Staging a
+// parent's whole row and writing whole rows instead took 3.3 us per row and SM, 219 us for the 17
+// levels of a forest of 4096.
+constexpr int kLevelThreads = 512;
+constexpr int kLevelCols = 8;  // columns per thread and pass (4096 a pass)
+
+template <bool REAL>
+__global__ void __launch_bounds__(kLevelThreads, REAL ? 3 : 2)
+    sg_level_kernel(const int *__restrict__ ptr, const int *__restrict__ col, const short2 *__restrict__ first2,
+                    const int *__restrict__ order, int n, int wp, uint64_t *S, double *X, double eps,
+                    long long tau_bits, unsigned long long *guard) {
+    extern __shared__ uint64_t parents_s[];  // wp words
+    __shared__ int2 queue_s[REAL ? kLevelThreads / 32 : 1][REAL ? 32 * kLevelCols : 1];  // column, its first two parents
+    grid_dep_launch();
+    const int i = order[blockIdx.x];
+    const int q0 = ptr[i], q1 = ptr[i + 1];
+    const int y0 = q1 > q0 ? col[q0] : 0;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t *row = reinterpret_cast<uint32_t *>(S + static_cast<int64_t>(i) * wp);
+    const uint32_t *u32 = reinterpret_cast<const uint32_t *>(parents_s);
+    double *xrow = REAL ? X + static_cast<int64_t>(i) * n : nullptr;
+    unsigned small = 0;  // entries in the guard band
+    for (int base = 0; base < n; base += kLevelThreads * kLevelCols) {
+        short2 par[kLevelCols];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-    if ((threadIdx.x & 31) == 0 && c) atomicAdd(ones, static_cast<unsigned long long>(c));
+        for (int c = 0; c < kLevelCols; ++c) {
+            const int j = base + c * kLevelThreads + static_cast<int>(threadIdx.x);
+            par[c] = q1 > q0 && j < n ? first2[j] : make_short2(-1, -1);
+        }
+        // lane c holds the word of the warp's c-th 32 columns
+        const int word = base / 32 + lane * (kLevelThreads / 32) + warp;
+        const bool holds = lane < kLevelCols && word < 2 * wp;
+        const uint32_t have = holds ? row[word] : 0u;
+        if (base == 0) {
+            grid_dep_wait();  // the levels below are final
+            for (int w = threadIdx.x; w < wp; w += kLevelThreads) {
+                uint64_t u = q1 > q0 ? S[static_cast<int64_t>(y0) * wp + w] : 0ull;
+                for (int q = q0 + 1; q < q1; ++q) u |= S[static_cast<int64_t>(col[q]) * wp + w];
+                parents_s[w] = u;
+            }
+            __syncthreads();
+        }
+        uint32_t got = 0u;  // lane c: the parents' part of word c
+        int queued = 0;
+#pragma unroll
+        for (int c = 0; c < kLevelCols; ++c) {
+            const int j = base + c * kLevelThreads + static_cast<int>(threadIdx.x);
+            bool hit = par[c].x >= 0 && ((u32[par[c].x >> 5] >> (par[c].x & 31)) & 1u);
+            if (par[c].y >= 0) hit |= (u32[par[c].y >> 5] >> (par[c].y & 31)) & 1u;
+            if (par[c].y == -2) {  // more than two parents
+                const int r1 = ptr[j + 1];
+                for (int r = ptr[j] + 1; r < r1 && !hit; ++r) hit = (u32[col[r] >> 5] >> (col[r] & 31)) & 1u;
+            }
+            const uint32_t bits = __ballot_sync(0xffffffffu, hit);
+            if (lane == c) got = bits;
+            if (REAL) {
+                const uint32_t b = __shfl_sync(0xffffffffu, have, c), all = bits | b;
+                if ((all >> lane) & 1u) {  // x: the column, bit 30: B, bit 31: no parent pair
+                    const int flags = static_cast<int>(((b >> lane) & 1u) << 30) | static_cast<int>(hit ? 0u : 1u << 31);
+                    const int w = (static_cast<int>(static_cast<unsigned short>(par[c].x)) << 16) |
+                                  static_cast<int>(static_cast<unsigned short>(par[c].y));
+                    queue_s[warp][queued + __popc(all & ((1u << lane) - 1u))] = make_int2(j | flags, w);
+                }
+                queued += __popc(all);
+            }
+        }
+        if (holds && (got & ~have) != 0u) row[word] = have | got;
+        if (REAL) {
+            __syncwarp();
+            for (int k = lane; k < queued; k += 32) {
+                const int2 e = queue_s[warp][k];
+                const int j = e.x & 0x3FFFFFFF;
+                const int w0 = static_cast<short>(e.y >> 16), w1 = static_cast<short>(e.y);
+                double v = 1.0;
+                if (e.x >= 0) {
+                    double s = 0.0;
+                    for (int q = q0; q < q1; ++q) {
+                        const double *xr = X + static_cast<int64_t>(q == q0 ? y0 : col[q]) * n;
+                        s = q == q0 ? xr[w0] : s + xr[w0];  // a first term is assigned, not added to 0
+                        if (w1 >= 0) s += xr[w1];
+                        if (w1 == -2)
+                            for (int r = ptr[j] + 1; r < ptr[j + 1]; ++r) s += xr[col[r]];
+                    }
+                    v = (e.x >> 30) & 1 ? s + 1.0 : s;
+                }
+                v *= eps;
+                xrow[j] = v;
+                small += __double_as_longlong(v) <= tau_bits;  // positive doubles compare as integers
+            }
+            __syncwarp();  // the queue is refilled by the next pass
+        }
+    }
+    if (REAL) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) small += __shfl_xor_sync(0xffffffffu, small, o);
+        if (lane == 0 && small) atomicAdd(guard, static_cast<unsigned long long>(small));
+    }
+}
+
+// Ones in rows < n of a bit matrix.
+__global__ void __launch_bounds__(256) bits_count_kernel(const uint64_t *M, int n, int64_t wp,
+                                                         unsigned long long *ones) {
+    const int64_t words = static_cast<int64_t>(n) * wp;
+    uint32_t c = 0, none = 0;
+    for (int64_t t = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; t < words;
+         t += static_cast<int64_t>(gridDim.x) * blockDim.x)
+        c += __popcll(M[t]);
+    block_reduce_sum_or(c, none);  // one atomic per CTA: an atomic per warp on one address took longer than the reads
+    if (threadIdx.x == 0 && c) atomicAdd(ones, static_cast<unsigned long long>(c));
 }
 
 // Rows < n get the identity, every other word is zero (np rows).
@@ -624,10 +738,24 @@ cudaError_t bits_gather(const int *ptr, const int *col, const int *unit_off, int
     return cudaGetLastError();
 }
 
+cudaError_t sg_level(const int *ptr, const int *col, const short2 *first2, const int *order, int count, int n,
+                     int64_t wp, uint64_t *S, double *X, double eps, double tau, unsigned long long *guard,
+                     cudaStream_t s) {
+    if (count <= 0) return cudaSuccess;
+    if (wp > 1024) return cudaErrorInvalidValue;  // the parents' row in 8 KB of shared memory beside the queues
+    long long tau_bits = 0;
+    std::memcpy(&tau_bits, &tau, sizeof tau);
+    const size_t smem = static_cast<size_t>(wp) * sizeof(uint64_t);
+    auto *kernel = X != nullptr ? sg_level_kernel<true> : sg_level_kernel<false>;
+    return launch_programmatic(kernel, dim3(static_cast<unsigned>(count)), dim3(kLevelThreads), smem, s, ptr, col,
+                               first2, order, n, static_cast<int>(wp), S, X, eps, tau_bits, guard);
+}
+
 cudaError_t bits_count(const uint64_t *M, int n, int64_t wp, unsigned long long *ones, cudaStream_t s) {
     const int64_t words = static_cast<int64_t>(n) * wp;
     if (words <= 0) return cudaSuccess;
-    bits_count_kernel<<<static_cast<unsigned>((words + 255) / 256), 256, 0, s>>>(M, n, wp, ones);
+    const int64_t blocks = std::min<int64_t>((words + 255) / 256, 4 * num_sms());
+    bits_count_kernel<<<static_cast<unsigned>(blocks), 256, 0, s>>>(M, n, wp, ones);
     return cudaGetLastError();
 }
 

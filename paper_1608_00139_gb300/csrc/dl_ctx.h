@@ -126,6 +126,7 @@ struct SolveArgs {
     const double *rhs_real = nullptr;  // a real right-hand side F of X = eps (F + E X) instead
                                        // (device, n x n FP64, row stride n; FP64 / mixed paths)
     double rhs_bound = 1.0;        // a bound on |F| (the mixed residual's fixed-point scale)
+    bool no_layers = false;        // same generation: leave out the layer-by-layer route
     bool skip_recheck = false;     // real paths: leave X > 0 in the bits unchecked, count its ones
     const uint8_t *E2 = nullptr;  // same generation: B (may be null); compose: R2
     dl_mem mem = DL_MEM_HOST;

@@ -293,7 +293,120 @@ __global__ void csr_fill_kernel(const uint8_t *__restrict__ E, int n, const int 
     }
 }
 
+// Layers of an acyclic relation: node i's level is 0 without successors, else one more than its
+// highest successor's (the successor lists of the same-generation relation are the parents).  One
+// CTA peels them: in round t every open node whose successors all have a level below t takes level t
+// and, since the rounds follow one another, its place in the order; a round that places nothing
+// while nodes are open has met a cycle, and kMaxLevels rounds without an end are given up as well
+// (info[0] = 0 either way).  Bound by the latency of one warp's chain in a round, so a thread looks
+// the levels of the first two successors (nearly always the whole list) of all its nodes up at once,
+// and a warp places all its nodes with one scan and one atomic: 22 rounds over 4096 nodes took
+// 55000 cycles with a test, a ballot and an atomic per node.
+template <int NODES>
+__global__ void __launch_bounds__(1024)
+    dag_levels_kernel(const int *__restrict__ ptr, const int *__restrict__ col, int n, const int *gate, int *info,
+                      int *order, short2 *first2) {
+    extern __shared__ uint8_t level_s[];  // n levels, then one 0 (the level looked up for a missing successor)
+    constexpr int kOpen = 0xFF;
+    __shared__ int cnt_s[kMaxLevels];
+    if (gate != nullptr && *gate != 0) {  // no successor lists: nothing to do
+        if (threadIdx.x == 0) info[0] = 0;
+        return;
+    }
+    const int lane = threadIdx.x & 31;
+    if (threadIdx.x < kMaxLevels) cnt_s[threadIdx.x] = 0;
+    for (int i = threadIdx.x; i <= n; i += 1024) level_s[i] = i < n ? kOpen : 0;
+    int first[NODES], deg[NODES];
+#pragma unroll
+    for (int k = 0; k < NODES; ++k) {
+        const int i = k * 1024 + static_cast<int>(threadIdx.x);
+        first[k] = i < n ? ptr[i] : 0;
+        deg[k] = i < n ? ptr[i + 1] - first[k] : 0;
+    }
+    short2 mine[NODES];  // the slots to look up: a missing successor's is n
+    unsigned open = 0, more = 0;  // bit k: this thread's node k has no level yet; has more than two successors
+#pragma unroll
+    for (int k = 0; k < NODES; ++k) {
+        const int i = k * 1024 + static_cast<int>(threadIdx.x);
+        const int x = deg[k] > 0 ? col[first[k]] : -1, y = deg[k] > 2 ? -2 : deg[k] == 2 ? col[first[k] + 1] : -1;
+        mine[k] = make_short2(static_cast<short>(x >= 0 ? x : n), static_cast<short>(y >= 0 ? y : n));
+        if (y == -2) more |= 1u << k;
+        if (i < n) {
+            open |= 1u << k;
+            first2[i] = make_short2(static_cast<short>(x), static_cast<short>(y));
+        }
+    }
+    __syncthreads();
+    int t = 0, base = 0;  // base: nodes placed before round t
+    for (; base < n && t < kMaxLevels; ++t) {
+        if (threadIdx.x == 0) info[1 + t] = base;
+        if (__any_sync(0xffffffffu, open != 0)) {
+            // the nodes whose successors all have a level below t: a level written in this round is
+            // t, an open one kOpen, and neither is below t
+            unsigned go = 0;
+#pragma unroll
+            for (int k = 0; k < NODES; ++k) {  // (a placed node looks the common slot up: no bank conflicts)
+                const bool o = (open >> k) & 1u;
+                if (max(level_s[o ? mine[k].x : n], level_s[o ? mine[k].y : n]) < t || t == 0) go |= 1u << k;
+            }
+            go &= open;
+            if (t == 0) {  // no successors at all
+#pragma unroll
+                for (int k = 0; k < NODES; ++k)
+                    if (mine[k].x != n) go &= ~(1u << k);
+            }
+            if (__any_sync(0xffffffffu, (go & more) != 0)) {
+                for (unsigned left = go & more; left != 0; left &= left - 1) {
+                    const int k = __ffs(left) - 1, i = k * 1024 + static_cast<int>(threadIdx.x);
+                    for (int q = ptr[i] + 1; q < ptr[i + 1]; ++q)
+                        if (level_s[col[q]] >= t) {
+                            go &= ~(1u << k);
+                            break;
+                        }
+                }
+            }
+            open &= ~go;
+            int at = __popc(go);
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int v = __shfl_up_sync(0xffffffffu, at, o);
+                if (lane >= o) at += v;
+            }
+            const int all = __shfl_sync(0xffffffffu, at, 31);
+            if (all != 0) {
+                int start = 0;
+                if (lane == 0) start = atomicAdd(&cnt_s[t], all);
+                at += base + __shfl_sync(0xffffffffu, start, 0) - __popc(go);
+                for (; go != 0; go &= go - 1) {
+                    const int i = (__ffs(go) - 1) * 1024 + static_cast<int>(threadIdx.x);
+                    order[at++] = i;
+                    level_s[i] = static_cast<uint8_t>(t);
+                }
+            }
+        }
+        __syncthreads();
+        const int now = cnt_s[t];  // (final: the next round counts in its own slot)
+        if (now == 0) break;       // a cycle
+        base += now;
+    }
+    if (threadIdx.x == 0) {
+        info[1 + t] = base;
+        info[0] = base == n ? t : 0;
+    }
+}
+
 }  // namespace
+
+bool dag_levels_fit(int n) { return n > 0 && n < (1 << 15); }  // (first2 holds 16-bit node numbers)
+
+cudaError_t dag_levels(const int *ptr, const int *col, int n, const int *gate, int *info, int *order, short2 *first2,
+                       cudaStream_t s) {
+    if (!dag_levels_fit(n)) return cudaErrorInvalidValue;
+    // nodes per thread: a thread's chain and registers grow with them (17 us for 4 at 17 layers)
+    auto *kernel = n <= 4 * 1024 ? dag_levels_kernel<4> : n <= 16 * 1024 ? dag_levels_kernel<16> : dag_levels_kernel<32>;
+    kernel<<<1, 1024, static_cast<size_t>(n) + 1, s>>>(ptr, col, n, gate, info, order, first2);
+    return cudaGetLastError();
+}
 
 cudaError_t csr_build(const uint8_t *E, int n, int *cnt, int *ptr, cudaStream_t s) {
     csr_count_kernel<<<static_cast<unsigned>((n + 7) / 8), 256, 0, s>>>(E, n, cnt);

@@ -183,6 +183,16 @@ cudaError_t bits_transpose(const uint64_t *src, uint64_t *dst, int np, int64_t w
 cudaError_t bits_gather(const int *ptr, const int *col, const int *unit_off, int n, const uint64_t *src, uint64_t *dst,
                         int64_t wp, int accumulate, unsigned long long *changed, const unsigned long long *skip,
                         cudaStream_t s);
+// Rows order[0 .. count) (one level of P's layers) of the same-generation model S = B | P S P^T
+// in place, row i holding B_i and the rows of i's parents being final:
+//     S_i |= {j < n : some w in succ(j) lies in OR_{y in succ(i)} S_y}.
+// With X (n x n FP64, row stride n, zero where it is not written) also the entries of
+// S~ = eps (B + P S~ P^T) at the bits of S_i, from the parents' rows of X, in the order of additions
+// of the fused series step; *guard += those <= tau (tau > 0).  first2: as written by dag_levels.
+// wp <= 1024.  A programmatic launch.
+cudaError_t sg_level(const int *ptr, const int *col, const short2 *first2, const int *order, int count, int n,
+                     int64_t wp, uint64_t *S, double *X, double eps, double tau, unsigned long long *guard,
+                     cudaStream_t s);
 // *ones += ones in rows < n.
 cudaError_t bits_count(const uint64_t *M, int n, int64_t wp, unsigned long long *ones, cudaStream_t s);
 // M = identity on rows < n, zero elsewhere (np rows).
@@ -229,6 +239,15 @@ cudaError_t csr_fill_from_bits_guarded(const uint64_t *M, int n, int64_t wp, con
 cudaError_t exclusive_scan(const int *cnt, int n, int *out, cudaStream_t s);
 // The same with every SM taking part, for long arrays (scratch: 2 * (ceil(n / 1024) + 1) ints).
 cudaError_t exclusive_scan_large(const int *cnt, int n, int *out, int *scratch, cudaStream_t s);
+// Layers of an acyclic relation from its CSR (level 0: no successors; else one more than the
+// highest successor's), at most kMaxLevels of them.  info (device, 2 + kMaxLevels ints):
+// info[0] = the number of levels L, 0 when the relation has a cycle or more levels (or *gate != 0);
+// info[1 + l] = the first place of level l in order (n nodes sorted by level), info[1 + L] = n.
+// first2[i] = i's first successor (-1 without any) and second one (-1 without, -2 with more than two).
+constexpr int kMaxLevels = 64;
+bool dag_levels_fit(int n);
+cudaError_t dag_levels(const int *ptr, const int *col, int n, const int *gate, int *info, int *order, short2 *first2,
+                       cudaStream_t s);
 
 // ---------------------------------------------------------------------------------------
 // FP64 path (dl_fp64.cu)

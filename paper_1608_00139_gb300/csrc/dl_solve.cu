@@ -37,6 +37,7 @@ namespace dl {
 namespace {
 
 constexpr size_t kHostPinned = 8u << 20;
+constexpr size_t kInfoOffset = 2048;  // of the layers' summary in the pinned staging
 constexpr size_t kTableOffset = 4096;
 
 int64_t round_up(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
@@ -918,14 +919,59 @@ dl_status solve_tc(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &
     return rc;
 }
 
+// The layers of an acyclic relation with short successor lists (dag_levels), found on the device
+// right after the pass that packed its bits, before the host knows the number of facts: read()
+// is valid after the stream's next synchronisation.  Rows of more than kLayerDeg successors (or
+// more facts than the column array holds) stop it on the device.
+constexpr int kLayerDeg = 16;
+
+struct Layers {
+    int *col = nullptr, *order = nullptr;
+    short2 *first2 = nullptr;
+    const int *info = nullptr;  // pinned copy: the number of levels and their first places
+    bool filled = false;        // the successor lists are in col
+    int levels() const { return info ? info[0] : 0; }
+    int count(int l) const { return info[2 + l] - info[1 + l]; }
+    const int *rows(int l) const { return order + info[1 + l]; }
+};
+
+dl_status layers_enqueue(Workspace &ws, cudaStream_t s, const uint64_t *bits, int32_t n, int64_t wp, const int *ptr,
+                         Layers *ly) {
+    const int64_t np = wp * 64;
+    const size_t want = std::max(ws.capacity("g_col"), static_cast<size_t>(np) * 8 * sizeof(int));
+    ly->col = static_cast<int *>(ws.get("g_col", want));
+    ly->order = static_cast<int *>(ws.get("g_order", np * sizeof(int)));
+    ly->first2 = static_cast<short2 *>(ws.get("g_first2", np * sizeof(short2)));
+    auto *info = static_cast<int *>(ws.get("g_info", (kMaxLevels + 2) * sizeof(int)));
+    NEED(ly->col && ly->order && ly->first2 && info);
+    int *gate = reinterpret_cast<int *>(ws.scal + SC_GATE);
+    CK(csr_fill_from_bits_guarded(bits, n, wp, ptr, ly->col, static_cast<int64_t>(ws.capacity("g_col") / sizeof(int)),
+                                  ws.scal + SC_DMAX, kLayerDeg, gate, s));
+    CK(dag_levels(ptr, ly->col, n, gate, info, ly->order, ly->first2, s));
+    auto *h = reinterpret_cast<int *>(static_cast<char *>(ws.host_pinned) + kInfoOffset);
+    CK(cudaMemcpyAsync(h, info, (kMaxLevels + 2) * sizeof(int), cudaMemcpyDeviceToHost, s));
+    ly->info = h;
+    return DL_OK;
+}
+
+// After the scalars have been read: whether the successor lists were written.
+void layers_read(Workspace &ws, Layers *ly) {
+    ly->filled = ly->info && *reinterpret_cast<const int *>(host_scal(ws) + SC_GATE) == 0;
+    if (!ly->filled) ly->info = nullptr;
+}
+
 // Same generation by the Iteration method on bits: S_{t+1} = B | P S_t P^T, from S_0 = B
 // (Kleene iteration from below, so an iteration that changes nothing has reached the least
 // fixpoint).  One iteration: Y = P S_t^T (rows of P gather rows of S^T), X = Y^T = S_t P^T,
 // S |= P X (rows of P gather rows of X); when B is symmetric so is every S_t and S^T = S.
+// When P is acyclic in few layers of short parent lists (a forest, a shallow DAG), the rows are
+// formed layer by layer instead, each once, from the final rows of its parents (sg_level):
+// forest N = 4096, 17 layers, one call: 0.85 ms by the doubling, 0.21 ms here.
+// Otherwise, and unless iterate is set, it returns at once.
 // Returns with *done = false (and nothing written) if the rows are too wide or the
 // iterations exceed the budget: the doubling below then solves the problem.
 dl_status sg_iteration(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &a, dl_stats *st, bool *done,
-                       const uint64_t *seed = nullptr) {
+                       bool iterate = true, const uint64_t *seed = nullptr) {
     (void)ctx;
     *done = false;
     const int32_t n = a.n;
@@ -968,28 +1014,45 @@ dl_status sg_iteration(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveAr
         CK(bits_or(S, seed, np * wp, s));
         ++launches;
     }
+    Layers ly;
+    if (!a.no_layers && !seed && dag_levels_fit(n)) {
+        if ((rc = layers_enqueue(ws, s, X, n, wp, ptr, &ly))) return rc;
+        launches += 2;
+    }
     if ((rc = read_scalars(ws, s))) return rc;
     if ((rc = check_status(ws, s))) return rc;
+    layers_read(ws, &ly);
     const double dmax = static_cast<double>(host_scal(ws)[SC_DMAX]);
     double eps = 0;
     if ((rc = choose_eps(a.eps, 1.0 / (1.0 + dmax * dmax), "Sec. 7.2 (1/(1+||P||^2))", &eps))) return rc;
     const bool sym = seed == nullptr && (Bm == nullptr || host_scal(ws)[SC_CQ] == 0);
     const int64_t nnz = static_cast<int64_t>(host_scal(ws)[SC_NNZ]);
-    auto *col = static_cast<int *>(ws.get("g_col", static_cast<size_t>(std::max<int64_t>(nnz, 1)) * 4));
+    if (!iterate && ly.levels() == 0) return DL_OK;
+    auto *col = ly.filled ? ly.col : static_cast<int *>(ws.get("g_col", static_cast<size_t>(std::max<int64_t>(nnz, 1)) * 4));
     NEED(col);
-    CK(csr_fill_from_bits(X, n, wp, ptr, col, s));
-    ++launches;
+    if (!ly.filled) {
+        CK(csr_fill_from_bits(X, n, wp, ptr, col, s));
+        ++launches;
+    }
     const int *units = nullptr;  // rows of more than 64 parents: edge-parallel gathers
     if (dmax > 64) {
         CK(sweep_units(ptr, n, cnt, uoff, s));
         launches += 2;
         units = uoff;
     }
-    CK(cudaMemsetAsync(Y, 0, np * wp * 8, s));  // rows >= n stay zero (the gathers write rows < n)
+    if (ly.levels() == 0)
+        CK(cudaMemsetAsync(Y, 0, np * wp * 8, s));  // rows >= n stay zero (the gathers write rows < n)
     tm.mark(1);
     unsigned long long *vslot = ws.scal + 32;
     int iters = 0;
     bool converged = false;
+    if (ly.levels() > 0) {  // level 0 (no parents) is B itself
+        for (int l = 1; l < ly.levels(); ++l)
+            CK(sg_level(ptr, col, ly.first2, ly.rows(l), ly.count(l), n, wp, S, nullptr, 0.0, 0.0, nullptr, s));
+        launches += ly.levels() - 1;
+        iters = ly.levels();
+        converged = true;
+    }
     while (!converged) {
         if (iters >= kBudget) return DL_OK;  // deep derivations: doubling instead
         CK(cudaMemsetAsync(vslot, 0, sizeof(unsigned long long) * kGroup, s));
@@ -1055,10 +1118,12 @@ dl_status solve_sg(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &
     // about 0.1 ms of launches, and about ten are needed.  The doubling is cheaper below
     // Np ~ 6000 (measured: 0.9 against 1.3 ms at N = 4096, 5.1 against 2.1 ms at N = 8192).
     const int64_t np = round_up(std::max<int64_t>(a.n, 1), 256);
+    // Layers, where P has them, are cheaper than either (and found by the same preparation).
     const int tuned_iteration = tuned(ctx, np).sg_iteration;  // measured crossover, when tuned
-    if (a.path == DL_PATH_AUTO && (tuned_iteration >= 0 ? tuned_iteration == 1 : np >= 6144)) {
+    const bool iterate = tuned_iteration >= 0 ? tuned_iteration == 1 : np >= 6144;
+    if (a.path == DL_PATH_AUTO && (iterate || !a.no_layers)) {
         bool done = false;
-        const dl_status rc = sg_iteration(ctx, ws, s, a, st, &done);
+        const dl_status rc = sg_iteration(ctx, ws, s, a, st, &done, iterate);
         if (rc != DL_OK || done) return rc;
     }
     return sg_doubling(ctx, ws, s, a, st);
@@ -1234,8 +1299,52 @@ dl_status solve_compose(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveA
     return DL_OK;
 }
 
+// S~ and its model on the layers of P (sg_level), S~ straight into a device output.  S: np x wp bits,
+// B's on entry, the model's on return.  N = 4096 forest, one call: 3.1 ms by the series and the
+// boolean iteration, 0.29 ms here.
+dl_status sg_real_layers(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &a, dl_stats *st,
+                         const Layers &ly, const int *ptr, uint64_t *S, int64_t wp, double eps, Timer *tm,
+                         int launches) {
+    const int32_t n = a.n;
+    const size_t nn = static_cast<size_t>(n) * n;
+    const bool device = a.mem == DL_MEM_DEVICE;
+    double *X = device ? a.out_rtilde : static_cast<double *>(ws.get("sr_X", nn * 8));
+    NEED(X);
+    CK(cudaMemsetAsync(X, 0, nn * 8, s));
+    tm->mark(1);
+    const double tau = ctx->cfg.guard_tau > 0 ? ctx->cfg.guard_tau : 1e-30;
+    for (int l = 0; l < ly.levels(); ++l)
+        CK(sg_level(ptr, ly.col, ly.first2, ly.rows(l), ly.count(l), n, wp, S, X, eps, tau, ws.scal + SC_GUARD, s));
+    launches += ly.levels();
+    tm->mark(2);
+    if (!device) CK(cudaMemcpyAsync(a.out_rtilde, X, nn * 8, cudaMemcpyDeviceToHost, s));
+    dl_status rc;
+    if (a.out_bits) {
+        CK(bits_count(S, n, wp, ws.scal + SC_ONES, s));
+        ++launches;
+        if ((rc = write_bits(s, S, wp, a.out_bits, n, a.mem))) return rc;
+    }
+    tm->mark(3);
+    if ((rc = read_scalars(ws, s))) return rc;
+    if (st) {
+        st->path_used = DL_PATH_FP64;
+        st->eps_used = eps;
+        st->iters = ly.levels();
+        st->final_resid = 0.0;
+        st->guard_flagged = a.out_bits ? static_cast<int64_t>(host_scal(ws)[SC_GUARD]) : 0;
+        st->model_ones = a.out_bits ? static_cast<int64_t>(host_scal(ws)[SC_ONES]) : -1;
+        st->ms_factor = tm->ms(0, 1);
+        st->ms_solve = tm->ms(1, 2);
+        st->ms_total = tm->ms(0, 3);
+        st->gpu_launches = launches;
+    }
+    return DL_OK;
+}
+
 // The real least solution S~ = eps (B + P S~ P^T) of same generation (Sec. 7.2; its positive
 // entries are the model, Theorem 2), in FP64, written to a.out_rtilde (n x n doubles).
+//  * P acyclic in few layers of short parent lists: row by row in the order of the layers, every
+//    entry once (sg_real_layers); it is what the series below would end with;
 //  * the series X_{t+1} = eps (B + P X_t P^T) from X_0 = 0 (FP64 gathers over the CSR of P;
 //    X_{t+1} - X_t is X_t's residual, so a step whose change is at most tol eps ends it).  It
 //    is exact after depth + 1 steps when P is nilpotent (a forest or a DAG);
@@ -1276,10 +1385,7 @@ dl_status solve_sg_real(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveA
     auto *cnt = static_cast<int *>(ws.get("g_cnt", (np + 1) * 4));
     auto *ptr = static_cast<int *>(ws.get("g_ptr", (np + 1) * 4));
     auto *colmask = static_cast<uint64_t *>(ws.get("g_colmask", wp * 8));
-    auto *Xd = static_cast<double *>(ws.get("sr_X", nn * 8));
-    auto *Xn = static_cast<double *>(ws.get("sr_Xn", nn * 8));
-    auto *U = static_cast<double *>(ws.get("sr_U", nn * 8));
-    NEED(bits && bitsB && cnt && ptr && colmask && Xd && Xn && U);
+    NEED(bits && bitsB && cnt && ptr && colmask);
     CK(cudaMemsetAsync(ws.scal, 0, kScalars * sizeof(unsigned long long), s));
     CK(cudaMemsetAsync(ws.status, 0, sizeof(int), s));
     CK(cudaMemsetAsync(colmask, 0, wp * 8, s));
@@ -1290,18 +1396,37 @@ dl_status solve_sg_real(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveA
     if (Bm) {
         CK(pack_bits(Bm, n, static_cast<int>(np), wp, bitsB, ws.status, s));
         ++launches;
+    } else {
+        CK(bits_identity(bitsB, n, static_cast<int>(np), wp, s));
+        ++launches;
+    }
+    Layers ly;
+    if (a.path != DL_PATH_MIXED && dag_levels_fit(n)) {
+        if ((rc = layers_enqueue(ws, s, bits, n, wp, ptr, &ly))) return rc;
+        launches += 2;
     }
     if ((rc = read_scalars(ws, s))) return rc;
     if ((rc = check_status(ws, s))) return rc;
+    layers_read(ws, &ly);
     const double dmax = static_cast<double>(host_scal(ws)[SC_DMAX]);
     double eps = 0;
     if ((rc = choose_eps(a.eps, 1.0 / (1.0 + dmax * dmax), "Sec. 7.2 (1/(1+||P||^2))", &eps))) return rc;
+    // P acyclic in few layers: every row once, in order (no entry is below eps^levels, so none
+    // underflows and X > 0 is the model)
+    if (ly.levels() > 0 && sg_real_fused(static_cast<int>(np), host_scal(ws)[SC_DMAX]) &&
+        -std::log2(eps) * (ly.levels() + 1) < 1000.0)
+        return sg_real_layers(ctx, ws, s, a, st, ly, ptr, bitsB, wp, eps, &tm, launches);
     const int64_t nnz = static_cast<int64_t>(host_scal(ws)[SC_NNZ]);
-    auto *col = static_cast<int *>(ws.get("g_col", static_cast<size_t>(std::max<int64_t>(nnz, 1)) * 4));
-    NEED(col);
-    CK(csr_fill_from_bits(bits, n, wp, ptr, col, s));
+    auto *Xd = static_cast<double *>(ws.get("sr_X", nn * 8));
+    auto *Xn = static_cast<double *>(ws.get("sr_Xn", nn * 8));
+    auto *U = static_cast<double *>(ws.get("sr_U", nn * 8));
+    auto *col = ly.filled ? ly.col : static_cast<int *>(ws.get("g_col", static_cast<size_t>(std::max<int64_t>(nnz, 1)) * 4));
+    NEED(Xd && Xn && U && col);
+    if (!ly.filled) {
+        CK(csr_fill_from_bits(bits, n, wp, ptr, col, s));
+        ++launches;
+    }
     CK(cudaMemsetAsync(Xd, 0, nn * 8, s));
-    ++launches;
     tm.mark(1);
 
     const double tol = ctx->cfg.refine_tol > 0 ? ctx->cfg.refine_tol : 1e-13;
@@ -1486,7 +1611,7 @@ dl_status solve_sg_real(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveA
         SolveArgs b = a;
         b.path = DL_PATH_AUTO;
         b.eps = 0.0;
-        if ((rc = sg_iteration(ctx, ws, s, b, &bs, &exact, M))) return rc;
+        if ((rc = sg_iteration(ctx, ws, s, b, &bs, &exact, true, M))) return rc;
         if (!exact && (rc = sg_doubling(ctx, ws, s, b, &bs))) return rc;
         launches += bs.gpu_launches;
         model_ones = bs.model_ones;
@@ -2033,6 +2158,7 @@ dl_status solve_transposed(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const Sol
     b.path = a.path == DL_PATH_BOOL_FP8 ? DL_PATH_BOOL_FP8 : DL_PATH_AUTO;
     b.out_bits = Mw;
     b.out_rtilde = nullptr;
+    b.no_layers = true;  // R1 is a general relation here, most often with cycles: not looked for
     dl_stats sgst{};
     if ((rc = solve_sg(ctx, ws, s, b, &sgst))) return rc;
     launches += sgst.gpu_launches;

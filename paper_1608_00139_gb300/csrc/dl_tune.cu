@@ -507,6 +507,7 @@ dl_status autotune_bucket(dl_ctx *ctx, Workspace &ws, cudaStream_t s, int32_t n_
                 a.mem = DL_MEM_DEVICE;
                 a.path = DL_PATH_AUTO;
                 a.out_bits = ob;
+                a.no_layers = true;  // the two routes of a relation without short layers
                 double t = 0;
                 for (int rep = 0; rep < 2; ++rep) {
                     dl_stats st{};
