@@ -748,7 +748,8 @@ dl_status tc_fp64(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &a
     auto *mbits = static_cast<uint64_t *>(ws.get("bits1", npb * wp * 8));
     const int64_t ldg = 2 * np;
     auto *G = static_cast<double *>(ws.get("fp64_G", np * ldg * 8));
-    NEED(C0 && mbits && G);
+    auto *scratch = static_cast<double *>(ws.get("fp64_S", 32 * 32 * 8));
+    NEED(C0 && mbits && G && scratch);
     CK(cudaMemsetAsync(ws.scal, 0, kScalars * sizeof(unsigned long long), s));
     CK(cudaMemsetAsync(ws.status, 0, sizeof(int), s));
     // validation and row sums (the e4m3 copy is not used by this path)
@@ -765,7 +766,7 @@ dl_status tc_fp64(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &a
         CK(fp64_build(E, a.rhs ? a.rhs : E, n, static_cast<int>(np), eps, G, ldg, s));
     ++launches;
     tm.mark(1);
-    CK(fp64_solve(G, ldg, static_cast<int>(np), &launches, s));
+    CK(fp64_solve(G, ldg, static_cast<int>(np), scratch, &launches, s));
     tm.mark(2);
     const double *X = G + np;
     const double tau = ctx->cfg.guard_tau > 0 ? ctx->cfg.guard_tau : 1e-30;
