@@ -284,10 +284,13 @@ DL_API dl_status dl_sg_real(dl_ctx *ctx, int32_t n, const uint8_t *P, const uint
  * R1: n x n 0/1.  out_bits (required): the least model of r2.  The model is computed through
  * the paper's reduction to a two-sided equation (eq. matrixeq:trans:2):
  * R2 = min1(B + R1 R2 R1^T) with B = min1(R1 + R1 R1^T) (one FP8 tensor-core product), solved as
- * dl_sg_least_model does (boolean doubling or the Iteration on bits).
+ * dl_sg_least_model does (boolean doubling or the Iteration on bits); with R~2 and n <= 16384 it
+ * is R~2 > 0 completed by the steps M <- R1 | R1 M^T on bits.
  * out_rtilde (optional, n x n doubles): the real least solution R~2, by the increasing series
  * X_{t+1} = eps (R1 + R1 X_t^T) from 0 in FP64 until a step changes no entry by more than
- * refine_tol * eps (DL_ENOTCONV after 100000 steps); stats->guard_flagged counts the 64-bit bit
+ * refine_tol * eps (DL_ENOTCONV after 100000 steps); DL_PATH_AUTO at n <= 16384 sums the series in
+ * FP32 for the corrections of an FP64 iterate until its FP64 residual is at most refine_tol * eps
+ * (relations on which that is slow take the FP64 series); stats->guard_flagged counts the 64-bit bit
  * words where R~2 > 0 differs from the model (nonzero only under FP64 underflow).
  * Paths: DL_PATH_AUTO (model; R~2 if out_rtilde is not NULL), DL_PATH_FP64 (model and the series,
  * out_rtilde optional), DL_PATH_BOOL_FP8 (model only: a non-NULL out_rtilde returns DL_EINVAL);

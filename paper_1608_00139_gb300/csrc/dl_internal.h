@@ -288,12 +288,38 @@ cudaError_t row_abs_sum_max(const float *A, int np, unsigned *out, cudaStream_t 
 cudaError_t negate_f32(const float *a, float *b, int64_t count, cudaStream_t s);
 cudaError_t add_f32_to_f64(double *x, const float *d, int64_t count, cudaStream_t s);
 cudaError_t transpose_f32(const float *src, int64_t lds, int rows, int cols, float *dst, int64_t ldd, cudaStream_t s);
-// One step of the transposed class's series (Sec. 6.2, eq. matrixeq:trans:1) over the CSR of R1:
-// U = X^T, then Xn = eps (R1 + R1 U), i.e. Xn[i][j] = eps (R1[i][j] + sum_{y in succ(i)} X[j][y])
-// (R1: n x n bytes; X, U, Xn: np x np, zero outside n x n); *dmax (zeroed by the caller) as
-// for the same-generation series (a power-of-two bound on the step's largest change).
+// The transposed class (Sec. 6.2, eq. matrixeq:trans:1).  trans_relabel: rank[i] = the place of
+// constant i by falling number of successors, perm its inverse, and the CSR under those labels
+// (cnt, ptr2: n + 1 ints; col2 as long as col).  The calls below take that CSR; every matrix is np x np
+// (zero outside n x n) in those labels; 8 n bytes of shared memory per row, n <= 29056.
+cudaError_t trans_relabel(const int *ptr, const int *col, int n, int *rank, int *perm, int *cnt, int *ptr2, int *col2,
+                          cudaStream_t s);
+// Two steps of the series X <- eps (R1 + R1 X^T) in place, U scratch; *dmax (zeroed by the caller) as
+// for the same-generation series, over both steps.
+cudaError_t trans_real_steps(const int *ptr, const int *col, int n, int np, double eps, double *X, double *U,
+                             unsigned long long *dmax, cudaStream_t s);
+// Two steps of the correction series D <- R + eps R1 D^T in FP32 from D_in (NULL: 0) into D; R and
+// RT = R^T, both NULL for the right-hand side eps R1; E scratch; slots[0], slots[1] (zeroed by the
+// caller) = bits of max |change| and max |D|.  Nothing runs when the pair whose slots `skip` names had
+// converged to FP32 rounding (or was itself left out).
+cudaError_t trans_correction_steps(const int *ptr, const int *col, int n, int np, double eps, const float *R,
+                                   const float *RT, const float *D_in, float *D, float *E, unsigned long long *slots,
+                                   const unsigned long long *skip, cudaStream_t s);
+// U = eps (R1 + R1 X^T)^T in FP64 and R = U^T - X, stored in FP32 with its transpose RT; *rmax (zeroed
+// by the caller) = bits of max |R| as a double.
+cudaError_t trans_residual(const int *ptr, const int *col, int n, int np, double eps, const double *X, double *U,
+                           float *R, float *RT, unsigned long long *rmax, cudaStream_t s);
+// X = eps (R1 + R1 U): the second FP64 step after trans_residual's, over X (*dmax as for two steps).
+cudaError_t trans_last_step(const int *ptr, const int *col, int n, int np, double eps, const double *U, double *X,
+                            unsigned long long *dmax, cudaStream_t s);
+// X back under its own labels: out (n x n, row stride n; optional) and the bits X > 0 (rows < n).
+cudaError_t trans_finish(const int *rank, int n, int np, int64_t wp, const double *X, double *out, uint64_t *bits,
+                         cudaStream_t s);
+// One step of the series under the given labels, for any n: U = X^T, then Xn = eps (R1 + R1 U) (R1:
+// bytes; *dmax over that step).
 cudaError_t trans_real_step(const int *ptr, const int *col, int n, int np, double eps, const uint8_t *R1,
                             const double *X, double *U, double *Xn, unsigned long long *dmax, cudaStream_t s);
+cudaError_t f32_to_f64(double *x, const float *d, int64_t count, cudaStream_t s);
 // dst |= src over `words` 64-bit words.
 cudaError_t bits_or(uint64_t *dst, const uint64_t *src, int64_t words, cudaStream_t s);
 

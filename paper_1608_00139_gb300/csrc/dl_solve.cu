@@ -2074,6 +2074,179 @@ __global__ void e4m3_to_u8_kernel(const uint8_t *__restrict__ C, int64_t ldc, in
 
 }  // namespace
 
+// The transposed class with its real solution, n <= 16384: X first, then the model from it.
+// X = R~2 by the series of eq. matrixeq:trans:1 (see solve_transposed) under labels sorted by the
+// length of the successor lists; X > 0 lies inside the model (every entry is a sum of products of
+// facts, an exact zero stays zero), and the steps M <- M | R1 | R1 M^T on bits from there reach it:
+// the first one confirms it unless entries underflowed or the series stopped above them.  So the
+// dense products of the model alone (0.71 ms at n = 4096) are not needed.  ER n = 4096, 4 facts per
+// row, one call: 11.1 ms -> 2.5 ms (22 steps at 0.44 ms and the model before; now 22 FP32 steps at
+// 0.06 ms, two FP64 residuals at 0.26 ms, a last FP64 step and the bits at 0.03 ms).
+dl_status trans_real_first(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &a, dl_stats *st,
+                           const uint8_t *R1, Timer *tm, bool *done_out) {
+    *done_out = false;
+    const int32_t n = a.n;
+    const int64_t np = round_up(std::max<int64_t>(n, 1), 256), wp = np / 64;
+    const size_t nq = static_cast<size_t>(np) * np;
+    int launches = 0;
+    auto *T = static_cast<uint64_t *>(ws.get("bits0", np * wp * 8));
+    auto *M = static_cast<uint64_t *>(ws.get("bits1", np * wp * 8));
+    auto *Mt = static_cast<uint64_t *>(ws.get("bits2", np * wp * 8));
+    auto ints = [&](const char *name, size_t count) {
+        return static_cast<int *>(ws.get(name, std::max<size_t>(count, 4) * sizeof(int)));
+    };
+    int *cnt = ints("g_cnt", np + 1), *ptr = ints("g_ptr", np + 1), *uoff = ints("g_units", np + 1);
+    int *rank = ints("tr_rank", np), *perm = ints("tr_perm", np), *cnt2 = ints("tr_cnt", np + 1);
+    int *ptr2 = ints("tr_ptr", np + 1);
+    auto *colmask = static_cast<uint64_t *>(ws.get("g_colmask", wp * 8));
+    auto *X = static_cast<double *>(ws.get("tr_X", nq * 8));
+    auto *U = static_cast<double *>(ws.get("tr_U", nq * 8));
+    NEED(T && M && Mt && cnt && ptr && uoff && rank && perm && cnt2 && ptr2 && colmask && X && U);
+    CK(cudaMemsetAsync(ws.scal, 0, kScalars * sizeof(unsigned long long), s));
+    CK(cudaMemsetAsync(ws.status, 0, sizeof(int), s));
+    CK(cudaMemsetAsync(colmask, 0, wp * 8, s));
+    CK(csr_pack_checked(R1, n, static_cast<int>(np), wp, cnt, ptr, Mt, ws.scal + SC_DMAX, ws.scal + SC_NNZ,
+                        ws.scal + SC_COUNT0, ws.status, colmask, s));
+    CK(pack_bits(R1, n, static_cast<int>(np), wp, M, ws.status, s));
+    launches += 3;
+    dl_status rc;
+    if ((rc = read_scalars(ws, s))) return rc;
+    if ((rc = check_status(ws, s))) return rc;
+    const unsigned long long dmax = host_scal(ws)[SC_DMAX];
+    double eps = 0;
+    if ((rc = choose_eps(a.eps, 1.0 / (1.0 + static_cast<double>(dmax)), "Sec. 6.2 (1/(1+||R1||_inf))", &eps)))
+        return rc;
+    const size_t nnz = static_cast<size_t>(host_scal(ws)[SC_NNZ]);
+    int *col = ints("g_col", nnz), *col2 = ints("tr_col", nnz);
+    NEED(col && col2);
+    CK(csr_fill_from_bits(Mt, n, wp, ptr, col, s));
+    CK(trans_relabel(ptr, col, n, rank, perm, cnt2, ptr2, col2, s));
+    launches += 5;
+    const int *units = nullptr;  // rows of more than 64 successors: edge-parallel gathers of the bits
+    if (dmax > 64) {
+        CK(sweep_units(ptr, n, cnt, uoff, s));
+        launches += 2;
+        units = uoff;
+    }
+    tm->mark(1);
+
+    const double tol = ctx->cfg.refine_tol > 0 ? ctx->cfg.refine_tol : 1e-13;
+    unsigned long long *slot = ws.scal + 32;
+    const int N = static_cast<int>(np);
+    bool done = false;
+    int steps = 0;
+    double resid = 0.0;
+    if (a.path == DL_PATH_AUTO) {
+        // refinement: X <- X + D, D = sum_m L^m R by the series in FP32 (L the equation's operator, R the
+        // FP64 residual, eps R1 at first), until max|R| <= tol eps; each step gains six digits when the
+        // series converges within kPairs pairs of steps.  When it does not (or scratch is short), the
+        // FP64 series below starts afresh.
+        auto f32 = [&](const char *name) { return static_cast<float *>(ws.get(name, nq * 4)); };
+        float *R = f32("tr_R"), *RT = f32("tr_RT"), *D = f32("tr_D"), *E = f32("tr_E");
+        constexpr int kPairs = 8, kMaxRefine = 4;
+        double before = 1.0;  // max|R| / eps of X = 0
+        bool more = R && RT && D && E;
+        for (int it = 0; more && !done && it < kMaxRefine; ++it) {
+            const float *r = it == 0 ? nullptr : R, *rt = it == 0 ? nullptr : RT;
+            CK(cudaMemsetAsync(slot, 0, (2 * kPairs + 1) * sizeof(unsigned long long), s));
+            for (int k = 0; k < kPairs; ++k)
+                CK(trans_correction_steps(ptr2, col2, n, N, eps, r, rt, k == 0 ? r : D, D, E, slot + 2 * k,
+                                          k == 0 ? nullptr : slot + 2 * (k - 1), s));
+            CK(it == 0 ? f32_to_f64(X, D, static_cast<int64_t>(nq), s)
+                       : add_f32_to_f64(X, D, static_cast<int64_t>(nq), s));
+            CK(trans_residual(ptr2, col2, n, N, eps, X, U, R, RT, slot + 2 * kPairs, s));
+            launches += 2 * kPairs + 3;
+            if ((rc = read_scalars(ws, s))) return rc;
+            for (int k = 0; k < kPairs; ++k) steps += host_scal(ws)[32 + 2 * k + 1] != 0 ? 2 : 0;
+            const unsigned long long rb = host_scal(ws)[32 + 2 * kPairs];
+            std::memcpy(&resid, &rb, sizeof resid);
+            resid /= eps;
+            done = resid <= tol;
+            more = resid <= 1e-3 * before;
+            before = resid;
+        }
+        if (done) {  // two FP64 steps end it: U^T, which the residual's pass has formed, and the gather of it
+            CK(trans_last_step(ptr2, col2, n, N, eps, U, X, slot, s));
+            ++launches;
+            steps += 2;
+        }
+    }
+    if (!done) {  // the FP64 series from 0, two steps per pair, four per host read
+        steps = 0;
+        constexpr int kGroup = 2, kBudget = 100000;
+        CK(cudaMemsetAsync(X, 0, nq * 8, s));
+        while (!done && steps < kBudget) {
+            CK(cudaMemsetAsync(slot, 0, kGroup * sizeof(unsigned long long), s));
+            for (int k = 0; k < kGroup; ++k) CK(trans_real_steps(ptr2, col2, n, N, eps, X, U, slot + k, s));
+            launches += 2 * kGroup;
+            if ((rc = read_scalars(ws, s))) return rc;
+            for (int k = 0; k < kGroup; ++k) {
+                steps += 2;
+                const unsigned long long code = host_scal(ws)[32 + k];  // max change < 2^(code - 4096)
+                resid = code == 0 ? 0.0 : std::ldexp(1.0, static_cast<int>(code) - 4096) / eps;
+                if (resid <= tol) {
+                    done = true;  // the iterates after this step are at least as close
+                    break;
+                }
+            }
+        }
+        if (!done) {
+            set_error("transposed class: the series did not reach max|change|/eps <= %g in %d steps", tol, steps);
+            return DL_ENOTCONV;
+        }
+    }
+    const bool device = a.mem == DL_MEM_DEVICE;
+    double *out = !a.out_rtilde ? nullptr : device ? a.out_rtilde : U;  // (U is free now)
+    CK(cudaMemsetAsync(T, 0, np * wp * 8, s));
+    CK(trans_finish(rank, n, N, wp, X, out, T, s));
+    ++launches;
+    if (out && !device)
+        CK(cudaMemcpyAsync(a.out_rtilde, out, static_cast<size_t>(n) * n * 8, cudaMemcpyDeviceToHost, s));
+    tm->mark(2);
+
+    // the model: M holds R1; M |= T, then M |= R1 M^T until nothing changes
+    CK(bits_or(M, T, np * wp, s));
+    constexpr int kIters = 2, kBudget = 64;
+    int iters = 0;
+    bool fixed = false;
+    while (!fixed) {
+        if (iters >= kBudget) return DL_OK;  // far from the model: the two-sided reduction instead
+        CK(cudaMemsetAsync(slot, 0, kIters * sizeof(unsigned long long), s));
+        CK(cudaMemsetAsync(ws.scal + SC_ONES, 0, 2 * sizeof(unsigned long long), s));
+        CK(cudaMemsetAsync(ws.scal + SC_GUARD, 0, sizeof(unsigned long long), s));
+        for (int k = 0; k < kIters; ++k) {
+            const unsigned long long *skip = k > 0 ? slot + k - 1 : nullptr;
+            CK(bits_transpose(M, Mt, N, wp, skip, s));
+            CK(bits_gather(ptr, col, units, n, Mt, M, wp, 1, slot + k, skip, s));
+        }
+        CK(bits_count(M, n, wp, ws.scal + SC_ONES, s));
+        CK(bits_diff(T, M, np * wp, ws.scal + SC_GUARD, s));
+        launches += 2 * kIters + 2;
+        if ((rc = read_scalars(ws, s))) return rc;
+        for (int k = 0; k < kIters; ++k) fixed |= host_scal(ws)[32 + k] == 0;
+        iters += kIters;
+    }
+    if ((rc = write_bits(s, M, wp, a.out_bits, n, a.mem))) return rc;
+    tm->mark(3);
+    if ((rc = check_status(ws, s))) return rc;
+    if (st) {
+        st->path_used = DL_PATH_FP64;
+        st->eps_used = eps;
+        st->iters = steps;
+        st->final_resid = resid;
+        st->guard_flagged = static_cast<int64_t>(host_scal(ws)[SC_GUARD]);
+        st->model_ones = static_cast<int64_t>(host_scal(ws)[SC_ONES]);
+        st->recheck_sweeps = iters;
+        st->ms_factor = tm->ms(0, 1);
+        st->ms_refine = tm->ms(1, 2);
+        st->ms_solve = tm->ms(2, 3);
+        st->ms_total = tm->ms(0, 3);
+        st->gpu_launches = launches;
+    }
+    *done_out = true;
+    return DL_OK;
+}
+
 // The transposed class (Sec. 6.2), program prog:2:
 //     r2(x,z) <- r1(x,z).      r2(x,z) <- r1(x,y), r2(z,y).
 // Its completion R2 = min1(R1 + R1 R2^T) substituted into itself gives the two-sided equation
@@ -2081,11 +2254,13 @@ __global__ void e4m3_to_u8_kernel(const uint8_t *__restrict__ C, int64_t ldc, in
 // least solution: the iterates of the two-step operator from 0 are every other iterate of the
 // one-step operator, which increase to its least fixpoint.  So the model is one FP8 product
 // (C = R1 R1^T with R1 added in the epilogue) and the same-generation solver with P = R1 and B.
-// The real R~2 = eps (R1 + R1 R~2^T) (eq. matrixeq:trans:1; DL_PATH_FP64, or DL_PATH_AUTO when
-// asked for): the increasing series X_{t+1} = eps (R1 + R1 X_t^T) from X_0 = 0 in FP64, four steps
-// per host read, until a step changes no entry by more than tol eps; its positive entries are
-// compared with the model (guard_flagged counts the bit words where they differ: only underflow
-// can make them).
+// The real R~2 = eps (R1 + R1 R~2^T) (eq. matrixeq:trans:1).  DL_PATH_FP64: the increasing series
+// X_{t+1} = eps (R1 + R1 X_t^T) from X_0 = 0 in FP64, four steps per host read, until a step changes
+// no entry by more than tol eps.  DL_PATH_AUTO when asked for R~2: the same series in FP32 for the
+// corrections of an FP64 iterate whose FP64 residual decides (an FP64 step is bound by the two FP64
+// lanes of an SM, an FP32 one by its bytes); relations whose series is slow fall back to FP64.  The
+// positive entries are compared with the model (guard_flagged counts the bit words where they
+// differ: only underflow can make them).
 dl_status solve_transposed(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &a, dl_stats *st) {
     if (a.thr != 0.0) {
         set_error("thr must be 0: the model is R~ > 0 (Theorem 2)");
@@ -2112,6 +2287,12 @@ dl_status solve_transposed(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const Sol
     const uint8_t *R1 = nullptr;
     dl_status rc = stage_input(ws, s, a.E, n, a.mem, "tr_in0", &R1);
     if (rc) return rc;
+    const bool real = a.out_rtilde != nullptr || a.path == DL_PATH_FP64;
+    if (real && wp <= 256) {
+        bool done = false;
+        if ((rc = trans_real_first(ctx, ws, s, a, st, R1, &tm, &done)) || done) return rc;
+        tm.mark(0);
+    }
     auto *R8 = static_cast<uint8_t *>(ws.get("tr_e8", np * np));
     auto *B8 = static_cast<uint8_t *>(ws.get("tr_b8", np * np));
     auto *Bu = static_cast<uint8_t *>(ws.get("tr_bu8", std::max<size_t>(static_cast<size_t>(n) * n, 16)));
@@ -2169,7 +2350,6 @@ dl_status solve_transposed(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const Sol
     int steps = 0;
     double resid = 0.0;
     unsigned long long differ = 0;
-    const bool real = a.out_rtilde != nullptr || a.path == DL_PATH_FP64;
     if (real) {
         const size_t nq = static_cast<size_t>(np) * np;
         auto *cnt = static_cast<int *>(ws.get("tr_cnt", (np + 1) * 4));
