@@ -203,6 +203,21 @@ cudaError_t bits_diff(const uint64_t *A, const uint64_t *B, int64_t words, unsig
 cudaError_t bits_to_e4m3(const uint64_t *bits, int64_t wp, int np, uint8_t *C, cudaStream_t s);
 
 // ---------------------------------------------------------------------------------------
+// The whole closure of a small relation in one launch (dl_small.cu)
+// ---------------------------------------------------------------------------------------
+struct SmallClosure {
+    unsigned long long nnz, ones, violations;  // facts, ones of the model, rows' words that fail the certificate
+    int dmax, status, steps, squarings;        // ||E||_inf, ST_* of bad input, steps (squarings among them)
+    int open;                                  // 1: given up
+};
+bool closure_small_fits(int n);
+// out (n rows of ceil(n/64) words) = the least model, from the bytes E or the packed rows Eb (the other
+// NULL); *result (pinned host memory) is valid once the stream has been synchronised.  Nothing is
+// written to out when the input is bad, nor when a relation of long paths is given up (result->open).
+cudaError_t closure_small(const uint8_t *E, const uint64_t *Eb, int n, uint64_t *out, SmallClosure *result,
+                          cudaStream_t s);
+
+// ---------------------------------------------------------------------------------------
 // Graph utilities (dl_graph.cu)
 // ---------------------------------------------------------------------------------------
 // CSR of a dense n x n 0/1 matrix: csr_build writes per-row counts and ptr (n + 1 entries,

@@ -166,10 +166,7 @@ dl_status read_scalars(Workspace &ws, cudaStream_t s) {
     return DL_OK;
 }
 
-dl_status check_status(Workspace &ws, cudaStream_t s) {
-    int st = 0;
-    CK(cudaMemcpyAsync(&st, ws.status, sizeof(int), cudaMemcpyDeviceToHost, s));
-    CK(cudaStreamSynchronize(s));
+dl_status status_error(int st) {
     if (st & ST_BAD_INPUT) {
         set_error("input matrix holds a byte that is neither 0 nor 1");
         return DL_EINVAL;
@@ -183,6 +180,13 @@ dl_status check_status(Workspace &ws, cudaStream_t s) {
         return DL_ETIMEOUT;
     }
     return DL_OK;
+}
+
+dl_status check_status(Workspace &ws, cudaStream_t s) {
+    int st = 0;
+    CK(cudaMemcpyAsync(&st, ws.status, sizeof(int), cudaMemcpyDeviceToHost, s));
+    CK(cudaStreamSynchronize(s));
+    return status_error(st);
 }
 
 // Upload `count` GEMM problems into the workspace table (device) and return it.
@@ -405,6 +409,51 @@ dl_status tc_bool(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &a
     return DL_OK;
 }
 
+// DL_PATH_AUTO for a small relation: one launch (closure_small) and one wait.  *done = false when
+// it has to go the general route (long paths).
+dl_status tc_small(Workspace &ws, cudaStream_t s, const SolveArgs &a, dl_stats *st, bool *done) {
+    *done = false;
+    const int32_t n = a.n;
+    const size_t out_bytes = static_cast<size_t>(n) * ((n + 63) / 64) * 8;
+    Timer tm{ws.ev, s, "tc_small"};
+    tm.mark(0);
+    const uint8_t *E = nullptr;
+    const uint64_t *Eb = nullptr;
+    dl_status rc = a.E_bits ? stage_bits(ws, s, a.E_bits, n, a.mem, &Eb) : stage_input(ws, s, a.E, n, in_mem(a), "in0", &E);
+    if (rc) return rc;
+    uint64_t *model = a.mem == DL_MEM_DEVICE ? a.out_bits : static_cast<uint64_t *>(ws.get("bits1", out_bytes));
+    NEED(model);
+    auto *r = reinterpret_cast<SmallClosure *>(static_cast<char *>(ws.host_pinned) + kInfoOffset);
+    tm.mark(1);
+    CK(closure_small(E, Eb, n, model, r, s));
+    tm.mark(2);
+    if (a.mem != DL_MEM_DEVICE) CK(cudaMemcpyAsync(a.out_bits, model, out_bytes, cudaMemcpyDeviceToHost, s));
+    tm.mark(3);
+    CK(cudaStreamSynchronize(s));
+    if ((rc = status_error(r->status))) return rc;
+    double eps = 0;
+    if ((rc = choose_eps(a.eps, 1.0 / (1.0 + static_cast<double>(r->dmax)), "Lemma 1 (1/(1+||E||))", &eps))) return rc;
+    if (r->open) return DL_OK;
+    if (r->violations != 0) {
+        set_error("internal: converged closure failed its certificate");
+        return DL_EDEVICE;
+    }
+    if (st) {
+        st->path_used = DL_PATH_AUTO;
+        st->eps_used = eps;
+        st->iters = r->squarings;
+        st->recheck_sweeps = r->steps - r->squarings + 1;
+        st->model_ones = static_cast<int64_t>(r->ones);
+        st->ms_factor = tm.ms(0, 1);
+        st->ms_solve = tm.ms(1, 2);
+        st->ms_epilogue = tm.ms(2, 3);
+        st->ms_total = tm.ms(0, 3);
+        st->gpu_launches = 1;
+    }
+    *done = true;
+    return DL_OK;
+}
+
 // DL_PATH_AUTO: tensor-core squarings and boolean sweeps, whichever is cheaper.
 // A sweep (in place, M <- M | E | E M on bits) is one step of the paper's Iteration method
 // (Sec. 7.1, eq. series:trcl) and adds at least one hop to every path; a squaring doubles
@@ -416,6 +465,11 @@ dl_status tc_auto(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &a
     const int32_t n = a.n;
     const int64_t np = round_up(std::max<int64_t>(n, 1), 256);
     const int64_t wp = np / 64;
+    if (closure_small_fits(n)) {
+        bool done = false;
+        const dl_status rs = tc_small(ws, s, a, st, &done);
+        if (rs != DL_OK || done) return rs;
+    }
     Timer tm{ws.ev, s, "tc_auto"};
     int launches = 0;
     tm.mark(0);

@@ -1,0 +1,79 @@
+"""The one-launch closure (AUTO up to n = 1024; 1025 and up take the general route) against the oracle: sizes at the edges of words, of the
+16-column pieces of the ingest and of the CTAs' rows; sparse, dense, saturated and empty relations, rows
+longer than a list, paths that need the squarings; bytes at any alignment and packed rows."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_1608_00139_gb300 import dl, inputs
+
+pytestmark = pytest.mark.gpu
+
+SIZES = [1, 2, 15, 16, 17, 63, 64, 65, 127, 128, 129, 257, 511, 512, 513, 1000, 1023, 1024, 1025]
+
+
+def relation(kind, n):
+    rng = np.random.default_rng(n)
+    if kind == "sparse":
+        return inputs.er_digraph(n, min(1.0, 2.5 / n), n + 3, self_loops=True)
+    if kind == "dense":
+        return inputs.er_digraph(n, 0.2, n + 4)
+    if kind == "idle":  # a fifth of the constants without facts, rows of some 40 successors
+        e = inputs.er_digraph(n, min(1.0, 40.0 / n), n + 5)
+        off = rng.random(n) < 0.2
+        e[off] = 0
+        e[:, off] = 0
+        return e
+    e = np.zeros((n, n), np.uint8)
+    if kind == "chain":  # the longest path there is, labels in random order
+        order = rng.permutation(n)
+        e[order[:-1], order[1:]] = 1
+    elif kind == "ones":
+        e[:] = 1
+    return e
+
+
+@pytest.mark.parametrize("kind", ["sparse", "dense", "idle", "chain", "ones", "empty"])
+@pytest.mark.parametrize("n", SIZES)
+def test_model(ctx, n, kind):
+    e = relation(kind, n)
+    want = oracle.tc_model(e)
+    bits, st = ctx.tc_closure(e)
+    assert np.array_equal(bits, want)
+    assert st["model_ones"] == int(np.unpackbits(want.view(np.uint8)).sum())
+    assert st["eps_used"] == oracle.tc_eps(e)
+    packed, _ = ctx.tc_closure_bits(oracle.pack(e), n)
+    assert np.array_equal(packed, want)
+
+
+@pytest.mark.parametrize("shift", [1, 7, 8, 15])
+@pytest.mark.parametrize("n", [33, 250, 1000])
+def test_any_alignment_of_device_rows(ctx, n, shift):
+    e = relation("sparse", n)
+    buf = torch.full((n * n + 32,), 255, dtype=torch.uint8, device="cuda")  # bytes around it are not read as facts
+    dev = buf[shift:shift + n * n].view(n, n)
+    dev.copy_(torch.from_numpy(e))
+    bits, _ = ctx.tc_closure(dev)
+    assert np.array_equal(bits.cpu().numpy().view(np.uint64), oracle.tc_model(e))
+
+
+@pytest.mark.parametrize("n", [5, 130, 700, 1024])
+def test_bad_input(ctx, n):
+    for i, j in ((0, 0), (n - 1, n - 1), (n // 2, n - 1)):
+        e = relation("sparse", n)
+        e[i, j] = 2
+        with pytest.raises(dl.DLError) as err:
+            ctx.tc_closure(e)
+        assert err.value.status == dl.DL_EINVAL
+    if n % 64:
+        packed = oracle.pack(relation("sparse", n)).copy()
+        packed[n - 1, -1] |= np.uint64(1) << np.uint64(63)
+        with pytest.raises(dl.DLError) as err:
+            ctx.tc_closure_bits(packed, n)
+        assert err.value.status == dl.DL_EINVAL
+    e = relation("sparse", n)
+    with pytest.raises(dl.DLError) as err:
+        ctx.tc_closure(e, eps=2.0)
+    assert err.value.status == dl.DL_EINVAL
+    assert np.array_equal(ctx.tc_closure(e)[0], oracle.tc_model(e))
