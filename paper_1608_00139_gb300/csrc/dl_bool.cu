@@ -217,8 +217,10 @@ __global__ void __launch_bounds__(256)
     sweep_rows_step_kernel(const int *__restrict__ ptr, const int *__restrict__ col, int n, uint64_t *M, int64_t wp,
                            unsigned long long *changed_rows, const unsigned long long *skip_if_zero,
                            const uint64_t *__restrict__ colmask, const int *gate) {
+    grid_dep_launch();
     const int lane = threadIdx.x & 31;
     const int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    grid_dep_wait();
     if (i >= n) return;
     if (skip_if_zero != nullptr && *skip_if_zero == 0) return;  // the previous sweep changed nothing
     if (gate != nullptr && *gate != 0) return;
@@ -257,8 +259,10 @@ __global__ void __launch_bounds__(256)
     sweep_rows_emit_kernel(const int *__restrict__ ptr, const int *__restrict__ col, int n, const uint64_t *M,
                            uint64_t *out, int64_t wp, unsigned long long *violations, unsigned long long *ones,
                            const uint64_t *__restrict__ colmask, const int *gate) {
+    grid_dep_launch();
     const int lane = threadIdx.x & 31;
     const int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    grid_dep_wait();
     if (i >= n) return;
     if (gate != nullptr && *gate != 0) return;
     uint64_t full[WPL], acc[WPL];
@@ -291,13 +295,14 @@ template <int WPL>
 cudaError_t launch_rows(const int *ptr, const int *col, int n, const uint64_t *M, uint64_t *out, int64_t wp,
                         int mode, unsigned long long *violations, unsigned long long *ones,
                         const unsigned long long *skip, const uint64_t *colmask, const int *gate, cudaStream_t s) {
+    // programmatic launches: a sweep's launch overlaps the end of the one before it (a closure is a chain
+    // of some ten kernels of 3-12 us)
+    const dim3 grid(static_cast<unsigned>((n + 7) / 8)), block(256);
     if (mode == 1)
-        sweep_rows_step_kernel<WPL><<<(n + 7) / 8, 256, 0, s>>>(ptr, col, n, const_cast<uint64_t *>(M), wp,
-                                                                 violations, skip, colmask, gate);
-    else
-        sweep_rows_emit_kernel<WPL><<<(n + 7) / 8, 256, 0, s>>>(ptr, col, n, M, out, wp, violations, ones,
-                                                                 colmask, gate);
-    return cudaGetLastError();
+        return launch_programmatic(sweep_rows_step_kernel<WPL>, grid, block, 0, s, ptr, col, n, const_cast<uint64_t *>(M),
+                                   wp, violations, skip, colmask, gate);
+    return launch_programmatic(sweep_rows_emit_kernel<WPL>, grid, block, 0, s, ptr, col, n, M, out, wp, violations, ones,
+                               colmask, gate);
 }
 
 // mode 1 (closure step, in place): M_i |= E_i | OR_{k in succ(i)} M_k; counts changed units.
@@ -382,6 +387,8 @@ __global__ void bits_to_e4m3_kernel(const uint64_t *__restrict__ bits, int64_t w
 __global__ void __launch_bounds__(256)
     row_iteration_kernel(const int *__restrict__ ptr, const int *__restrict__ col, int n, int wp, uint64_t *M,
                          unsigned long long *open_rows, const int *gate) {
+    grid_dep_launch();
+    grid_dep_wait();
     if (gate != nullptr && (*gate != 0 || ptr[n] > 2 * n)) {
         if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(open_rows, static_cast<unsigned long long>(n));
         return;
@@ -704,8 +711,8 @@ cudaError_t row_iteration(const int *ptr, const int *col, int n, int64_t wp, uin
     if (n <= 0) return cudaSuccess;
     if (!row_iteration_fits(wp)) return cudaErrorInvalidValue;
     const size_t smem = 8 * (static_cast<size_t>(wp) + kRowFront + 1) * sizeof(uint64_t);
-    row_iteration_kernel<<<(n + 7) / 8, 256, smem, s>>>(ptr, col, n, static_cast<int>(wp), M, open_rows, gate);
-    return cudaGetLastError();
+    return launch_programmatic(row_iteration_kernel, dim3(static_cast<unsigned>((n + 7) / 8)), dim3(256), smem, s, ptr,
+                               col, n, static_cast<int>(wp), M, open_rows, gate);
 }
 
 cudaError_t bits_transpose(const uint64_t *src, uint64_t *dst, int np, int64_t wp, const unsigned long long *skip,

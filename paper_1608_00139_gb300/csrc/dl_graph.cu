@@ -6,6 +6,7 @@
 #include <cstdint>
 
 #include "dl_internal.h"
+#include "dl_ptx.cuh"
 #include "dl_rows.cuh"
 
 namespace dl {
@@ -100,7 +101,7 @@ __global__ void __launch_bounds__(256, 4)
             }
             if (w == idw) self = (e & idb) != 0ull;
             c += __popcll(e);
-            if (e != 0ull) atomicOr(reinterpret_cast<unsigned long long *>(colmask_s + w), e);
+            if (e != 0ull) or_shared(colmask_s + w, e);
             row[w] = e | (w == idw ? idb : 0ull);
         }
 #pragma unroll
@@ -165,6 +166,8 @@ __global__ void __launch_bounds__(256) unpack_bits_u8_kernel(const uint64_t *__r
 __global__ void __launch_bounds__(256)
     csr_fill_bits_kernel(const uint64_t *__restrict__ M, int n, int wp, const int *__restrict__ ptr, int *col,
                          int64_t cap, const unsigned long long *dmax, int max_deg, int *gate) {
+    grid_dep_launch();
+    grid_dep_wait();
     if (cap >= 0) {
         const bool stop = ptr[n] > cap || *dmax > static_cast<unsigned long long>(max_deg);
         if (blockIdx.x == 0 && threadIdx.x == 0) *gate = stop ? 1 : 0;
@@ -197,8 +200,10 @@ __global__ void __launch_bounds__(256, 4)
 // scan and a scan of the warp totals place them; long inputs go round in tiles of 16384.
 __global__ void __launch_bounds__(1024) exclusive_scan_kernel(const int *cnt, int n, int *ptr) {
     __shared__ int warp_tot[32];
+    grid_dep_launch();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const bool vec = (reinterpret_cast<uintptr_t>(cnt) & 15) == 0;
+    const bool vec = ((reinterpret_cast<uintptr_t>(cnt) | reinterpret_cast<uintptr_t>(ptr)) & 15) == 0;
+    grid_dep_wait();
     int carry = 0;
     for (int base = 0; base < n; base += 1024 * 16) {
         const int b = base + static_cast<int>(threadIdx.x) * 16;
@@ -239,10 +244,24 @@ __global__ void __launch_bounds__(1024) exclusive_scan_kernel(const int *cnt, in
         }
         __syncthreads();
         int run = carry + (warp > 0 ? warp_tot[warp - 1] : 0) + inc - sum;
+        if (vec && b + 16 <= n) {  // (sixteen separate stores per thread took as long as the rest)
+            int4 *p4 = reinterpret_cast<int4 *>(ptr + b);
 #pragma unroll
-        for (int j = 0; j < 16; ++j) {
-            if (b + j < n) ptr[b + j] = run;
-            run += v[j];
+            for (int q = 0; q < 4; ++q) {
+                int4 x;
+                x.x = run;
+                x.y = x.x + v[4 * q];
+                x.z = x.y + v[4 * q + 1];
+                x.w = x.z + v[4 * q + 2];
+                run = x.w + v[4 * q + 3];
+                p4[q] = x;
+            }
+        } else {
+#pragma unroll
+            for (int j = 0; j < 16; ++j) {
+                if (b + j < n) ptr[b + j] = run;
+                run += v[j];
+            }
         }
         carry += warp_tot[31];
         __syncthreads();  // warp_tot is rewritten by the next tile
@@ -421,8 +440,7 @@ cudaError_t csr_pack_checked(const uint8_t *E, int n, int np, int64_t wp, int *c
     const size_t smem = static_cast<size_t>(wp) * sizeof(uint64_t);
     csr_pack_check_kernel<<<static_cast<unsigned>((np + 7) / 8), 256, smem, s>>>(
         E, n, np, static_cast<int>(wp), cnt, M, dmax, nnz, diag, status, colmask);
-    exclusive_scan_kernel<<<1, 1024, 0, s>>>(cnt, n, ptr);
-    return cudaGetLastError();
+    return launch_programmatic(exclusive_scan_kernel, dim3(1), dim3(1024), 0, s, static_cast<const int *>(cnt), n, ptr);
 }
 
 cudaError_t bits_ingest_checked(const uint64_t *Eb, int n, int np, int64_t wp, int *cnt, int *ptr, uint64_t *M,
@@ -432,8 +450,7 @@ cudaError_t bits_ingest_checked(const uint64_t *Eb, int n, int np, int64_t wp, i
     const size_t smem = static_cast<size_t>(wp) * sizeof(uint64_t);
     bits_ingest_check_kernel<<<static_cast<unsigned>((np + 7) / 8), 256, smem, s>>>(
         Eb, n, np, static_cast<int>(wp), cnt, M, dmax, nnz, diag, status, colmask);
-    exclusive_scan_kernel<<<1, 1024, 0, s>>>(cnt, n, ptr);
-    return cudaGetLastError();
+    return launch_programmatic(exclusive_scan_kernel, dim3(1), dim3(1024), 0, s, static_cast<const int *>(cnt), n, ptr);
 }
 
 cudaError_t unpack_bits_u8(const uint64_t *Eb, int n, uint8_t *E, int *status, cudaStream_t s) {
@@ -449,16 +466,15 @@ cudaError_t pack_bits(const uint8_t *E, int n, int np, int64_t wp, uint64_t *M, 
 }
 
 cudaError_t csr_fill_from_bits(const uint64_t *M, int n, int64_t wp, const int *ptr, int *col, cudaStream_t s) {
-    csr_fill_bits_kernel<<<static_cast<unsigned>((n + 7) / 8), 256, 0, s>>>(M, n, static_cast<int>(wp), ptr, col, -1,
-                                                                           nullptr, 0, nullptr);
-    return cudaGetLastError();
+    return launch_programmatic(csr_fill_bits_kernel, dim3(static_cast<unsigned>((n + 7) / 8)), dim3(256), 0, s, M, n,
+                               static_cast<int>(wp), ptr, col, int64_t{-1}, static_cast<const unsigned long long *>(nullptr), 0,
+                               static_cast<int *>(nullptr));
 }
 
 cudaError_t csr_fill_from_bits_guarded(const uint64_t *M, int n, int64_t wp, const int *ptr, int *col, int64_t cap,
                                        const unsigned long long *dmax, int max_deg, int *gate, cudaStream_t s) {
-    csr_fill_bits_kernel<<<static_cast<unsigned>((n + 7) / 8), 256, 0, s>>>(M, n, static_cast<int>(wp), ptr, col, cap,
-                                                                           dmax, max_deg, gate);
-    return cudaGetLastError();
+    return launch_programmatic(csr_fill_bits_kernel, dim3(static_cast<unsigned>((n + 7) / 8)), dim3(256), 0, s, M, n,
+                               static_cast<int>(wp), ptr, col, cap, dmax, max_deg, gate);
 }
 
 // Two-level scan for long arrays: block sums of 1024 elements, a scan of those sums (the

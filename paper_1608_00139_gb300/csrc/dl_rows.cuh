@@ -203,6 +203,15 @@ __device__ __forceinline__ uint32_t byte_bad(uint32_t x) {
     return byte_lsbs(((t + 0x7F7F7F7Fu) | t) >> 7);
 }
 
+// *word |= e on shared memory, as 32-bit operations on the halves that have bits (a 64-bit one is a loop
+// of compare and swap).
+__device__ __forceinline__ void or_shared(uint64_t *word, uint64_t e) {
+    unsigned *h = reinterpret_cast<unsigned *>(word);
+    const unsigned lo = static_cast<unsigned>(e), hi = static_cast<unsigned>(e >> 32);
+    if (lo != 0u) atomicOr(h, lo);
+    if (hi != 0u) atomicOr(h + 1, hi);
+}
+
 // One warp packs row r of a 0/1 byte matrix (the n bytes at a, any alignment) into wp 64-bit
 // words at `row`, plus the identity bit r.  The row is read as aligned 16-byte chunks: lane
 // L of segment s holds the 64 bytes that start 64 (32 s + L) bytes after the aligned address
@@ -259,7 +268,7 @@ __device__ __forceinline__ void pack_row_bits(const uint8_t *a, int n, int r, in
         const uint64_t first = __shfl_sync(0xffffffffu, vw, 0);
         auto put = [&](int w, uint64_t e) {  // e: the facts of word w
             row[w] = e | (w == idw ? idb : 0ull);
-            if (colmask != nullptr && e != 0ull) atomicOr(reinterpret_cast<unsigned long long *>(colmask + w), e);
+            if (colmask != nullptr && e != 0ull) or_shared(colmask + w, e);
         };
         if (sg > 0 && lane == 31) {
             const int w = 32 * (sg - 1) + 31;
@@ -278,7 +287,7 @@ __device__ __forceinline__ void pack_row_bits(const uint8_t *a, int n, int r, in
         if (w < wp) {
             const uint64_t e = shifted(carry, 0ull);
             row[w] = e | (w == idw ? idb : 0ull);
-            if (colmask != nullptr && e != 0ull) atomicOr(reinterpret_cast<unsigned long long *>(colmask + w), e);
+            if (colmask != nullptr && e != 0ull) or_shared(colmask + w, e);
         }
     }
 #pragma unroll
@@ -356,9 +365,8 @@ __device__ __forceinline__ bool iterate_row(const int *__restrict__ ptr, const i
             const int q1 = ptr[k + 1];
             for (int q = ptr[k]; q < q1; ++q) {
                 const int j = col[q];
-                const unsigned long long b = 1ull << (j & 63);
-                const unsigned long long old = atomicOr(reinterpret_cast<unsigned long long *>(bits + (j >> 6)), b);
-                if (!(old & b)) {
+                const unsigned b = 1u << (j & 31);  // (32-bit halves: a 64-bit shared atomic is a loop)
+                if (!(atomicOr(reinterpret_cast<unsigned *>(bits) + (j >> 5), b) & b)) {
                     const int pos = atomicAdd(next_cnt, 1);
                     if (pos < kRowFront) fn[pos] = j;
                 }

@@ -159,10 +159,17 @@ unsigned long long *host_scal(Workspace &ws) {
     return static_cast<unsigned long long *>(ws.host_pinned);
 }
 
+// The scalars and, behind them, the status word.
 dl_status read_scalars(Workspace &ws, cudaStream_t s) {
-    CK(cudaMemcpyAsync(ws.host_pinned, ws.scal, kScalars * sizeof(unsigned long long),
+    CK(cudaMemcpyAsync(ws.host_pinned, ws.scal, (kScalars + 1) * sizeof(unsigned long long),
                        cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
+    return DL_OK;
+}
+
+// Scalars and status word zeroed, in one operation.
+dl_status reset_scalars(Workspace &ws, cudaStream_t s) {
+    CK(cudaMemsetAsync(ws.scal, 0, (kScalars + 1) * sizeof(unsigned long long), s));
     return DL_OK;
 }
 
@@ -182,11 +189,21 @@ dl_status status_error(int st) {
     return DL_OK;
 }
 
+// The status word as the last read_scalars found it.
+dl_status read_status(Workspace &ws) { return status_error(*reinterpret_cast<const int *>(host_scal(ws) + kScalars)); }
+
 dl_status check_status(Workspace &ws, cudaStream_t s) {
     int st = 0;
     CK(cudaMemcpyAsync(&st, ws.status, sizeof(int), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
     return status_error(st);
+}
+
+// The end of a call whose last read_scalars came after the last kernel that can set the status word:
+// wait for what was enqueued since (copies, events).
+dl_status finish(Workspace &ws, cudaStream_t s) {
+    CK(cudaStreamSynchronize(s));
+    return read_status(ws);
 }
 
 // Upload `count` GEMM problems into the workspace table (device) and return it.
@@ -305,11 +322,9 @@ dl_status tc_bool(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &a
     auto *rbits = static_cast<uint64_t *>(ws.get("bits0", np * wp * 8));
     auto *mbits = static_cast<uint64_t *>(ws.get("bits1", np * wp * 8));
     NEED(C0 && C1 && rbits && mbits);
-    CK(cudaMemsetAsync(ws.scal, 0, kScalars * sizeof(unsigned long long), s));
-    CK(cudaMemsetAsync(ws.status, 0, sizeof(int), s));
+    if (const dl_status zr = reset_scalars(ws, s)) return zr;
     if ((rc = ingest(ctx, ws, s, E, n, np, C0, 1, SC_DMAX, SC_NNZ, SC_COUNT0, &launches))) return rc;
-    if ((rc = read_scalars(ws, s))) return rc;
-    if ((rc = check_status(ws, s))) return rc;
+    if ((rc = read_scalars(ws, s)) || (rc = read_status(ws))) return rc;
     const unsigned long long dmax = host_scal(ws)[SC_DMAX];
     double eps = 0;
     if ((rc = choose_eps(a.eps, 1.0 / (1.0 + static_cast<double>(dmax)), "Lemma 1 (1/(1+||E||))", &eps)))
@@ -391,7 +406,7 @@ dl_status tc_bool(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &a
     }
     if ((rc = write_bits(s, mbits, wp, a.out_bits, n, a.mem))) return rc;
     tm.mark(3);
-    if ((rc = check_status(ws, s))) return rc;
+    if ((rc = finish(ws, s))) return rc;
     if (st) {
         st->path_used = DL_PATH_BOOL_FP8;
         st->eps_used = eps;
@@ -485,8 +500,7 @@ dl_status tc_auto(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &a
     auto *uoff = static_cast<int *>(ws.get("g_units", (np + 1) * 4));
     auto *colmask = static_cast<uint64_t *>(ws.get("g_colmask", wp * 8));
     NEED(C[0] && C[1] && rbits && mbits && cnt && ptr && uoff && colmask);
-    CK(cudaMemsetAsync(ws.scal, 0, kScalars * sizeof(unsigned long long), s));
-    CK(cudaMemsetAsync(ws.status, 0, sizeof(int), s));
+    if (const dl_status zr = reset_scalars(ws, s)) return zr;
     CK(cudaMemsetAsync(colmask, 0, wp * 8, s));
     // one pass over E: the bits of C_0 = I + E, 0/1 check, row counts, ||E||_inf, nnz,
     // self-loops (the e4m3 operand is only built if a squaring happens)
@@ -526,7 +540,8 @@ dl_status tc_auto(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &a
     int *col = nullptr;
     unsigned long long dmax = 0;
     auto emit = [&](const int *g) -> dl_status {
-        CK(cudaMemsetAsync(ws.scal + SC_VIOL, 0, 2 * sizeof(unsigned long long), s));
+        // (the speculative phase's emission finds its counters zeroed; a fill would part it from the sweeps)
+        if (!g) CK(cudaMemsetAsync(ws.scal + SC_VIOL, 0, 2 * sizeof(unsigned long long), s));
         sc.start();
         CK(bits_sweep_csr(ptr, col, uoff, n, rbits, model, wp, 0, ws.scal + SC_VIOL, ws.scal + SC_ONES, &launches, s,
                           g ? 0 : static_cast<int>(dmax), nullptr, colmask, g));
@@ -566,8 +581,7 @@ dl_status tc_auto(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &a
         sc.stop();
         if ((rc = emit(gate))) return rc;
     }
-    if ((rc = read_scalars(ws, s))) return rc;
-    if ((rc = check_status(ws, s))) return rc;
+    if ((rc = read_scalars(ws, s)) || (rc = read_status(ws))) return rc;
     dmax = host_scal(ws)[SC_DMAX];
     ws.last_heavy = dmax > 256;
     double eps = 0;
@@ -609,10 +623,6 @@ dl_status tc_auto(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &a
         NEED(col);
         CK(csr_fill_from_bits(rbits, n, wp, ptr, col, s));
         ++launches;
-        if (!row_direct(static_cast<int>(dmax), wp)) {  // heavy rows: edge-parallel work units
-            CK(sweep_units(ptr, n, cnt, uoff, s));
-            launches += 2;
-        }
     }
     tm.mark(1);
     // ones of C_0 = I + E over the padded size: the diagonal plus the facts off it
@@ -652,6 +662,10 @@ dl_status tc_auto(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &a
         grid = std::min(tiles, ctx->sms);
         return r;
     };
+    if (!spec && !converged && !row_direct(static_cast<int>(dmax), wp)) {  // heavy rows: edge-parallel work units
+        CK(sweep_units(ptr, n, cnt, uoff, s));
+        launches += 2;
+    }
     // sparse graphs planned on the host (at most two facts per row on average, no heavy rows):
     // the Iteration on single rows closes every row whose reachable set stays small in one
     // launch; the rows it leaves open keep what they reached and the sweeps below finish them
@@ -740,7 +754,7 @@ dl_status tc_auto(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &a
     }
     if (!direct && (rc = write_bits(s, mbits, wp, a.out_bits, n, a.mem))) return rc;
     tm.mark(3);
-    if ((rc = check_status(ws, s))) return rc;
+    if ((rc = finish(ws, s))) return rc;
     if (st) {
         st->path_used = DL_PATH_AUTO;
         st->eps_used = eps;
@@ -804,12 +818,10 @@ dl_status tc_fp64(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &a
     auto *G = static_cast<double *>(ws.get("fp64_G", np * ldg * 8));
     auto *scratch = static_cast<double *>(ws.get("fp64_S", 32 * 32 * 8));
     NEED(C0 && mbits && G && scratch);
-    CK(cudaMemsetAsync(ws.scal, 0, kScalars * sizeof(unsigned long long), s));
-    CK(cudaMemsetAsync(ws.status, 0, sizeof(int), s));
+    if (const dl_status zr = reset_scalars(ws, s)) return zr;
     // validation and row sums (the e4m3 copy is not used by this path)
     if ((rc = ingest(ctx, ws, s, E, n, npb, C0, 0, SC_DMAX, SC_NNZ, SC_COUNT0, &launches))) return rc;
-    if ((rc = read_scalars(ws, s))) return rc;
-    if ((rc = check_status(ws, s))) return rc;
+    if ((rc = read_scalars(ws, s)) || (rc = read_status(ws))) return rc;
     const unsigned long long dmax = host_scal(ws)[SC_DMAX];
     double eps = 0;
     if ((rc = choose_eps(a.eps, 1.0 / (1.0 + static_cast<double>(dmax)), "Lemma 1 (1/(1+||E||))", &eps)))
@@ -838,7 +850,7 @@ dl_status tc_fp64(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &a
                              a.mem == DL_MEM_DEVICE ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s));
     }
     tm.mark(3);
-    if ((rc = check_status(ws, s))) return rc;
+    if ((rc = finish(ws, s))) return rc;
     if (st) {
         st->path_used = DL_PATH_FP64;
         st->eps_used = eps;
@@ -870,12 +882,10 @@ dl_status tc_mixed_path(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveA
     auto *C0 = static_cast<uint8_t *>(ws.get("c0", np * np));
     auto *mbits = static_cast<uint64_t *>(ws.get("bits1", np * wp * 8));
     NEED(C0 && mbits);
-    CK(cudaMemsetAsync(ws.scal, 0, kScalars * sizeof(unsigned long long), s));
-    CK(cudaMemsetAsync(ws.status, 0, sizeof(int), s));
+    if (const dl_status zr = reset_scalars(ws, s)) return zr;
     // validation and row sums (the e4m3 copy is not used by this path)
     if ((rc = ingest(ctx, ws, s, E, n, np, C0, 0, SC_DMAX, SC_NNZ, SC_COUNT0, &launches))) return rc;
-    if ((rc = read_scalars(ws, s))) return rc;
-    if ((rc = check_status(ws, s))) return rc;
+    if ((rc = read_scalars(ws, s)) || (rc = read_status(ws))) return rc;
     const unsigned long long dmax = host_scal(ws)[SC_DMAX];
     double eps = 0;
     if ((rc = choose_eps(a.eps, 1.0 / (1.0 + static_cast<double>(dmax)), "Lemma 1 (1/(1+||E||))", &eps)))
@@ -898,7 +908,7 @@ dl_status tc_mixed_path(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveA
                              a.mem == DL_MEM_DEVICE ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s));
     }
     tm.mark(3);
-    if ((rc = check_status(ws, s))) return rc;
+    if ((rc = finish(ws, s))) return rc;
     if (st) {
         st->path_used = DL_PATH_MIXED;
         st->eps_used = eps;
@@ -1026,7 +1036,7 @@ void layers_read(Workspace &ws, Layers *ly) {
 // Returns with *done = false (and nothing written) if the rows are too wide or the
 // iterations exceed the budget: the doubling below then solves the problem.
 dl_status sg_iteration(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &a, dl_stats *st, bool *done,
-                       bool iterate = true, const uint64_t *seed = nullptr) {
+                       bool iterate = true, const uint64_t *seed = nullptr, bool *layered = nullptr) {
     (void)ctx;
     *done = false;
     const int32_t n = a.n;
@@ -1049,8 +1059,7 @@ dl_status sg_iteration(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveAr
     auto *colmask = static_cast<uint64_t *>(ws.get("g_colmask", wp * 8));
     auto *uoff = static_cast<int *>(ws.get("g_units", (np + 1) * 4));
     NEED(S && Y && X && cnt && ptr && colmask && uoff);
-    CK(cudaMemsetAsync(ws.scal, 0, kScalars * sizeof(unsigned long long), s));
-    CK(cudaMemsetAsync(ws.status, 0, sizeof(int), s));
+    if (const dl_status zr = reset_scalars(ws, s)) return zr;
     CK(cudaMemsetAsync(colmask, 0, wp * 8, s));
     // the CSR of P (its bits of I + P go to X, a scratch here) and S_0 = B
     CK(csr_pack_checked(P, n, static_cast<int>(np), wp, cnt, ptr, X, ws.scal + SC_DMAX, ws.scal + SC_NNZ,
@@ -1074,9 +1083,9 @@ dl_status sg_iteration(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveAr
         if ((rc = layers_enqueue(ws, s, X, n, wp, ptr, &ly))) return rc;
         launches += 2;
     }
-    if ((rc = read_scalars(ws, s))) return rc;
-    if ((rc = check_status(ws, s))) return rc;
+    if ((rc = read_scalars(ws, s)) || (rc = read_status(ws))) return rc;
     layers_read(ws, &ly);
+    if (layered) *layered = ly.levels() > 0;
     const double dmax = static_cast<double>(host_scal(ws)[SC_DMAX]);
     double eps = 0;
     if ((rc = choose_eps(a.eps, 1.0 / (1.0 + dmax * dmax), "Sec. 7.2 (1/(1+||P||^2))", &eps))) return rc;
@@ -1139,8 +1148,7 @@ dl_status sg_iteration(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveAr
     ++launches;
     if ((rc = write_bits(s, S, wp, a.out_bits, n, a.mem))) return rc;
     tm.mark(3);
-    if ((rc = read_scalars(ws, s))) return rc;
-    if ((rc = check_status(ws, s))) return rc;
+    if ((rc = read_scalars(ws, s)) || (rc = read_status(ws))) return rc;
     if (st) {
         st->path_used = DL_PATH_AUTO;
         st->eps_used = eps;
@@ -1176,9 +1184,18 @@ dl_status solve_sg(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &
     // Layers, where P has them, are cheaper than either (and found by the same preparation).
     const int tuned_iteration = tuned(ctx, np).sg_iteration;  // measured crossover, when tuned
     const bool iterate = tuned_iteration >= 0 ? tuned_iteration == 1 : np >= 6144;
-    if (a.path == DL_PATH_AUTO && (iterate || !a.no_layers)) {
-        bool done = false;
-        const dl_status rc = sg_iteration(ctx, ws, s, a, st, &done, iterate);
+    // (not looked for in the next kLayerSkips calls of a workspace whose last search found none: it costs
+    // some 30 us, a tenth of a small doubling)
+    constexpr int kLayerSkips = 7;
+    SolveArgs b = a;
+    if (!b.no_layers && ws.layer_skips > 0) {
+        --ws.layer_skips;
+        b.no_layers = true;
+    }
+    if (a.path == DL_PATH_AUTO && (iterate || !b.no_layers)) {
+        bool done = false, layered = false;
+        const dl_status rc = sg_iteration(ctx, ws, s, b, st, &done, iterate, nullptr, &layered);
+        if (!b.no_layers && !layered) ws.layer_skips = kLayerSkips;
         if (rc != DL_OK || done) return rc;
     }
     return sg_doubling(ctx, ws, s, a, st);
@@ -1204,8 +1221,7 @@ dl_status sg_doubling(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArg
     uint8_t *T = static_cast<uint8_t *>(ws.get("c4", np * np));
     auto *sbits = static_cast<uint64_t *>(ws.get("bits0", np * wp * 8));
     NEED(Sa && Sb && Qa && Qb && T && sbits);
-    CK(cudaMemsetAsync(ws.scal, 0, kScalars * sizeof(unsigned long long), s));
-    CK(cudaMemsetAsync(ws.status, 0, sizeof(int), s));
+    if (const dl_status zr = reset_scalars(ws, s)) return zr;
     if ((rc = ingest(ctx, ws, s, P, n, np, Qa, 0, SC_DMAX, SC_NNZ, SC_COUNT0, &launches))) return rc;
     if (Bm) {
         if ((rc = ingest(ctx, ws, s, Bm, n, np, Sa, 0, SC_DMAX2, SC_NNZ2, SC_COUNT2, &launches))) return rc;
@@ -1215,8 +1231,7 @@ dl_status sg_doubling(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArg
             return rc;
     }
     tm.mark(1);
-    if ((rc = read_scalars(ws, s))) return rc;
-    if ((rc = check_status(ws, s))) return rc;
+    if ((rc = read_scalars(ws, s)) || (rc = read_status(ws))) return rc;
     const double dmax = static_cast<double>(host_scal(ws)[SC_DMAX]);
     double eps = 0;
     if ((rc = choose_eps(a.eps, 1.0 / (1.0 + dmax * dmax), "Sec. 7.2 (1/(1+||P||^2))", &eps))) return rc;
@@ -1280,7 +1295,7 @@ dl_status sg_doubling(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArg
     tm.mark(2);
     if ((rc = write_bits(s, sbits, wp, a.out_bits, n, a.mem))) return rc;
     tm.mark(3);
-    if ((rc = check_status(ws, s))) return rc;
+    if ((rc = finish(ws, s))) return rc;
     if (st) {
         st->path_used = DL_PATH_BOOL_FP8;
         st->eps_used = eps;
@@ -1313,8 +1328,7 @@ dl_status solve_compose(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveA
     auto *B8 = static_cast<uint8_t *>(ws.get("c1", np * np));
     auto *bits = static_cast<uint64_t *>(ws.get("bits0", np * wp * 8));
     NEED(A8 && B8 && bits);
-    CK(cudaMemsetAsync(ws.scal, 0, kScalars * sizeof(unsigned long long), s));
-    CK(cudaMemsetAsync(ws.status, 0, sizeof(int), s));
+    if (const dl_status zr = reset_scalars(ws, s)) return zr;
     if ((rc = ingest(ctx, ws, s, R1, n, np, A8, 0, SC_DMAX, SC_NNZ, SC_COUNT0, &launches))) return rc;
     if ((rc = ingest(ctx, ws, s, R2, n, np, B8, 0, SC_DMAX2, SC_NNZ2, SC_COUNT2, &launches))) return rc;
     tm.mark(1);
@@ -1339,8 +1353,7 @@ dl_status solve_compose(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveA
     tm.mark(2);
     if ((rc = write_bits(s, bits, wp, a.out_bits, n, a.mem))) return rc;
     tm.mark(3);
-    if ((rc = read_scalars(ws, s))) return rc;
-    if ((rc = check_status(ws, s))) return rc;
+    if ((rc = read_scalars(ws, s)) || (rc = read_status(ws))) return rc;
     if (st) {
         st->path_used = DL_PATH_BOOL_FP8;
         gc.fill(st);
@@ -1441,8 +1454,7 @@ dl_status solve_sg_real(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveA
     auto *ptr = static_cast<int *>(ws.get("g_ptr", (np + 1) * 4));
     auto *colmask = static_cast<uint64_t *>(ws.get("g_colmask", wp * 8));
     NEED(bits && bitsB && cnt && ptr && colmask);
-    CK(cudaMemsetAsync(ws.scal, 0, kScalars * sizeof(unsigned long long), s));
-    CK(cudaMemsetAsync(ws.status, 0, sizeof(int), s));
+    if (const dl_status zr = reset_scalars(ws, s)) return zr;
     CK(cudaMemsetAsync(colmask, 0, wp * 8, s));
     // P: 0/1 check, ||P||_inf, the CSR; B: 0/1 check
     CK(csr_pack_checked(P, n, static_cast<int>(np), wp, cnt, ptr, bits, ws.scal + SC_DMAX, ws.scal + SC_NNZ,
@@ -1460,8 +1472,7 @@ dl_status solve_sg_real(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveA
         if ((rc = layers_enqueue(ws, s, bits, n, wp, ptr, &ly))) return rc;
         launches += 2;
     }
-    if ((rc = read_scalars(ws, s))) return rc;
-    if ((rc = check_status(ws, s))) return rc;
+    if ((rc = read_scalars(ws, s)) || (rc = read_status(ws))) return rc;
     layers_read(ws, &ly);
     const double dmax = static_cast<double>(host_scal(ws)[SC_DMAX]);
     double eps = 0;
@@ -1899,8 +1910,7 @@ dl_status solve_tail_real(dl_ctx *ctx, Workspace &ws, cudaStream_t s, int32_t n,
     positive_bytes_kernel<<<stream_grid(nn), 256, 0, s>>>(F, nn, Ab, ws.scal + SC_GUARD);
     CK(cudaGetLastError());
     ++launches;
-    if ((rc = read_scalars(ws, s))) return rc;
-    if ((rc = check_status(ws, s))) return rc;
+    if ((rc = read_scalars(ws, s)) || (rc = read_status(ws))) return rc;
     double fmax = 0.0;
     {
         const unsigned long long b = host_scal(ws)[SC_GUARD];
@@ -2156,16 +2166,14 @@ dl_status trans_real_first(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const Sol
     auto *X = static_cast<double *>(ws.get("tr_X", nq * 8));
     auto *U = static_cast<double *>(ws.get("tr_U", nq * 8));
     NEED(T && M && Mt && cnt && ptr && uoff && rank && perm && cnt2 && ptr2 && colmask && X && U);
-    CK(cudaMemsetAsync(ws.scal, 0, kScalars * sizeof(unsigned long long), s));
-    CK(cudaMemsetAsync(ws.status, 0, sizeof(int), s));
+    if (const dl_status zr = reset_scalars(ws, s)) return zr;
     CK(cudaMemsetAsync(colmask, 0, wp * 8, s));
     CK(csr_pack_checked(R1, n, static_cast<int>(np), wp, cnt, ptr, Mt, ws.scal + SC_DMAX, ws.scal + SC_NNZ,
                         ws.scal + SC_COUNT0, ws.status, colmask, s));
     CK(pack_bits(R1, n, static_cast<int>(np), wp, M, ws.status, s));
     launches += 3;
     dl_status rc;
-    if ((rc = read_scalars(ws, s))) return rc;
-    if ((rc = check_status(ws, s))) return rc;
+    if ((rc = read_scalars(ws, s)) || (rc = read_status(ws))) return rc;
     const unsigned long long dmax = host_scal(ws)[SC_DMAX];
     double eps = 0;
     if ((rc = choose_eps(a.eps, 1.0 / (1.0 + static_cast<double>(dmax)), "Sec. 6.2 (1/(1+||R1||_inf))", &eps)))
@@ -2282,7 +2290,7 @@ dl_status trans_real_first(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const Sol
     }
     if ((rc = write_bits(s, M, wp, a.out_bits, n, a.mem))) return rc;
     tm->mark(3);
-    if ((rc = check_status(ws, s))) return rc;
+    if ((rc = finish(ws, s))) return rc;
     if (st) {
         st->path_used = DL_PATH_FP64;
         st->eps_used = eps;
@@ -2352,11 +2360,9 @@ dl_status solve_transposed(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const Sol
     auto *Bu = static_cast<uint8_t *>(ws.get("tr_bu8", std::max<size_t>(static_cast<size_t>(n) * n, 16)));
     auto *Mw = static_cast<uint64_t *>(ws.get("tr_bits", std::max<size_t>(static_cast<size_t>(n) * w * 8, 16)));
     NEED(R8 && B8 && Bu && Mw);
-    CK(cudaMemsetAsync(ws.scal, 0, kScalars * sizeof(unsigned long long), s));
-    CK(cudaMemsetAsync(ws.status, 0, sizeof(int), s));
+    if (const dl_status zr = reset_scalars(ws, s)) return zr;
     if ((rc = ingest(ctx, ws, s, R1, n, np, R8, 0, SC_DMAX, SC_NNZ, SC_COUNT0, &launches))) return rc;
-    if ((rc = read_scalars(ws, s))) return rc;
-    if ((rc = check_status(ws, s))) return rc;
+    if ((rc = read_scalars(ws, s)) || (rc = read_status(ws))) return rc;
     const unsigned long long dmax = host_scal(ws)[SC_DMAX];
     double eps = 0;
     if ((rc = choose_eps(a.eps, 1.0 / (1.0 + static_cast<double>(dmax)), "Sec. 6.2 (1/(1+||R1||_inf))", &eps)))
@@ -2381,8 +2387,7 @@ dl_status solve_transposed(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const Sol
     e4m3_to_u8_kernel<<<static_cast<unsigned>((nn + 255) / 256), 256, 0, s>>>(B8, np, n, Bu);
     CK(cudaGetLastError());
     launches += 2;
-    if ((rc = read_scalars(ws, s))) return rc;  // (the GEMM table's staging is free again)
-    if ((rc = check_status(ws, s))) return rc;
+    if ((rc = read_scalars(ws, s)) || (rc = read_status(ws))) return rc;  // (the GEMM table's staging is free again)
     const double b_gemm_ms = gc.ms(), b_gemm_flops = gc.timed_flops;  // (its events are reused below)
     tm.mark(1);
     SolveArgs b = a;
@@ -2466,7 +2471,7 @@ dl_status solve_transposed(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const Sol
         differ = host_scal(ws)[SC_GUARD + 1];
     }
     tm.mark(3);
-    if ((rc = check_status(ws, s))) return rc;
+    if ((rc = finish(ws, s))) return rc;
     if (st) {
         st->path_used = real ? DL_PATH_FP64 : sgst.path_used;
         st->eps_used = eps;
@@ -2494,10 +2499,11 @@ cudaError_t Workspace::init() {
         if ((e = host_pinned_alloc(&host_pinned, kHostPinned)) != cudaSuccess) return e;
         host_bytes = kHostPinned;
     }
-    if (!status && (e = device_alloc(reinterpret_cast<void **>(&status), 256)) != cudaSuccess) return e;
-    if (!scal && (e = device_alloc(reinterpret_cast<void **>(&scal), kScalars * sizeof(unsigned long long))) !=
+    // the status word lies behind the scalars: one copy reads both
+    if (!scal && (e = device_alloc(reinterpret_cast<void **>(&scal), kScalars * sizeof(unsigned long long) + 256)) !=
                      cudaSuccess)
         return e;
+    status = reinterpret_cast<int *>(scal + kScalars);
     for (auto &x : ev)
         if (!x && (e = cudaEventCreate(&x)) != cudaSuccess) return e;
     for (auto &x : gev)
@@ -2519,8 +2525,7 @@ void Workspace::release() {
         if (kv.second.p) cudaFree(kv.second.p);
     bufs.clear();
     if (host_pinned) cudaFreeHost(host_pinned);
-    if (status) cudaFree(status);
-    if (scal) cudaFree(scal);
+    if (scal) cudaFree(scal);  // (and the status word with it)
     for (auto &x : ev)
         if (x) cudaEventDestroy(x);
     for (auto &x : gev)
