@@ -402,6 +402,152 @@ __global__ void __launch_bounds__(256)
         atomicAdd(open_rows, 1ull);
 }
 
+// ---- rows of the model by reachability ------------------------------------------------------
+// Heavy-tailed relations with small closures (a citation-like DAG of 16384 constants: rows of up to
+// thousands of successors, 32 reachable constants on average): the model's row i is what paths of one
+// edge or more reach from i, found by a breadth-first walk over the successor lists with the row's bits
+// in shared memory.  A sweep over such a relation reads nnz rows of 2 KB (164 MB at n = 16384: 163 us,
+// and nine are needed); the walks read each reached constant's list once.
+//  (1) reach_rows_kernel: a warp per row, lanes take frontier constants, whole warps the long lists.  A
+//      row whose frontier outgrows kReachFront or whose paths are longer than kReachSteps stays open.
+//  (2) reach_open_kernel: a CTA per open row, any frontier.  It gives all up when too many are open
+//      (the closure is not small: sweeps and squarings are for that).
+constexpr int kReachFront = 512, kReachSteps = 64, kReachLight = 16;
+
+// The successors of the constants nodes[0 .. cnt), 32 per turn from `first` on by `stride`: visit(j) for
+// every one, short lists by their lane, long ones by the warp.  A lane leaves off once visit says so
+// (a walk that has outgrown its frontier: a hub's list would be read for nothing).
+template <class Visit>
+__device__ __forceinline__ void expand_nodes(const int *__restrict__ ptr, const int *__restrict__ col,
+                                             const uint16_t *nodes, int cnt, int first, int stride, Visit visit) {
+    bool on = true;
+    const int lane = threadIdx.x & 31;
+    for (int f0 = first; f0 < cnt; f0 += stride) {
+        const bool live = f0 + lane < cnt;
+        const int k = live ? nodes[f0 + lane] : 0;
+        const int q0 = live ? ptr[k] : 0, q1 = live ? ptr[k + 1] : 0;
+        const bool heavy = q1 - q0 > kReachLight;
+        if (!heavy)
+            for (int q = q0; q < q1 && on; ++q) on = visit(col[q]);
+        if (!__any_sync(0xffffffffu, on)) return;
+        for (unsigned left = __ballot_sync(0xffffffffu, heavy); left != 0u; left &= left - 1) {
+            const int src = __ffs(left) - 1;
+            const int h0 = __shfl_sync(0xffffffffu, q0, src), h1 = __shfl_sync(0xffffffffu, q1, src);
+            for (int q = h0 + lane; q < h1 && on; q += 32) on = visit(col[q]);
+            if (!__any_sync(0xffffffffu, on)) return;
+        }
+    }
+}
+
+// counters[0] = open rows, [1] = rows given up, [2] = ones of the rows written.
+__global__ void __launch_bounds__(256)
+    reach_rows_kernel(const int *__restrict__ ptr, const int *__restrict__ col, int n, int wp, uint64_t *__restrict__ out,
+                      int *__restrict__ open_rows, unsigned *counters) {
+    extern __shared__ uint64_t reach_s[];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    // per warp: the row's bits, two frontiers, the next frontier's length
+    uint64_t *bits = reach_s + static_cast<size_t>(wid) * (wp + kReachFront / 2 + 1);
+    uint16_t *front = reinterpret_cast<uint16_t *>(bits + wp);
+    int *next_cnt = reinterpret_cast<int *>(front + 2 * kReachFront);
+    const int i = blockIdx.x * (blockDim.x >> 5) + wid;
+    if (i >= n) return;
+    // (with an eighth of the rows open the second kernel gives up: this one need not go on)
+    unsigned open_now = lane == 0 ? *reinterpret_cast<volatile unsigned *>(counters) : 0u;
+    open_now = __shfl_sync(0xffffffffu, open_now, 0);
+    if (open_now > static_cast<unsigned>(n) / 8) return;
+    for (int w = lane; w < wp; w += 32) bits[w] = 0ull;
+    if (lane == 0) front[0] = static_cast<uint16_t>(i);
+    int cnt = 1, cur = 0, steps = 0;
+    bool closed = true;
+    __syncwarp();
+    while (cnt > 0) {
+        if (cnt > kReachFront || ++steps > kReachSteps) {
+            closed = false;
+            break;
+        }
+        if (lane == 0) *next_cnt = 0;
+        __syncwarp();
+        uint16_t *fn = front + (cur ^ 1) * kReachFront;
+        expand_nodes(ptr, col, front + cur * kReachFront, cnt, 0, 32, [&](int j) {
+            const unsigned b = 1u << (j & 31);
+            if (atomicOr(reinterpret_cast<unsigned *>(bits) + (j >> 5), b) & b) return true;
+            const int pos = atomicAdd(next_cnt, 1);
+            if (pos < kReachFront) fn[pos] = static_cast<uint16_t>(j);
+            return pos < kReachFront;
+        });
+        __syncwarp();
+        cnt = *next_cnt;
+        __syncwarp();  // every lane has read the count before lane 0 clears it
+        cur ^= 1;
+    }
+    if (!closed) {
+        if (lane == 0) open_rows[atomicAdd(counters, 1u)] = i;
+        return;
+    }
+    unsigned ones = 0;
+    for (int w = lane; w < wp; w += 32) {
+        out[static_cast<int64_t>(i) * wp + w] = bits[w];
+        ones += __popcll(bits[w]);
+    }
+    ones = __reduce_add_sync(0xffffffffu, ones);
+    if (lane == 0 && ones) atomicAdd(reinterpret_cast<unsigned long long *>(counters + 2), static_cast<unsigned long long>(ones));
+}
+
+__global__ void __launch_bounds__(256)
+    reach_open_kernel(const int *__restrict__ ptr, const int *__restrict__ col, int n, int wp, uint64_t *__restrict__ out,
+                      const int *__restrict__ open_rows, unsigned *counters) {
+    extern __shared__ uint64_t reach_s[];
+    uint64_t *bits = reach_s, *done = bits + wp;              // reached; reached and expanded
+    uint16_t *list = reinterpret_cast<uint16_t *>(done + wp);  // the step's constants (at most n)
+    __shared__ int cnt_s;
+    const unsigned open = counters[0];
+    if (open > static_cast<unsigned>(n) / 8) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) counters[1] = open;
+        return;
+    }
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (unsigned t = blockIdx.x; t < open; t += gridDim.x) {
+        const int i = open_rows[t];
+        for (int w = threadIdx.x; w < wp; w += blockDim.x) bits[w] = done[w] = 0ull;
+        if (threadIdx.x == 0) {
+            list[0] = static_cast<uint16_t>(i);
+            cnt_s = 1;
+        }
+        __syncthreads();
+        int cnt = 1, steps = 0;
+        while (cnt > 0 && steps < 2 * kReachSteps) {
+            ++steps;
+            expand_nodes(ptr, col, list, cnt, 32 * warp, static_cast<int>(blockDim.x), [&](int j) {
+                atomicOr(reinterpret_cast<unsigned *>(bits) + (j >> 5), 1u << (j & 31));
+                return true;
+            });
+            __syncthreads();
+            if (threadIdx.x == 0) cnt_s = 0;
+            __syncthreads();
+            for (int w = threadIdx.x; w < wp; w += blockDim.x) {
+                uint64_t x = bits[w] & ~done[w];
+                if (x == 0ull) continue;
+                done[w] |= x;
+                int at = atomicAdd(&cnt_s, __popcll(x));
+                for (; x != 0ull; x &= x - 1)
+                    list[at++] = static_cast<uint16_t>(64 * w + __ffsll(static_cast<long long>(x)) - 1);
+            }
+            __syncthreads();
+            cnt = cnt_s;
+        }
+        unsigned ones = 0;
+        for (int w = threadIdx.x; w < wp; w += blockDim.x) {
+            out[static_cast<int64_t>(i) * wp + w] = bits[w];
+            ones += __popcll(bits[w]);
+        }
+        ones = __reduce_add_sync(0xffffffffu, ones);
+        if (lane == 0 && ones)
+            atomicAdd(reinterpret_cast<unsigned long long *>(counters + 2), static_cast<unsigned long long>(ones));
+        if (threadIdx.x == 0 && cnt > 0) atomicAdd(counters + 1, 1u);  // a path too long for the walk
+        __syncthreads();
+    }
+}
+
 // ---- same generation on bits --------------------------------------------------------------
 // 64 x 64 bit-block transpose, one warp per block (lane l holds rows l and l + 32 of the
 // block; bit c of a word is column c): the off-diagonal j x j sub-blocks of every 2j x 2j
@@ -713,6 +859,19 @@ cudaError_t row_iteration(const int *ptr, const int *col, int n, int64_t wp, uin
     const size_t smem = 8 * (static_cast<size_t>(wp) + kRowFront + 1) * sizeof(uint64_t);
     return launch_programmatic(row_iteration_kernel, dim3(static_cast<unsigned>((n + 7) / 8)), dim3(256), smem, s, ptr,
                                col, n, static_cast<int>(wp), M, open_rows, gate);
+}
+
+cudaError_t reach_rows(const int *ptr, const int *col, int n, int64_t wp, uint64_t *out, int *open_rows,
+                       unsigned *counters, cudaStream_t s) {
+    if (n <= 0) return cudaSuccess;
+    if (wp > 256) return cudaErrorInvalidValue;  // 16-bit names of constants, rows in shared memory
+    const size_t smem = 8 * (static_cast<size_t>(wp) + kReachFront / 2 + 1) * sizeof(uint64_t);
+    reach_rows_kernel<<<static_cast<unsigned>((n + 7) / 8), 256, smem, s>>>(ptr, col, n, static_cast<int>(wp), out,
+                                                                          open_rows, counters);
+    const size_t smem_open = static_cast<size_t>(wp) * 2 * sizeof(uint64_t) + static_cast<size_t>(wp) * 64 * sizeof(uint16_t);
+    reach_open_kernel<<<static_cast<unsigned>(num_sms() * 4), 256, smem_open, s>>>(ptr, col, n, static_cast<int>(wp),
+                                                                                 out, open_rows, counters);
+    return cudaGetLastError();
 }
 
 cudaError_t bits_transpose(const uint64_t *src, uint64_t *dst, int np, int64_t wp, const unsigned long long *skip,

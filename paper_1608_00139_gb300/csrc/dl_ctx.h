@@ -51,6 +51,7 @@ struct Workspace {
     int mx_graph_launches = 0;
     BatchPlan *batch_plan = nullptr;
     bool last_heavy = false;  // the last closure on this workspace had rows of > 256 successors
+    bool last_wide = false;   // ... and a model of more than 256 facts per row (no walks next time)
     int layer_skips = 0;      // same-generation calls left before layers are looked for again
     bool last_rows_closed = false;  // ... was closed by the Iteration on single rows alone
     bool last_dense = false;        // ... had more than two facts per row (no single-row Iteration)

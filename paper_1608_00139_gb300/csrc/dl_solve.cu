@@ -662,6 +662,26 @@ dl_status tc_auto(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &a
         grid = std::min(tiles, ctx->sms);
         return r;
     };
+    // rows of more than 256 successors: the model by walks over the successor lists, which a closure of
+    // few facts per row (a citation-like DAG) needs no more than (n = 16384: 2.05 ms by sweeps, 0.36 ms);
+    // given up on the device when it is not, and not tried after a heavy closure that was wide
+    if (!spec && !dense && dmax > 256 && wp <= 256 && !ws.last_wide) {
+        auto *open_rows = static_cast<int *>(ws.get("g_open", (np + 1) * 4));
+        NEED(open_rows);
+        auto *counters = reinterpret_cast<unsigned *>(ws.scal + SC_OPEN);
+        CK(cudaMemsetAsync(counters, 0, 2 * sizeof(unsigned long long), s));
+        sc.start();
+        CK(reach_rows(ptr, col, n, wp, model, open_rows, counters, s));
+        sc.stop();
+        launches += 2;
+        if ((rc = read_scalars(ws, s))) return rc;
+        const auto *h = reinterpret_cast<const unsigned *>(host_scal(ws) + SC_OPEN);
+        if (h[1] == 0) {
+            host_scal(ws)[SC_ONES] = host_scal(ws)[SC_OPEN + 1];
+            host_scal(ws)[SC_VIOL] = 0;
+            converged = emitted = true;
+        }
+    }
     if (!spec && !converged && !row_direct(static_cast<int>(dmax), wp)) {  // heavy rows: edge-parallel work units
         CK(sweep_units(ptr, n, cnt, uoff, s));
         launches += 2;
@@ -752,6 +772,7 @@ dl_status tc_auto(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &a
         set_error("internal: converged closure failed its certificate");
         return DL_EDEVICE;
     }
+    if (ws.last_heavy) ws.last_wide = host_scal(ws)[SC_ONES] > 256ull * static_cast<unsigned long long>(n);
     if (!direct && (rc = write_bits(s, mbits, wp, a.out_bits, n, a.mem))) return rc;
     tm.mark(3);
     if ((rc = finish(ws, s))) return rc;
