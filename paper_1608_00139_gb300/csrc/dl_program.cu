@@ -64,10 +64,23 @@ struct Factor {
     bool transposed = false, negated = false;
 };
 
+// The byte matrices a program's runs work on, kept between them (cudaMalloc and cudaFree of a dozen
+// matrices took 0.9 of a run's 1.4 ms at n = 2048); as many as the largest run needed, freed with the
+// program.  A program's calls are serialised by its context.
+struct MatrixStore {
+    struct Block {
+        void *p;
+        size_t bytes;
+        bool used;
+    };
+    std::vector<Block> blocks;
+};
+
 }  // namespace dl
 
 struct dl_program {
     dl_ctx *ctx = nullptr;
+    dl::MatrixStore store;
     std::vector<dl::PClause> clauses;
     std::set<std::string> idb, edb;
     std::vector<std::vector<std::string>> layers;  // topological order
@@ -285,41 +298,73 @@ __global__ void transpose_u8_kernel(const uint8_t *__restrict__ src, int n, uint
     }
 }
 
+// The byte kernels take 16 bytes per step (the matrices are allocations of their own, so aligned) and the
+// last few one by one: 4 MiB in 10-15 us byte by byte, bound by the instructions.
 __global__ void or_u8_kernel(uint8_t *__restrict__ dst, const uint8_t *__restrict__ src, int64_t count) {
-    for (int64_t t = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; t < count;
-         t += static_cast<int64_t>(gridDim.x) * blockDim.x)
-        dst[t] |= src[t];
+    const int64_t t0 = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
+    const int64_t step = static_cast<int64_t>(gridDim.x) * blockDim.x, chunks = count / 16;
+    for (int64_t t = t0; t < chunks; t += step) {
+        uint4 d = reinterpret_cast<const uint4 *>(dst)[t];
+        const uint4 x = reinterpret_cast<const uint4 *>(src)[t];
+        d.x |= x.x, d.y |= x.y, d.z |= x.z, d.w |= x.w;
+        reinterpret_cast<uint4 *>(dst)[t] = d;
+    }
+    if (t0 < count - 16 * chunks) dst[16 * chunks + t0] |= src[16 * chunks + t0];
 }
 
 __global__ void complement_u8_kernel(const uint8_t *__restrict__ src, int64_t count, uint8_t *__restrict__ dst) {
-    for (int64_t t = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; t < count;
-         t += static_cast<int64_t>(gridDim.x) * blockDim.x)
-        dst[t] = src[t] ? 0 : 1;
+    const int64_t t0 = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
+    const int64_t step = static_cast<int64_t>(gridDim.x) * blockDim.x, chunks = count / 16;
+    for (int64_t t = t0; t < chunks; t += step) {  // (0/1 bytes: checked before a run)
+        uint4 x = reinterpret_cast<const uint4 *>(src)[t];
+        x.x ^= 0x01010101u, x.y ^= 0x01010101u, x.z ^= 0x01010101u, x.w ^= 0x01010101u;
+        reinterpret_cast<uint4 *>(dst)[t] = x;
+    }
+    if (t0 < count - 16 * chunks) dst[16 * chunks + t0] = src[16 * chunks + t0] ? 0 : 1;
 }
 
+// *diff += 16-byte pieces (or single bytes at the end) in which a and b differ.
 __global__ void differ_u8_kernel(const uint8_t *__restrict__ a, const uint8_t *__restrict__ b, int64_t count,
                                  unsigned long long *diff) {
+    const int64_t t0 = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
+    const int64_t step = static_cast<int64_t>(gridDim.x) * blockDim.x, chunks = count / 16;
     unsigned long long d = 0;
-    for (int64_t t = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; t < count;
-         t += static_cast<int64_t>(gridDim.x) * blockDim.x)
-        d += a[t] != b[t];
+    for (int64_t t = t0; t < chunks; t += step) {
+        const uint4 x = reinterpret_cast<const uint4 *>(a)[t], y = reinterpret_cast<const uint4 *>(b)[t];
+        d += ((x.x ^ y.x) | (x.y ^ y.y) | (x.z ^ y.z) | (x.w ^ y.w)) != 0u;
+    }
+    if (t0 < count - 16 * chunks) d += a[16 * chunks + t0] != b[16 * chunks + t0];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
     if ((threadIdx.x & 31) == 0 && d) atomicAdd(diff, d);
 }
 
-unsigned grid_for(int64_t count) { return static_cast<unsigned>(std::min<int64_t>((count + 255) / 256, 8192)); }
+unsigned grid_for(int64_t count) {
+    return static_cast<unsigned>(std::max<int64_t>(1, std::min<int64_t>((count / 16 + 255) / 256, 2048)));
+}
 
-// Relations of one run: device byte matrices owned by the run (freed at its end).
+// Byte matrices of one run, taken from the program's store and given back to it at the run's end (every
+// run ends with a wait for its stream, a failed one too, so the next may use them on any stream).
 struct Pool {
-    std::vector<void *> owned;
+    MatrixStore &store;
+    std::vector<size_t> taken;
+    explicit Pool(MatrixStore &m) : store(m) {}
+    Pool(const Pool &) = delete;
     ~Pool() {
-        for (void *p : owned) cudaFree(p);
+        for (size_t k : taken) store.blocks[k].used = false;
     }
     uint8_t *alloc(size_t bytes) {
+        bytes = std::max<size_t>(bytes, 16);
+        for (size_t k = 0; k < store.blocks.size(); ++k)
+            if (!store.blocks[k].used && store.blocks[k].bytes == bytes) {
+                store.blocks[k].used = true;
+                taken.push_back(k);
+                return static_cast<uint8_t *>(store.blocks[k].p);
+            }
         void *p = nullptr;
-        if (device_alloc(&p, std::max<size_t>(bytes, 16)) != cudaSuccess) return nullptr;
-        owned.push_back(p);
+        if (device_alloc(&p, bytes) != cudaSuccess) return nullptr;
+        store.blocks.push_back(MatrixStore::Block{p, bytes, true});
+        taken.push_back(store.blocks.size() - 1);
         return static_cast<uint8_t *>(p);
     }
 };
@@ -523,6 +568,7 @@ dl_status program_create(dl_ctx *ctx, const char *text, dl_program **out) {
 void program_destroy(dl_program *p) {
     if (!p) return;
     for (auto &kv : p->rel) cudaFree(kv.second);
+    for (auto &b : p->store.blocks) cudaFree(b.p);
     delete p;
 }
 
@@ -563,7 +609,7 @@ dl_status program_run(dl_ctx *ctx, Workspace &ws, cudaStream_t s, dl_program *p,
     const int32_t n = p->n;
     const size_t nbytes = std::max<size_t>(static_cast<size_t>(n) * n, 16);
     std::ostringstream plan;
-    Pool pool;
+    Pool pool(p->store);
     Runner R{ctx, ws, s, n, &pool};
     dl_status rc;
     std::map<std::string, uint8_t *> model;  // this run's models (pool-owned until kept)
@@ -619,6 +665,7 @@ dl_status program_run(dl_ctx *ctx, Workspace &ws, cudaStream_t s, dl_program *p,
         } else {
             // the layer's equations: A_h = OR of the non-recursive clauses' products, and the terms
             std::vector<uint8_t *> A(M, nullptr);
+            std::vector<std::vector<const uint8_t *>> parts(M);  // the matrices that A_h is the OR of
             std::vector<std::vector<Term>> terms(M);
             for (int h = 0; h < M; ++h)
                 if ((rc = R.zero(&A[h]))) return rc;
@@ -634,6 +681,7 @@ dl_status program_run(dl_ctx *ctx, Workspace &ws, cudaStream_t s, dl_program *p,
                 if (rpos < 0) {
                     if ((rc = chain_product(fs, 0, fs.size(), &t.A))) return rc;
                     if ((rc = R.or_into(A[h], t.A))) return rc;
+                    parts[h].push_back(t.A);
                 } else {
                     t.recursive = true;
                     t.j = idx[fs[rpos].pred];
@@ -702,7 +750,10 @@ dl_status program_run(dl_ctx *ctx, Workspace &ws, cudaStream_t s, dl_program *p,
                     uint8_t *B0 = Bj[0][0];
                     uint64_t *bits = R.bitbuf();
                     if (!bits) return DL_ENOMEM;
-                    if ((rc = tail(n, B0, Aa[0], bits))) return rc;
+                    // r <- b, r <- b r (or r b): A and B0 are one matrix, which solve_tail is told
+                    const bool closure = terms[0].size() == 1 && parts[0].size() == 1 &&
+                                         (left ? terms[0][0].B : terms[0][0].C) == parts[0][0];
+                    if ((rc = tail(n, closure ? Aa[0] : B0, Aa[0], bits))) return rc;
                     if ((rc = R.unpack(bits, &out[0]))) return rc;
                 } else {  // the stacked system over M n constants: R = min1(A + B R)
                     const int32_t N = M * n;
@@ -769,7 +820,7 @@ dl_status program_run(dl_ctx *ctx, Workspace &ws, cudaStream_t s, dl_program *p,
                         return DL_ENOTCONV;
                     }
                     {
-                        Pool inner;
+                        Pool inner(p->store);
                         R.pool = &inner;
                         for (int h = 0; h < M && !rc; ++h) {
                             if ((rc = R.copy(nxt[h], A[h]))) break;

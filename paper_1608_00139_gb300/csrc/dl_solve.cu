@@ -1768,9 +1768,11 @@ dl_status solve_tail(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs
         if ((rc = solve_tc(ctx, ws, s, r, &sr))) return rc;
         thresh_ones = sr.model_ones;
     }
-    auto *cl = static_cast<uint64_t *>(ws.get("tr_cl", static_cast<size_t>(n) * w * 8));
-    auto *clb = static_cast<uint8_t *>(ws.get("tr_clb", std::max<size_t>(static_cast<size_t>(n) * n, 16)));
-    NEED(cl && clb);
+    const bool closure = a.E == a.E2;  // A = B0: the model is B0^+ itself
+    auto *cl = closure && a.mem == DL_MEM_DEVICE
+                   ? a.out_bits
+                   : static_cast<uint64_t *>(ws.get("tr_cl", static_cast<size_t>(n) * w * 8));
+    NEED(cl);
     SolveArgs c;
     c.n = n;
     c.E = B0;
@@ -1779,16 +1781,26 @@ dl_status solve_tail(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs
     c.path = a.path == DL_PATH_BOOL_FP8 ? DL_PATH_BOOL_FP8 : DL_PATH_AUTO;
     c.out_bits = cl;
     if ((rc = solve_tc(ctx, ws, s, c, &sc))) return rc;  // B0^+ (and eps checked against ||B0||)
-    CK(unpack_bits_u8(cl, n, clb, ws.status, s));
-    CK(cudaMemset2DAsync(clb, static_cast<size_t>(n) + 1, 1, 1, n, s));  // + I: the diagonal bytes
-    SolveArgs m;
-    m.n = n;
-    m.E = clb;
-    m.E2 = A;
-    m.e_device = true;
-    m.mem = a.mem;
-    m.out_bits = a.out_bits;
-    if ((rc = solve_compose(ctx, ws, s, m, &sm))) return rc;  // min1((I + B0^+) A)
+    if (closure) {
+        if (cl != a.out_bits) {
+            CK(cudaMemcpyAsync(a.out_bits, cl, static_cast<size_t>(n) * w * 8, cudaMemcpyDeviceToHost, s));
+            CK(cudaStreamSynchronize(s));
+        }
+        sm.model_ones = sc.model_ones;
+    } else {
+        auto *clb = static_cast<uint8_t *>(ws.get("tr_clb", std::max<size_t>(static_cast<size_t>(n) * n, 16)));
+        NEED(clb);
+        CK(unpack_bits_u8(cl, n, clb, ws.status, s));
+        CK(cudaMemset2DAsync(clb, static_cast<size_t>(n) + 1, 1, 1, n, s));  // + I: the diagonal bytes
+        SolveArgs m;
+        m.n = n;
+        m.E = clb;
+        m.E2 = A;
+        m.e_device = true;
+        m.mem = a.mem;
+        m.out_bits = a.out_bits;
+        if ((rc = solve_compose(ctx, ws, s, m, &sm))) return rc;  // min1((I + B0^+) A)
+    }
     if (st) {
         st->path_used = a.path;
         st->eps_used = real ? sr.eps_used : sc.eps_used;
