@@ -1,20 +1,23 @@
 // dl_batch.cu -- many independent closure problems of uneven size in one call (dl_tc_batch).
 //
 // Every instance k gets the AUTO closure of dl_solve.cu (Iteration steps on bits, with
-// repeated squaring of the reflexive closure for the instances that keep changing), but all
-// instances advance together and every decision is taken on the device:
-//   1. (every call) one pass over all inputs packs the bits of I + E_k, checks that every
-//      byte is 0/1 and counts successors; a scan gives one CSR over all instances' rows.
-//   2. (captured CUDA graph) fill the CSR column indices from the packed bits; 24 batched
-//      in-place sweeps M <- M | E | E M; an instance whose sweep changes nothing holds its
-//      reflexive closure and leaves the active list.  Then rounds for the instances still
-//      active: their bits become e4m3 operands, one persistent grouped tcgen05 launch squares
-//      exactly those instances (a tile schedule written on the device), 4 more sweeps.
-//      Finally the model E_k C_k* of every instance with its certificate C = min1(I + E C).
-// After every sweep a single-CTA kernel rebuilds the list of active instances (their rows,
-// padded rows and GEMM tiles as prefix sums), so that later kernels touch only live rows and
-// a round with nothing left active costs a few empty launches.  The graph is cached and
-// relaunched while the inputs and outputs stay the same buffers.
+// repeated squaring of the reflexive closure for the instances that keep changing):
+//   1. One pass over all inputs packs the bits of I + E_k, checks that every byte is 0/1 and
+//      counts successors; a scan gives one CSR over all instances' rows, a second pass fills it.
+//   2. The columns of M <- M | E M are independent of one another, so every instance of up to
+//      kSliceRows constants is cut into column slices that fit a CTA's shared memory: each
+//      slice iterates there until nothing changes and writes its columns of the model E C*
+//      with the certificate C = min1(I + E C).  No slice waits for another.
+//   3. Only instances with a slice that still changed after kSliceSweeps sweeps, and larger
+//      ones, go on together (a captured CUDA graph, every decision on the device): 24 batched
+//      in-place sweeps; an instance whose sweep changes nothing leaves the active list.  Then
+//      rounds for the instances still active: their bits become e4m3 operands, one persistent
+//      grouped tcgen05 launch squares exactly those instances (a tile schedule written on the
+//      device), 4 more sweeps.  Finally their models and certificates.  After every sweep a
+//      single-CTA kernel rebuilds the list of active instances (their rows, padded rows and
+//      GEMM tiles as prefix sums), so that later kernels touch only live rows and a round with
+//      nothing left active costs a few empty launches.  The graph reads its pointers from
+//      tables that every call uploads; it is kept while the sizes and the work space stay.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -38,6 +41,7 @@ constexpr int kRoundSweeps = 4;   // sweeps after each squaring round
 constexpr int kMainRounds = 2;    // squaring rounds in the main graph (the rest only if needed)
 constexpr int kChunk = 32;        // rows a warp claims at a time in the row kernels
 constexpr int kListThreads = 1024;
+constexpr int kBatchBn = 128;     // GEMM tile width (small instances waste less padding)
 
 struct BatchInst {
     const uint8_t *E;  // n x n input bytes on the device (row stride n)
@@ -87,164 +91,390 @@ __global__ void batch_map_kernel(const BatchInst *__restrict__ inst, int *pinst)
 }
 
 // Bits of row r of I + E_k into M, the row's successor count and the 0/1 check.  A warp takes
-// kPackRows consecutive padded rows and looks the instance up again only where the rows cross
-// into the next one (rows are short: per-row lookups would put two dependent loads before
-// every row's own).
-constexpr int kPackRows = 4;
+// kPackRows consecutive padded rows, 32 words of a row at a time: 16 bytes a lane, four
+// coalesced 512-byte loads (and the 16-byte block behind them where the row starts off a
+// 16-byte boundary), those of the next step in flight while this one's are packed.  The 16-bit
+// pieces meet in shared memory, where word w is read at its bit offset.  Bound by the read of
+// the bytes: 1024 instances of 33..2044 constants, 1.43 GB, 547 -> PACK_US us (PACK_TB TB/s; each
+// lane loading its own word's 64 bytes, and a row's loads only after the row before was
+// packed, left both the L1 lines and the memory idle half of the time).
+constexpr int kPackRows = 8;
+constexpr int kPackBuf = 36;  // 64-bit words of a step's bits: 2064 bits and the word behind
 
 __global__ void __launch_bounds__(256, 4)
     batch_pack_kernel(const BatchInst *__restrict__ inst, const int *__restrict__ pinst, int total_prows,
                       int *cnt, int *status) {
-    const int lane = threadIdx.x & 31;
-    const int g0 = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * kPackRows;
+    __shared__ uint64_t buf_s[8][2][kPackBuf];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int g0 = (blockIdx.x * (blockDim.x >> 5) + warp) * kPackRows;
     if (g0 >= total_prows) return;
     const int g1 = min(g0 + kPackRows, total_prows);
-    int k = pinst[g0];
-    const uint8_t *E = inst[k].E;
-    uint64_t *rbits = inst[k].rbits;
-    int n = inst[k].n, np = inst[k].np, wp = inst[k].wp, prow0 = inst[k].prow0, row0 = inst[k].row0;
-    for (int g = g0; g < g1; ++g) {
-        if (g - prow0 >= np) {  // the next instance
-            k = pinst[g];
-            E = inst[k].E;
-            rbits = inst[k].rbits;
-            n = inst[k].n;
-            np = inst[k].np;
-            wp = inst[k].wp;
-            prow0 = inst[k].prow0;
-            row0 = inst[k].row0;
+    if (lane < 2 * (kPackBuf - 32)) buf_s[warp][lane & 1][32 + (lane >> 1)] = 0ull;  // never written beyond 16 bits
+    __syncwarp();
+    struct Cursor {  // a step: the words [32 seg, 32 seg + 32) of padded row g
+        const uint8_t *E;
+        uint64_t *rbits;
+        int g, seg, n, np, wp, prow0, row0;
+    };
+    auto open = [&](Cursor &c, int k) {
+        c.E = inst[k].E;
+        c.rbits = inst[k].rbits;
+        c.n = inst[k].n;
+        c.np = inst[k].np;
+        c.wp = inst[k].wp;
+        c.prow0 = inst[k].prow0;
+        c.row0 = inst[k].row0;
+    };
+    auto step = [&](Cursor &c) {
+        if (c.g - c.prow0 < c.n && 32 * (c.seg + 1) < c.wp) {
+            ++c.seg;
+            return;
         }
-        const int r = g - prow0;
-        uint64_t *row = rbits + static_cast<int64_t>(r) * wp;
-        if (r >= n) {  // padding: identity only
-            for (int w = lane; w < wp; w += 32) row[w] = w == (r >> 6) ? 1ull << (r & 63) : 0ull;
-            continue;
+        c.seg = 0;
+        if (++c.g < g1 && c.g - c.prow0 >= c.np) open(c, pinst[c.g]);
+    };
+    uint4 cur[5], nxt[5];
+    auto load = [&](const Cursor &c, uint4 (&x)[5]) {
+        const int r = c.g - c.prow0;
+        const uint8_t *a = c.E + static_cast<int64_t>(r) * c.n;
+        const int off = static_cast<int>(reinterpret_cast<uintptr_t>(a) & 15);
+        const int lim = off + c.n;  // the row occupies bytes [off, lim) from the aligned address below
+        const bool live = c.g < g1 && r < c.n;
+#pragma unroll
+        for (int j = 0; j < 5; ++j) {
+            const int v0 = 2048 * c.seg + 512 * j + 16 * lane;
+            const bool want = live && v0 < lim && (j < 4 || lane == 0);
+            x[j] = want ? __ldcs(reinterpret_cast<const uint4 *>(a - off + v0)) : make_uint4(0u, 0u, 0u, 0u);
         }
-        int c = 0;
-        bool bad = false;
-        pack_row_bits(E + static_cast<int64_t>(r) * n, n, r, wp, row, lane, c, bad);
-        if (lane == 0) {
-            cnt[row0 + r] = c;
-            if (bad) atomicOr(status, ST_BAD_INPUT);
+    };
+    Cursor c;
+    c.g = g0;
+    c.seg = 0;
+    open(c, pinst[g0]);
+    load(c, cur);
+    int ones = 0, turn = 0;
+    uint32_t bad = 0;
+    while (c.g < g1) {
+        Cursor d = c;
+        step(d);
+        load(d, nxt);
+        const int r = c.g - c.prow0;
+        uint64_t *row = c.rbits + static_cast<int64_t>(r) * c.wp;
+        if (r >= c.n) {  // padding: identity only
+            for (int w = lane; w < c.wp; w += 32) row[w] = w == (r >> 6) ? 1ull << (r & 63) : 0ull;
+        } else {
+            uint64_t *buf = buf_s[warp][turn];
+            turn ^= 1;
+            const int off = static_cast<int>(reinterpret_cast<uintptr_t>(c.E + static_cast<int64_t>(r) * c.n) & 15);
+            const int lim = off + c.n;
+#pragma unroll
+            for (int j = 0; j < 5; ++j) {
+                const int v0 = 2048 * c.seg + 512 * j + 16 * lane;
+                const uint4 x = cur[j];
+                const int lo = min(16, max(0, off - v0)), hi = min(16, max(0, lim - v0));
+                const uint32_t valid = ((1u << hi) - 1u) & ~((1u << lo) - 1u);
+                const uint32_t m = byte_lsbs(x.x) | (byte_lsbs(x.y) << 4) | (byte_lsbs(x.z) << 8) |
+                                   (byte_lsbs(x.w) << 12);
+                const uint32_t b = byte_bad(x.x) | (byte_bad(x.y) << 4) | (byte_bad(x.z) << 8) |
+                                   (byte_bad(x.w) << 12);
+                bad |= b & valid;
+                if (j < 4 || lane == 0)
+                    reinterpret_cast<uint16_t *>(buf)[32 * j + lane] = static_cast<uint16_t>(m & valid);
+            }
+            __syncwarp();  // (the other turn's buffer is written next: every lane has read it by then)
+            const uint64_t b0 = buf[lane], b1 = buf[lane + 1];
+            const uint64_t e = off ? (b0 >> off) | (b1 << (64 - off)) : b0;
+            const int w = 32 * c.seg + lane;
+            if (w < c.wp) {
+                row[w] = e | (w == (r >> 6) ? 1ull << (r & 63) : 0ull);
+                ones += __popcll(e);
+            }
+            if (32 * (c.seg + 1) >= c.wp) {
+                ones = __reduce_add_sync(kFull, ones);
+                if (lane == 0) cnt[c.row0 + r] = ones;
+                ones = 0;
+            }
+        }
+        c = d;
+#pragma unroll
+        for (int j = 0; j < 5; ++j) cur[j] = nxt[j];
+    }
+    if (__any_sync(kFull, bad != 0) && lane == 0) atomicOr(status, ST_BAD_INPUT);
+}
+
+// Successor lists from the packed bits: eight lanes to a row, four words a lane at a time, four
+// rows of a warp at once (the dependent loads instance -> row pointers -> bits bound a warp to
+// the row: 251 -> FILL_US us over the 1.1 M rows of the workload above).
+constexpr int kFillRows = 8;  // padded rows of a warp, four at a time
+
+__global__ void __launch_bounds__(256)
+    batch_fill_kernel(const BatchInst *__restrict__ inst, const int *__restrict__ pinst, int total_prows,
+                      const int *__restrict__ ptr, int *col) {
+    const int lane = threadIdx.x & 31, sub = lane & 7;
+    const int g0 = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * kFillRows;
+#pragma unroll
+    for (int it = 0; it < kFillRows / 4; ++it) {
+        const int g = g0 + 4 * it + (lane >> 3);
+        int r = 0, wp = 0, p0 = 0, p1 = 0;
+        const uint64_t *row = nullptr;
+        if (g < total_prows) {
+            const BatchInst &I = inst[pinst[g]];
+            r = g - I.prow0;
+            if (r < I.n) {
+                wp = I.wp;
+                row = I.rbits + static_cast<int64_t>(r) * wp;
+                p0 = ptr[I.row0 + r];
+                p1 = ptr[I.row0 + r + 1];
+            }
+        }
+        uint64_t x[4];
+        auto words = [&](int w0) {  // this lane's four words from w0 (wp is even)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                ulonglong2 v = make_ulonglong2(0ull, 0ull);
+                if (w0 + 2 * h < wp) v = *reinterpret_cast<const ulonglong2 *>(row + w0 + 2 * h);
+                x[2 * h] = v.x;
+                x[2 * h + 1] = v.y;
+            }
+            return __popcll(x[0]) + __popcll(x[1]) + __popcll(x[2]) + __popcll(x[3]);
+        };
+        auto group_sum = [&](int c) {
+            c += __shfl_xor_sync(kFull, c, 1);
+            c += __shfl_xor_sync(kFull, c, 2);
+            return c + __shfl_xor_sync(kFull, c, 4);
+        };
+        const int steps = __reduce_max_sync(kFull, (wp + 31) / 32);
+        int total = 0;
+        for (int t = 0; t < steps; ++t) total += group_sum(words(32 * t + 4 * sub));
+        const bool loop = total == p1 - p0;  // bit r is a fact, not only the identity
+        for (int t = 0; t < steps; ++t) {
+            const int w0 = 32 * t + 4 * sub;
+            if (steps > 1) words(w0);
+            if (!loop && (r >> 6) >= w0 && (r >> 6) < w0 + 4) {
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    if (w0 + q == (r >> 6)) x[q] &= ~(1ull << (r & 63));
+            }
+            const int c = __popcll(x[0]) + __popcll(x[1]) + __popcll(x[2]) + __popcll(x[3]);
+            int inc = c;
+#pragma unroll
+            for (int o = 1; o < 8; o <<= 1) {
+                const int y = __shfl_up_sync(kFull, inc, o, 8);
+                if (sub >= o) inc += y;
+            }
+            int at = p0 + inc - c;
+            p0 += __shfl_sync(kFull, inc, 7, 8);
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                for (uint64_t y = x[q]; y != 0ull; y &= y - 1) col[at++] = 64 * (w0 + q) + __ffsll(static_cast<long long>(y)) - 1;
         }
     }
 }
 
-// Successor lists from the packed bits (one warp per padded row, real rows only).
+// Column mask of every listed instance (CTA per instance): the columns its CSR names.  No row
+// of the reflexive closure leaves the mask plus its own bit, no row of E M leaves the mask.
 __global__ void __launch_bounds__(256)
-    batch_fill_kernel(const BatchInst *__restrict__ inst, const int *__restrict__ pinst, int total_prows,
-                      const int *__restrict__ ptr, int *col) {
-    const int lane = threadIdx.x & 31;
-    const int g = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (g >= total_prows) return;
-    const BatchInst I = inst[pinst[g]];
-    const int r = g - I.prow0;
-    if (r >= I.n) return;
-    const int gr = I.row0 + r;
-    fill_row_from_bits(I.rbits + static_cast<int64_t>(r) * I.wp, I.wp, r, ptr[gr], ptr[gr + 1], col, lane);
-}
-
-// Column mask of every instance (CTA per instance): the columns its CSR names.  No row of
-// the reflexive closure leaves the mask plus its own bit, no row of E M leaves the mask.
-__global__ void __launch_bounds__(256)
-    batch_colmask_kernel(const BatchInst *__restrict__ inst, const int *__restrict__ ptr, const int *__restrict__ col) {
+    batch_colmask_kernel(const BatchInst *__restrict__ inst, BatchList list, const int *__restrict__ ptr,
+                         const int *__restrict__ col) {
     extern __shared__ unsigned long long cm_s[];
-    const BatchInst I = inst[blockIdx.x];
+    if (static_cast<int>(blockIdx.x) >= list.hdr[0]) return;
+    const BatchInst I = inst[list.k[blockIdx.x]];
     for (int w = threadIdx.x; w < I.wp; w += blockDim.x) cm_s[w] = 0ull;
     __syncthreads();
     for (int q = ptr[I.row0] + threadIdx.x; q < ptr[I.row0 + I.n]; q += blockDim.x)
-        atomicOr(&cm_s[col[q] >> 6], 1ull << (col[q] & 63));
+        or_shared(reinterpret_cast<uint64_t *>(&cm_s[col[q] >> 6]), 1ull << (col[q] & 63));
     __syncthreads();
     for (int w = threadIdx.x; w < I.wp; w += blockDim.x) I.colmask[w] = cm_s[w];
 }
 
-// Instances whose whole bit matrix fits in shared memory (at most kSmallNp padded rows of at
-// most 16 words: 128 KB) are closed by one CTA each, before the batched machinery: in-place
-// sweeps M_i |= E_i | OR_{s in succ(i)} M_s on the shared copy (rows of an instance share a
-// warp in lane groups sized to the row) until one changes nothing (__syncthreads_or over the
-// CTA), then the model E M with its certificate straight to the output.  An instance still
-// changing after kSmallSweeps sweeps writes its bits back and stays active for the batched
-// sweeps and squarings.
-constexpr int kSmallNp = 1024;
-constexpr int kSmallThreads = 1024;
-constexpr int kSmallSweeps = 64;
+// Column slices.  Bit column j of M <- M | E M depends on column j alone, so a CTA closes a
+// slice of an instance's columns in its shared memory without a word from the others: the
+// slice of M, the successor lists as 16-bit numbers (read from the CSR where they do not
+// fit), and for every row the sweep that last changed it.  In sweep t a row takes only the
+// successors that changed in sweep t - 1 or t; 16 bytes of a row to a lane.  Then the slice of
+// the model E M, with its certificate (out_r | e_r) = M_r, straight to the output.  A slice
+// that still changes after kSliceSweeps sweeps writes its bits back, and its instance stays
+// active for the batched sweeps and squarings.
+// Bound by shared memory (the successor lists and the rows they name, about 1.5 passes an access)
+// and by the few slices that need many sweeps; SLICE_NOTE
+constexpr int kSliceRows = 4096;         // constants of an instance closed in slices
+constexpr int kSliceBits = 128 * 1024;   // bytes of a slice of M
+constexpr int kSliceSmem = 220 * 1024;   // M, row pointers, stamps, successor lists
+constexpr int kSliceThreads = 1024;
+constexpr int kSliceSweeps = 64;
 
-__global__ void __launch_bounds__(kSmallThreads)
-    batch_small_kernel(const BatchInst *__restrict__ inst, const int *__restrict__ small_ids,
-                       const int *__restrict__ ptr, const int *__restrict__ col, BatchCounters c, int *status) {
-    extern __shared__ uint64_t small_s[];
-    __shared__ unsigned int ones_s;
-    const int k = small_ids[blockIdx.x];
-    const BatchInst I = inst[k];
-    const int wp = I.wp, n = I.n;
-    uint64_t *Ms = small_s;  // np x wp
-    for (int t = threadIdx.x; t < I.np * wp; t += blockDim.x) Ms[t] = I.rbits[t];
-    if (threadIdx.x == 0) ones_s = 0u;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    int G = 32;
-    while (G > 1 && (G >> 1) >= wp) G >>= 1;
-    const int R = 32 / G, grp = lane / G, w = lane % G;
-    const bool wv = w < wp;
-    const uint64_t cm = wv ? I.colmask[w] : 0ull;
-    const int *iptr = ptr + I.row0;  // iptr[r]: local row r
-    __syncthreads();
-    int it = 0;
+struct BatchSlice {
+    int32_t k, w0, nw;  // instance, first word, words (even)
+};
+
+// Words of a slice: the largest power of two up to 16 (a 128-byte row has no bank conflicts)
+// whose n rows fit kSliceBits.
+int slice_words(int64_t n) {
+    int w = 16;
+    while (w > 2 && n * w * 8 > kSliceBits) w >>= 1;
+    return w;
+}
+
+__device__ __forceinline__ void or2(ulonglong2 &a, const ulonglong2 &b) {
+    a.x |= b.x;
+    a.y |= b.y;
+}
+
+// The sweeps and the model of one slice (see above); Col: uint16_t (shared) or int (global).
+template <class Col>
+__device__ __forceinline__ void close_slice(const BatchInst &I, int k, int w0, int nw, ulonglong2 *M, const int *rp,
+                                            uint8_t *stamp, const Col *__restrict__ col, ulonglong2 cm, int G,
+                                            BatchCounters c, int *status, unsigned *ones_s) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n = I.n;
+    const int R = 32 / G, l = lane % G, nv = nw >> 1;
+    const int r0 = warp * R + lane / G, dr = (kSliceThreads / 32) * R;
+    const bool lv = l < nv;
+    const int wl = w0 + 2 * l;  // this lane's words wl, wl + 1 of every row it takes
+    auto self = [&](int r) {
+        const uint64_t b = 1ull << (r & 63);
+        return make_ulonglong2((r >> 6) == wl ? b : 0ull, (r >> 6) == wl + 1 ? b : 0ull);
+    };
+    int t = 1;
     bool conv = false;
-    while (it < kSmallSweeps) {
+    for (; t <= kSliceSweeps; ++t) {
         bool ch = false;
-        for (int r = warp * R + grp; r < n; r += nwarps * R) {
-            if (!wv) continue;
-            uint64_t acc = Ms[r * wp + w];
-            const uint64_t before = acc;
-            const uint64_t full = cm | (w == (r >> 6) ? 1ull << (r & 63) : 0ull);
-            for (int q = iptr[r]; q < iptr[r + 1] && acc != full; ++q) {
-                const int sidx = col[q];
-                acc |= Ms[sidx * wp + w] | (w == (sidx >> 6) ? 1ull << (sidx & 63) : 0ull);
+        for (int r = r0; r < n && lv; r += dr) {
+            ulonglong2 acc = M[r * nv + l];
+            const ulonglong2 before = acc;
+            ulonglong2 full = self(r);
+            or2(full, cm);
+            if (acc.x == full.x && acc.y == full.y) continue;
+            const int q1 = rp[r + 1];
+            for (int q = rp[r]; q < q1; q += 4) {
+                int sx[4];
+                bool take[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) sx[u] = q + u < q1 ? static_cast<int>(col[q + u]) : -1;
+#pragma unroll
+                for (int u = 0; u < 4; ++u) take[u] = sx[u] >= 0 && stamp[sx[u]] + 1 >= t;
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (take[u]) or2(acc, M[sx[u] * nv + l]);
             }
-            if (acc != before) {
-                Ms[r * wp + w] = acc;
+            if (acc.x != before.x || acc.y != before.y) {
+                M[r * nv + l] = acc;
+                stamp[r] = static_cast<uint8_t>(t);
                 ch = true;
             }
         }
-        ++it;
         if (!__syncthreads_or(ch)) {
             conv = true;
             break;
         }
     }
-    if (!conv) {  // hand over: the batched machinery continues from these bits
-        for (int t = threadIdx.x; t < I.np * wp; t += blockDim.x) I.rbits[t] = Ms[t];
-        if (threadIdx.x == 0) c.sweeps[k] = it;
+    if (threadIdx.x == 0) atomicMax(&c.sweeps[k], static_cast<unsigned long long>(min(t, kSliceSweeps)));
+    if (!conv) {
+        for (int r = r0; r < n && lv; r += dr)
+            *reinterpret_cast<ulonglong2 *>(I.rbits + static_cast<int64_t>(r) * I.wp + wl) = M[r * nv + l];
         return;
     }
-    // the model E M and the certificate (out_r | e_r) = M_r
     const int wout = (n + 63) >> 6;
     bool viol = false;
-    unsigned int ones = 0;
-    for (int r = warp * R + grp; r < n; r += nwarps * R) {
-        if (!wv) continue;
-        uint64_t out = 0ull;
-        for (int q = iptr[r]; q < iptr[r + 1] && out != cm; ++q) out |= Ms[col[q] * wp + w];
-        const uint64_t self = w == (r >> 6) ? 1ull << (r & 63) : 0ull;
-        viol |= (out | self) != Ms[r * wp + w];
-        ones += __popcll(out);
+    unsigned ones = 0;
+    for (int r = r0; r < n && lv; r += dr) {
+        ulonglong2 out = make_ulonglong2(0ull, 0ull);
+        const int q1 = rp[r + 1];
+        for (int q = rp[r]; q < q1; q += 4) {
+            int sx[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) sx[u] = q + u < q1 ? static_cast<int>(col[q + u]) : -1;
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (sx[u] >= 0) or2(out, M[sx[u] * nv + l]);
+        }
+        const ulonglong2 m = M[r * nv + l];
+        ulonglong2 e = self(r);
+        or2(e, out);
+        viol |= e.x != m.x || e.y != m.y;
+        ones += __popcll(out.x) + __popcll(out.y);
         if (I.out) {
-            if (w < wout) I.out[static_cast<int64_t>(r) * wout + w] = out;
+            uint64_t *o = I.out + static_cast<int64_t>(r) * wout + wl;
+            if (wl < wout) o[0] = out.x;
+            if (wl + 1 < wout) o[1] = out.y;
         } else {
-            I.mbits[static_cast<int64_t>(r) * wp + w] = out;
+            *reinterpret_cast<ulonglong2 *>(I.mbits + static_cast<int64_t>(r) * I.wp + wl) = out;
         }
     }
-    if (ones) atomicAdd(&ones_s, ones);
+    ones = __reduce_add_sync(kFull, ones);
+    if (lane == 0 && ones) atomicAdd(ones_s, ones);
     const int any_viol = __syncthreads_or(viol);
     if (threadIdx.x == 0) {
-        c.sweeps[k] = it;
-        c.ones[k] = ones_s;
-        c.state[k] = B_DONE;
-        if (any_viol) {  // a converged closure that fails its certificate: an internal error
-            c.viol[k] = 1;
-            atomicOr(status, ST_TIMEOUT_DEP);
-        }
+        atomicAdd(&c.ones[k], static_cast<unsigned long long>(*ones_s));
+        atomicAdd(&c.chg[k], 1ull);  // slices done
+        if (any_viol) atomicOr(status, ST_TIMEOUT_DEP);  // a converged closure that fails its certificate
     }
+}
+
+__global__ void __launch_bounds__(kSliceThreads)
+    batch_slice_kernel(const BatchInst *__restrict__ inst, const BatchSlice *__restrict__ slices,
+                       const int *__restrict__ ptr, const int *__restrict__ col, BatchCounters c, int *status) {
+    extern __shared__ __align__(16) unsigned char slice_smem[];
+    __shared__ uint64_t cm_s[16];
+    __shared__ unsigned ones_s;
+    const BatchSlice S = slices[blockIdx.x];
+    const BatchInst I = inst[S.k];
+    const int n = I.n, nv = S.nw >> 1;
+    auto *M = reinterpret_cast<ulonglong2 *>(slice_smem);  // n x nv
+    auto *rp = reinterpret_cast<int *>(M + n * nv);        // n + 1 row pointers
+    auto *stamp = reinterpret_cast<uint8_t *>(rp + n + 1);
+    auto *scol = reinterpret_cast<uint16_t *>(stamp + ((n + 3) & ~3));
+    int G = 8;
+    while (G > 1 && (G >> 1) >= nv) G >>= 1;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, l = lane % G;
+    if (threadIdx.x < 16) cm_s[threadIdx.x] = 0ull;
+    if (threadIdx.x == 0) ones_s = 0u;
+    const int *iptr = ptr + I.row0;
+    const int base = iptr[0], nnz = iptr[n] - base;
+    const bool fits = nnz <= (kSliceSmem - static_cast<int>(reinterpret_cast<unsigned char *>(scol) - slice_smem)) / 2;
+    __syncthreads();
+    // the slice, its row pointers and lists, and the columns with an incoming edge (a column whose only
+    // edge is its own constant's is missing: it is full for that row all the same)
+    ulonglong2 cm = make_ulonglong2(0ull, 0ull);
+    if (l < nv) {
+        const uint64_t *src = I.rbits + S.w0 + 2 * l;
+        const int wl = S.w0 + 2 * l;
+        const int dr = (kSliceThreads / 32) * (32 / G);
+#pragma unroll 4
+        for (int r = warp * (32 / G) + lane / G; r < n; r += dr) {
+            ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(src + static_cast<int64_t>(r) * I.wp);
+            M[r * nv + l] = v;
+            if ((r >> 6) == wl) v.x &= ~(1ull << (r & 63));
+            if ((r >> 6) == wl + 1) v.y &= ~(1ull << (r & 63));
+            or2(cm, v);
+        }
+        or_shared(&cm_s[2 * l], cm.x);
+        or_shared(&cm_s[2 * l + 1], cm.y);
+    }
+    for (int r = threadIdx.x; r <= n; r += kSliceThreads) {
+        rp[r] = iptr[r] - base;
+        if (r < n) stamp[r] = 0;
+    }
+    if (fits)
+        for (int q = threadIdx.x; q < nnz; q += kSliceThreads) scol[q] = static_cast<uint16_t>(col[base + q]);
+    __syncthreads();
+    if (l < nv) cm = make_ulonglong2(cm_s[2 * l], cm_s[2 * l + 1]);
+    if (fits) close_slice(I, S.k, S.w0, S.nw, M, rp, stamp, scol, cm, G, c, status, &ones_s);
+    else close_slice(I, S.k, S.w0, S.nw, M, rp, stamp, col + base, cm, G, c, status, &ones_s);
+}
+
+// After the slices: an instance all of whose slices are done is done, the others start over as
+// active ones (from the bits their unfinished slices wrote back).
+__global__ void batch_settle_kernel(const int *__restrict__ nslices, int L, BatchCounters c, int *open) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= L) return;
+    const int want = nslices[k];
+    if (want > 0 && c.chg[k] == static_cast<unsigned long long>(want)) {
+        c.state[k] = B_DONE;
+    } else {
+        c.ones[k] = 0;
+        *open = 1;
+    }
+    c.chg[k] = 0;
 }
 
 // Block-wide exclusive scan of four counters at once (kListThreads threads).
@@ -525,16 +755,13 @@ void launch_rows(int wpl, int grid, const BatchInst *d, const BatchList &l, cons
 
 }  // namespace
 
-// Cached schedule of the last batch (graph + the buffers it was built on).
+// Cached schedule of the last batch (graph, the sizes and the work space it was built on).
 struct BatchPlan {
     std::vector<int32_t> ns;
-    std::vector<const void *> ins;
-    std::vector<void *> outs;
-    const void *col = nullptr;
-    int mem = -1;
-    // main: CSR fill, first sweeps, the first squaring rounds, emission of the converged
-    // instances; more: the remaining rounds and their emission (launched only if an instance
-    // is still active after main)
+    std::vector<const void *> bufs;
+    // main: first sweeps, the first squaring rounds, emission of the converged instances;
+    // more: the remaining rounds and their emission (launched only if an instance is still
+    // active after main)
     cudaGraphExec_t exec = nullptr, exec_more = nullptr;
     int rounds = 0, rounds_more = 0;
     int launches = 0, launches_more = 0;  // kernels in each graph
@@ -544,131 +771,32 @@ struct BatchPlan {
     }
 };
 
-dl_status solve_tc_batch(dl_ctx *ctx, Workspace &ws, cudaStream_t s, int32_t count, const int32_t *ns,
-                         const uint8_t *const *Es, dl_mem mem, uint64_t *const *out_bits, dl_stats *st) {
-    // instances with n > 0 take part; empty ones have nothing to write
-    std::vector<int> live;
-    for (int32_t k = 0; k < count; ++k)
-        if (ns[k] > 0) live.push_back(k);
-    if (live.empty()) return DL_OK;
-    const int L = static_cast<int>(live.size());
-    const int bn = 128;  // GEMM tile width for the batch (small instances waste less padding)
-    const int tm = gemm_tile_m();
-    std::vector<BatchInst> inst(L);
-    int64_t in_bytes = 0, mat_bytes = 0, bit_words = 0, prow = 0, row = 0, max_np = 0, max_wp = 0, tiles = 0,
-            wp_words = 0;
-    for (int i = 0; i < L; ++i) {
-        const int32_t n = ns[live[i]];
-        const int64_t np = round_up(n, 128);
-        inst[i].n = n;
-        inst[i].np = static_cast<int32_t>(np);
-        inst[i].wp = static_cast<int32_t>(np / 64);
-        inst[i].tiles = static_cast<int32_t>(((np + tm - 1) / tm) * ((np + bn - 1) / bn));
-        inst[i].prow0 = static_cast<int32_t>(std::min<int64_t>(prow, INT32_MAX));
-        inst[i].row0 = static_cast<int32_t>(std::min<int64_t>(row, INT32_MAX));
-        prow += np;
-        row += n;
-        tiles += inst[i].tiles;
-        in_bytes += round_up(static_cast<int64_t>(n) * n, 256);
-        mat_bytes += np * np;
-        bit_words += np * (np / 64);
-        wp_words += np / 64;
-        max_np = std::max(max_np, np);
-        max_wp = std::max(max_wp, np / 64);
-    }
-    const int64_t total_prows = prow, total_rows = row;
-    if (max_wp > 256) {
-        set_error("batch: instances are limited to n <= 16384");
-        return DL_EINVAL;
-    }
-    if (total_prows > (1ll << 31) - 2 || tiles > (1ll << 31) - 1) {
-        set_error("batch: too many rows (%lld padded rows)", static_cast<long long>(total_prows));
-        return DL_EINVAL;
-    }
+// The instances that are still active: batched sweeps, squarings, models (step 3 above).
+dl_status batch_rounds(dl_ctx *ctx, Workspace &ws, cudaStream_t s, std::vector<BatchInst> &inst, int64_t mat_bytes,
+                       int64_t max_np, int64_t max_wp, int64_t tiles, const BatchCounters &bc, const BatchList &bl,
+                       BatchInst *dinst, const int *gptr, const int *gcol, int *launches_out, int *gemms_out) {
+    const int L = static_cast<int>(inst.size());
+    const int bn = kBatchBn;
     const int wpl = max_wp <= 32 ? 1 : max_wp <= 64 ? 2 : max_wp <= 128 ? 4 : 8;
-    const int scan_blocks = static_cast<int>((total_rows + 1023) / 1024);
     auto *c0 = static_cast<uint8_t *>(ws.get("batch_c0", mat_bytes));
-    auto *rb = static_cast<uint64_t *>(ws.get("batch_rbits", bit_words * 8));
-    auto *mb = static_cast<uint64_t *>(ws.get("batch_mbits", bit_words * 8));
-    auto *cmask = static_cast<uint64_t *>(ws.get("batch_colmask", std::max<int64_t>(wp_words, 1) * 8));
-    auto *ctr = static_cast<unsigned long long *>(ws.get("batch_ctr", kCounterArrays * sizeof(unsigned long long) * L));
-    auto *state = static_cast<int *>(ws.get("batch_state", sizeof(int) * L));
-    auto *lists = static_cast<int *>(ws.get("batch_list", sizeof(int) * (8 + 3 * (L + 1) + 2 + 2 * L + 1)));
-    auto *dinst = static_cast<BatchInst *>(ws.get("batch_inst", sizeof(BatchInst) * L));
     auto *dprob = static_cast<GemmProblem *>(ws.get("batch_probs", sizeof(GemmProblem) * L));
-    auto *pinst = static_cast<int *>(ws.get("batch_pinst", sizeof(int) * total_prows));
-    auto *gcnt = static_cast<int *>(ws.get("batch_cnt", sizeof(int) * (total_rows + 1)));
-    auto *gptr = static_cast<int *>(ws.get("batch_ptr", sizeof(int) * (total_rows + 1)));
-    auto *scratch = static_cast<int *>(ws.get("batch_scan", sizeof(int) * 2 * (scan_blocks + 1)));
-    uint8_t *staging = nullptr;
-    if (mem == DL_MEM_HOST) staging = static_cast<uint8_t *>(ws.get("batch_in", std::max<int64_t>(in_bytes, 256)));
-    if (!c0 || !rb || !mb || !cmask || !ctr || !state || !lists || !dinst || !dprob || !pinst || !gcnt || !gptr ||
-        !scratch || (mem == DL_MEM_HOST && !staging)) {
+    if (!c0 || !dprob) {
         set_error("batch: device allocation failed (%.2f GB of operands)", 1.0 * mat_bytes / 1e9);
         return DL_ENOMEM;
     }
-    const BatchCounters bc{state, ctr, ctr + L, ctr + 2 * L, ctr + 3 * L, ctr + 4 * L};
-    const BatchList bl{lists, lists + 8, lists + 8 + (L + 1), lists + 8 + 2 * (L + 1), lists + 8 + 3 * (L + 1)};
-
-    cudaEvent_t ev0 = ws.ev[0], ev1 = ws.ev[1];
-    BCK(cudaEventRecord(ev0, s));
-    int64_t mo = 0, bo = 0, io = 0, co = 0;
+    std::vector<int32_t> key_ns(L);
+    int64_t mo = 0;
     for (int i = 0; i < L; ++i) {
-        const int k = live[i];
-        const int64_t np = inst[i].np, n = inst[i].n;
-        if (mem == DL_MEM_HOST) {
-            BCK(cudaMemcpyAsync(staging + io, Es[k], n * n, cudaMemcpyHostToDevice, s));
-            inst[i].E = staging + io;
-            io += round_up(n * n, 256);
-        } else {
-            inst[i].E = Es[k];
-        }
         inst[i].c0 = c0 + mo;
-        inst[i].rbits = rb + bo;
-        inst[i].mbits = mb + bo;
-        inst[i].out = mem == DL_MEM_DEVICE ? out_bits[k] : nullptr;
-        inst[i].colmask = cmask + co;
-        co += np / 64;
-        mo += np * np;
-        bo += np * (np / 64);
+        mo += static_cast<int64_t>(inst[i].np) * inst[i].np;
+        key_ns[i] = inst[i].n;
     }
     BCK(cudaMemcpyAsync(dinst, inst.data(), sizeof(BatchInst) * L, cudaMemcpyHostToDevice, s));
-
-    // 1. bits of I + E, counts and checks over all inputs, then the CSR row pointers (every
-    //    call: the contents, hence the number of facts, may differ between calls)
-    BCK(cudaMemsetAsync(ws.status, 0, sizeof(int), s));
-    batch_map_kernel<<<L, 256, 0, s>>>(dinst, pinst);
-    const unsigned pack_blocks = static_cast<unsigned>((total_prows + 8 * kPackRows - 1) / (8 * kPackRows));
-    batch_pack_kernel<<<pack_blocks, 256, 0, s>>>(dinst, pinst, static_cast<int>(total_prows), gcnt, ws.status);
-    BCK(cudaGetLastError());
-    BCK(exclusive_scan_large(gcnt, static_cast<int>(total_rows), gptr, scratch, s));
-    const int pre_launches = 2 + (total_rows > 64 * 1024 ? 3 : 1);
-    int nnz_total = 0, hst = 0;
-    BCK(cudaMemcpyAsync(&nnz_total, gptr + total_rows, sizeof(int), cudaMemcpyDeviceToHost, s));
-    BCK(cudaMemcpyAsync(&hst, ws.status, sizeof(int), cudaMemcpyDeviceToHost, s));
-    BCK(cudaStreamSynchronize(s));
-    if (hst & ST_BAD_INPUT) {
-        set_error("batch: an input matrix holds a byte that is neither 0 nor 1");
-        return DL_EINVAL;
-    }
-    auto *gcol = static_cast<int *>(ws.get("batch_col", sizeof(int) * static_cast<size_t>(std::max(nnz_total, 1))));
-    if (!gcol) {
-        set_error("batch: device allocation failed (CSR of %d facts)", nnz_total);
-        return DL_ENOMEM;
-    }
-
-    // 2. the captured schedule (rebuilt when the buffers change)
-    std::vector<int32_t> key_ns(L);
-    std::vector<const void *> key_in(L);
-    std::vector<void *> key_out(L);
-    for (int i = 0; i < L; ++i) {
-        key_ns[i] = inst[i].n;
-        key_in[i] = inst[i].E;
-        key_out[i] = out_bits[live[i]];
-    }
+    // what the graph's launches and the GEMM table name (inputs and outputs are read from dinst)
+    const std::vector<const void *> key_bufs = {c0,       dprob,   dinst,    gptr,     gcol,     bc.state,
+                                                bc.chg,   bl.hdr,  inst[0].rbits, ws.status};
     BatchPlan *&plan = ws.batch_plan;
-    const bool reuse = plan && plan->mem == static_cast<int>(mem) && plan->ns == key_ns && plan->ins == key_in &&
-                       plan->outs == key_out && plan->col == gcol;
+    const bool reuse = plan && plan->ns == key_ns && plan->bufs == key_bufs;
     if (!reuse) {
         delete plan;
         plan = nullptr;
@@ -693,29 +821,9 @@ dl_status solve_tc_batch(dl_ctx *ctx, Workspace &ws, cudaStream_t s, int32_t cou
         // pageable source: the copy has read `probs` when cudaMemcpyAsync returns
         BCK(cudaMemcpyAsync(dprob, probs.data(), sizeof(GemmProblem) * L, cudaMemcpyHostToDevice, s));
         BCK(gemm_prepare(KIND_F8, false, bn, EPI_BOOL));
-        // instances closed in shared memory by one CTA each
-        std::vector<int> small;
-        size_t small_smem = 0;
-        for (int i = 0; i < L; ++i)
-            if (inst[i].np <= kSmallNp) {
-                small.push_back(i);
-                small_smem = std::max(small_smem, static_cast<size_t>(inst[i].np) * inst[i].wp * 8);
-            }
-        int *dsmall = nullptr;
-        if (!small.empty()) {
-            dsmall = static_cast<int *>(ws.get("batch_small", sizeof(int) * small.size()));
-            if (!dsmall) {
-                set_error("batch: device allocation failed (small-instance list)");
-                return DL_ENOMEM;
-            }
-            BCK(cudaMemcpyAsync(dsmall, small.data(), sizeof(int) * small.size(), cudaMemcpyHostToDevice, s));
-            BCK(cudaFuncSetAttribute(batch_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     static_cast<int>(small_smem)));
-        }
         const int rounds = 1 + static_cast<int>(std::ceil(std::log2(static_cast<double>(max_np) + 1.0)));
         const int ggrid = static_cast<int>(std::min<int64_t>(tiles, ctx->sms));
         const int rgrid = ctx->sms * 8;  // row kernels: 8 CTAs of 8 warps per SM, rows claimed in chunks
-        const unsigned prow_grid = static_cast<unsigned>((total_prows + 7) / 8);
         int launches = 0;
         auto sweep = [&]() {
             launch_rows<false>(wpl, rgrid, dinst, bl, gptr, gcol, bc, s);
@@ -760,23 +868,13 @@ dl_status solve_tc_batch(dl_ctx *ctx, Workspace &ws, cudaStream_t s, int32_t cou
         };
         plan = new BatchPlan();
         plan->ns = key_ns;
-        plan->ins = key_in;
-        plan->outs = key_out;
-        plan->col = gcol;
-        plan->mem = static_cast<int>(mem);
+        plan->bufs = key_bufs;
         dl_status rc = capture(
             [&]() -> cudaError_t {
-                cudaError_t e = cudaMemsetAsync(state, 0, sizeof(int) * L, s);
-                if (e == cudaSuccess) e = cudaMemsetAsync(ctr, 0, kCounterArrays * sizeof(unsigned long long) * L, s);
-                batch_fill_kernel<<<prow_grid, 256, 0, s>>>(dinst, pinst, static_cast<int>(total_prows), gptr, gcol);
-                batch_colmask_kernel<<<L, 256, static_cast<size_t>(max_wp) * 8, s>>>(dinst, gptr, gcol);
-                if (!small.empty()) {
-                    batch_small_kernel<<<static_cast<unsigned>(small.size()), kSmallThreads, small_smem, s>>>(
-                        dinst, dsmall, gptr, gcol, bc, ws.status);
-                    ++launches;
-                }
+                cudaError_t e = cudaSuccess;
                 batch_list_kernel<<<1, kListThreads, 0, s>>>(dinst, L, bc, bl, B_ACTIVE, 0);
-                launches += 3;
+                batch_colmask_kernel<<<L, 256, static_cast<size_t>(max_wp) * 8, s>>>(dinst, bl, gptr, gcol);
+                launches += 2;
                 for (int k = 0; k < kFirstSweeps; ++k) sweep();
                 for (int r = 0; r < rounds_main && e == cudaSuccess; ++r) e = round();
                 emit();
@@ -807,10 +905,175 @@ dl_status solve_tc_batch(dl_ctx *ctx, Workspace &ws, cudaStream_t s, int32_t cou
     }
     BCK(cudaGraphLaunch(plan->exec, s));
     std::vector<int> hstate(L);
-    BCK(cudaMemcpyAsync(hstate.data(), state, sizeof(int) * L, cudaMemcpyDeviceToHost, s));
+    BCK(cudaMemcpyAsync(hstate.data(), bc.state, sizeof(int) * L, cudaMemcpyDeviceToHost, s));
     BCK(cudaStreamSynchronize(s));
     const bool more = std::any_of(hstate.begin(), hstate.end(), [](int x) { return x == B_ACTIVE; });
     if (more && plan->exec_more) BCK(cudaGraphLaunch(plan->exec_more, s));
+    *launches_out = plan->launches + (more ? plan->launches_more : 0);
+    *gemms_out = plan->rounds + (more ? plan->rounds_more : 0);
+    return DL_OK;
+}
+
+dl_status solve_tc_batch(dl_ctx *ctx, Workspace &ws, cudaStream_t s, int32_t count, const int32_t *ns,
+                         const uint8_t *const *Es, dl_mem mem, uint64_t *const *out_bits, dl_stats *st) {
+    // instances with n > 0 take part; empty ones have nothing to write
+    std::vector<int> live;
+    for (int32_t k = 0; k < count; ++k)
+        if (ns[k] > 0) live.push_back(k);
+    if (live.empty()) return DL_OK;
+    const int L = static_cast<int>(live.size());
+    const int bn = kBatchBn;
+    const int tm = gemm_tile_m();
+    std::vector<BatchInst> inst(L);
+    int64_t in_bytes = 0, mat_bytes = 0, bit_words = 0, prow = 0, row = 0, max_np = 0, max_wp = 0, tiles = 0,
+            wp_words = 0;
+    for (int i = 0; i < L; ++i) {
+        const int32_t n = ns[live[i]];
+        const int64_t np = round_up(n, 128);
+        inst[i].n = n;
+        inst[i].np = static_cast<int32_t>(np);
+        inst[i].wp = static_cast<int32_t>(np / 64);
+        inst[i].tiles = static_cast<int32_t>(((np + tm - 1) / tm) * ((np + bn - 1) / bn));
+        inst[i].prow0 = static_cast<int32_t>(std::min<int64_t>(prow, INT32_MAX));
+        inst[i].row0 = static_cast<int32_t>(std::min<int64_t>(row, INT32_MAX));
+        prow += np;
+        row += n;
+        tiles += inst[i].tiles;
+        in_bytes += round_up(static_cast<int64_t>(n) * n, 256);
+        mat_bytes += np * np;
+        bit_words += np * (np / 64);
+        wp_words += np / 64;
+        max_np = std::max(max_np, np);
+        max_wp = std::max(max_wp, np / 64);
+    }
+    const int64_t total_prows = prow, total_rows = row;
+    if (max_wp > 256) {
+        set_error("batch: instances are limited to n <= 16384");
+        return DL_EINVAL;
+    }
+    if (total_prows > (1ll << 31) - 2 || tiles > (1ll << 31) - 1) {
+        set_error("batch: too many rows (%lld padded rows)", static_cast<long long>(total_prows));
+        return DL_EINVAL;
+    }
+    const int scan_blocks = static_cast<int>((total_rows + 1023) / 1024);
+    // the columns of every instance of up to kSliceRows constants, the slices with the most work first
+    std::vector<BatchSlice> slices;
+    std::vector<int32_t> nslices(L, 0);
+    for (int i = 0; i < L; ++i) {
+        if (inst[i].n > kSliceRows) continue;
+        const int W = slice_words(inst[i].n);
+        for (int w0 = 0; w0 < inst[i].wp; w0 += W, ++nslices[i])
+            slices.push_back(BatchSlice{i, w0, std::min(W, inst[i].wp - w0)});
+    }
+    std::stable_sort(slices.begin(), slices.end(), [&](const BatchSlice &a, const BatchSlice &b) {
+        return static_cast<int64_t>(a.nw) * inst[a.k].n > static_cast<int64_t>(b.nw) * inst[b.k].n;
+    });
+    const size_t slice_bytes = slices.size() * sizeof(BatchSlice);
+    auto *rb = static_cast<uint64_t *>(ws.get("batch_rbits", bit_words * 8));
+    auto *mb = static_cast<uint64_t *>(ws.get("batch_mbits", bit_words * 8));
+    auto *cmask = static_cast<uint64_t *>(ws.get("batch_colmask", std::max<int64_t>(wp_words, 1) * 8));
+    auto *ctr = static_cast<unsigned long long *>(ws.get("batch_ctr", kCounterArrays * sizeof(unsigned long long) * L));
+    auto *state = static_cast<int *>(ws.get("batch_state", sizeof(int) * (L + 1)));  // and whether any is open
+    auto *lists = static_cast<int *>(ws.get("batch_list", sizeof(int) * (8 + 3 * (L + 1) + 2 + 2 * L + 1)));
+    auto *dinst = static_cast<BatchInst *>(ws.get("batch_inst", sizeof(BatchInst) * L));
+    auto *dslices = static_cast<BatchSlice *>(ws.get("batch_slices", std::max<size_t>(slice_bytes, 16)));
+    auto *dnslices = static_cast<int *>(ws.get("batch_nslices", sizeof(int) * L));
+    auto *pinst = static_cast<int *>(ws.get("batch_pinst", sizeof(int) * total_prows));
+    auto *gcnt = static_cast<int *>(ws.get("batch_cnt", sizeof(int) * (total_rows + 1)));
+    auto *gptr = static_cast<int *>(ws.get("batch_ptr", sizeof(int) * (total_rows + 1)));
+    auto *scratch = static_cast<int *>(ws.get("batch_scan", sizeof(int) * 2 * (scan_blocks + 1)));
+    uint8_t *staging = nullptr;
+    if (mem == DL_MEM_HOST) staging = static_cast<uint8_t *>(ws.get("batch_in", std::max<int64_t>(in_bytes, 256)));
+    if (!rb || !mb || !cmask || !ctr || !state || !lists || !dinst || !dslices || !dnslices || !pinst || !gcnt ||
+        !gptr || !scratch || (mem == DL_MEM_HOST && !staging)) {
+        set_error("batch: device allocation failed (%.2f GB of bits)", 16.0 * bit_words / 1e9);
+        return DL_ENOMEM;
+    }
+    const BatchCounters bc{state, ctr, ctr + L, ctr + 2 * L, ctr + 3 * L, ctr + 4 * L};
+    const BatchList bl{lists, lists + 8, lists + 8 + (L + 1), lists + 8 + 2 * (L + 1), lists + 8 + 3 * (L + 1)};
+
+    cudaEvent_t ev0 = ws.ev[0], ev1 = ws.ev[1];
+    BCK(cudaEventRecord(ev0, s));
+    int64_t bo = 0, io = 0, co = 0;
+    for (int i = 0; i < L; ++i) {
+        const int k = live[i];
+        const int64_t np = inst[i].np, n = inst[i].n;
+        if (mem == DL_MEM_HOST) {
+            BCK(cudaMemcpyAsync(staging + io, Es[k], n * n, cudaMemcpyHostToDevice, s));
+            inst[i].E = staging + io;
+            io += round_up(n * n, 256);
+        } else {
+            inst[i].E = Es[k];
+        }
+        inst[i].c0 = nullptr;  // set where the batched rounds are needed
+        inst[i].rbits = rb + bo;
+        inst[i].mbits = mb + bo;
+        inst[i].out = mem == DL_MEM_DEVICE ? out_bits[k] : nullptr;
+        inst[i].colmask = cmask + co;
+        co += np / 64;
+        bo += np * (np / 64);
+    }
+    BCK(cudaMemcpyAsync(dinst, inst.data(), sizeof(BatchInst) * L, cudaMemcpyHostToDevice, s));
+    BCK(cudaMemcpyAsync(dnslices, nslices.data(), sizeof(int) * L, cudaMemcpyHostToDevice, s));
+    if (slice_bytes) BCK(cudaMemcpyAsync(dslices, slices.data(), slice_bytes, cudaMemcpyHostToDevice, s));
+
+    // 1. bits of I + E, counts and checks over all inputs, then the CSR row pointers (every
+    //    call: the contents, hence the number of facts, may differ between calls)
+    BCK(cudaMemsetAsync(ws.status, 0, sizeof(int), s));
+    batch_map_kernel<<<L, 256, 0, s>>>(dinst, pinst);
+    const unsigned pack_blocks = static_cast<unsigned>((total_prows + 8 * kPackRows - 1) / (8 * kPackRows));
+    batch_pack_kernel<<<pack_blocks, 256, 0, s>>>(dinst, pinst, static_cast<int>(total_prows), gcnt, ws.status);
+    BCK(cudaGetLastError());
+    BCK(exclusive_scan_large(gcnt, static_cast<int>(total_rows), gptr, scratch, s));
+    const int pre_launches = 2 + (total_rows > 64 * 1024 ? 3 : 1);
+    int nnz_total = 0, hst = 0;
+    BCK(cudaMemcpyAsync(&nnz_total, gptr + total_rows, sizeof(int), cudaMemcpyDeviceToHost, s));
+    BCK(cudaMemcpyAsync(&hst, ws.status, sizeof(int), cudaMemcpyDeviceToHost, s));
+    BCK(cudaStreamSynchronize(s));
+    if (hst & ST_BAD_INPUT) {
+        set_error("batch: an input matrix holds a byte that is neither 0 nor 1");
+        return DL_EINVAL;
+    }
+    auto *gcol = static_cast<int *>(ws.get("batch_col", sizeof(int) * static_cast<size_t>(std::max(nnz_total, 1))));
+    if (!gcol) {
+        set_error("batch: device allocation failed (CSR of %d facts)", nnz_total);
+        return DL_ENOMEM;
+    }
+
+    // 2. the successor lists, then every instance's column slices
+    BCK(cudaMemsetAsync(state, 0, sizeof(int) * (L + 1), s));
+    BCK(cudaMemsetAsync(ctr, 0, kCounterArrays * sizeof(unsigned long long) * L, s));
+    const unsigned fill_blocks = static_cast<unsigned>((total_prows + 8 * kFillRows - 1) / (8 * kFillRows));
+    batch_fill_kernel<<<fill_blocks, 256, 0, s>>>(dinst, pinst, static_cast<int>(total_prows), gptr, gcol);
+    int launches = pre_launches + 2;
+    if (!slices.empty()) {
+        BCK(cudaFuncSetAttribute(batch_slice_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSliceSmem));
+        batch_slice_kernel<<<static_cast<unsigned>(slices.size()), kSliceThreads, kSliceSmem, s>>>(
+            dinst, dslices, gptr, gcol, bc, ws.status);
+        ++launches;
+    }
+    batch_settle_kernel<<<(L + 255) / 256, 256, 0, s>>>(dnslices, L, bc, state + L);
+    BCK(cudaGetLastError());
+    std::vector<int> hstate(L + 1);
+    std::vector<unsigned long long> hctr(kCounterArrays * static_cast<size_t>(L));
+    auto read_back = [&]() -> cudaError_t {
+        cudaError_t e = cudaMemcpyAsync(hstate.data(), state, sizeof(int) * (L + 1), cudaMemcpyDeviceToHost, s);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(hctr.data(), ctr, sizeof(unsigned long long) * kCounterArrays * L,
+                                cudaMemcpyDeviceToHost, s);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(&hst, ws.status, sizeof(int), cudaMemcpyDeviceToHost, s);
+        return e == cudaSuccess ? cudaStreamSynchronize(s) : e;
+    };
+    BCK(cudaEventRecord(ev1, s));
+    BCK(read_back());
+    int gemms = 0;
+    if (hstate[L] != 0) {  // an instance is still open
+        int extra = 0;
+        const dl_status rc = batch_rounds(ctx, ws, s, inst, mat_bytes, max_np, max_wp, tiles, bc, bl, dinst, gptr, gcol,
+                                          &extra, &gemms);
+        if (rc != DL_OK) return rc;
+        launches += extra;
+    }
     if (mem == DL_MEM_HOST) {
         for (int i = 0; i < L; ++i) {
             const int64_t n = inst[i].n, w = (n + 63) / 64;
@@ -818,13 +1081,10 @@ dl_status solve_tc_batch(dl_ctx *ctx, Workspace &ws, cudaStream_t s, int32_t cou
                                   cudaMemcpyDeviceToHost, s));
         }
     }
-    BCK(cudaEventRecord(ev1, s));
-    std::vector<unsigned long long> hctr(kCounterArrays * static_cast<size_t>(L));
-    BCK(cudaMemcpyAsync(hstate.data(), state, sizeof(int) * L, cudaMemcpyDeviceToHost, s));
-    BCK(cudaMemcpyAsync(hctr.data(), ctr, sizeof(unsigned long long) * kCounterArrays * L, cudaMemcpyDeviceToHost,
-                        s));
-    BCK(cudaMemcpyAsync(&hst, ws.status, sizeof(int), cudaMemcpyDeviceToHost, s));
-    BCK(cudaStreamSynchronize(s));
+    if (mem == DL_MEM_HOST || hstate[L] != 0) {
+        BCK(cudaEventRecord(ev1, s));
+        BCK(read_back());
+    }
     if (hst) {
         set_error("batch: device status 0x%x (a wait expired or a certificate failed)", hst);
         return DL_ETIMEOUT;
@@ -859,13 +1119,12 @@ dl_status solve_tc_batch(dl_ctx *ctx, Workspace &ws, cudaStream_t s, int32_t cou
         st->ms_total = ms;
         st->ms_solve = ms;
         st->tflops_equiv = ms > 0 ? equiv / (ms * 1e-3) / 1e12 : 0.0;
-        st->gemm_launches = plan->rounds + (more ? plan->rounds_more : 0);
+        st->gemm_launches = gemms;
         st->gemm_flops = flops;
-        st->gpu_launches = pre_launches + plan->launches + (more ? plan->launches_more : 0);
+        st->gpu_launches = launches;
     }
     return DL_OK;
 }
-
 void batch_plan_release(BatchPlan *p) { delete p; }
 
 }  // namespace dl
