@@ -55,6 +55,7 @@ struct BatchInst {
     int32_t tiles;  // GEMM tiles of the squaring
     int32_t prow0;  // first padded row in the order of all instances
     int32_t row0;   // first real row in the order of all instances
+    int32_t tile0;  // first tile of rows of the packing, in the order of all instances
 };
 
 // Per-instance counters (arrays of `count` entries) and the active-instance counter.
@@ -84,122 +85,39 @@ __device__ __forceinline__ int last_le(const int *pre, int count, int x) {  // l
     return lo;
 }
 
-// Padded row -> instance, rebuilt every call (one CTA per instance).
-__global__ void batch_map_kernel(const BatchInst *__restrict__ inst, int *pinst) {
+// Padded row -> instance and tile of rows -> instance, rebuilt every call (one CTA per instance).
+__global__ void batch_map_kernel(const BatchInst *__restrict__ inst, int *pinst, int *tinst) {
     const BatchInst I = inst[blockIdx.x];
+    const int R = tile_rows(I.n), nt = (I.np + R - 1) / R;
     for (int r = threadIdx.x; r < I.np; r += blockDim.x) pinst[I.prow0 + r] = blockIdx.x;
+    for (int t = threadIdx.x; t < nt; t += blockDim.x) tinst[I.tile0 + t] = blockIdx.x;
 }
 
-// Bits of row r of I + E_k into M, the row's successor count and the 0/1 check.  A warp takes
-// kPackRows consecutive padded rows, 32 words of a row at a time: 16 bytes a lane, four
-// coalesced 512-byte loads (and the 16-byte block behind them where the row starts off a
-// 16-byte boundary), those of the next step in flight while this one's are packed.  The 16-bit
-// pieces meet in shared memory, where word w is read at its bit offset.  Bound by the read of
-// the bytes: 1024 instances of 33..2044 constants, 1.43 GB, 547 -> PACK_US us (PACK_TB TB/s; each
-// lane loading its own word's 64 bytes, and a row's loads only after the row before was
-// packed, left both the L1 lines and the memory idle half of the time).
-constexpr int kPackRows = 8;
-constexpr int kPackBuf = 36;  // 64-bit words of a step's bits: 2064 bits and the word behind
-
+// Bits of I + E_k into M, successor counts and the 0/1 check: a CTA per tile of rows of one instance
+// (pack_tile).  Bound by the read of the bytes: 1024 instances of 33..2044 constants, 1.43 GB,
+// 547 -> PACK_US us.
 __global__ void __launch_bounds__(256, 4)
-    batch_pack_kernel(const BatchInst *__restrict__ inst, const int *__restrict__ pinst, int total_prows,
-                      int *cnt, int *status) {
-    __shared__ uint64_t buf_s[8][2][kPackBuf];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int g0 = (blockIdx.x * (blockDim.x >> 5) + warp) * kPackRows;
-    if (g0 >= total_prows) return;
-    const int g1 = min(g0 + kPackRows, total_prows);
-    if (lane < 2 * (kPackBuf - 32)) buf_s[warp][lane & 1][32 + (lane >> 1)] = 0ull;  // never written beyond 16 bits
-    __syncwarp();
-    struct Cursor {  // a step: the words [32 seg, 32 seg + 32) of padded row g
-        const uint8_t *E;
-        uint64_t *rbits;
-        int g, seg, n, np, wp, prow0, row0;
-    };
-    auto open = [&](Cursor &c, int k) {
-        c.E = inst[k].E;
-        c.rbits = inst[k].rbits;
-        c.n = inst[k].n;
-        c.np = inst[k].np;
-        c.wp = inst[k].wp;
-        c.prow0 = inst[k].prow0;
-        c.row0 = inst[k].row0;
-    };
-    auto step = [&](Cursor &c) {
-        if (c.g - c.prow0 < c.n && 32 * (c.seg + 1) < c.wp) {
-            ++c.seg;
-            return;
-        }
-        c.seg = 0;
-        if (++c.g < g1 && c.g - c.prow0 >= c.np) open(c, pinst[c.g]);
-    };
-    uint4 cur[5], nxt[5];
-    auto load = [&](const Cursor &c, uint4 (&x)[5]) {
-        const int r = c.g - c.prow0;
-        const uint8_t *a = c.E + static_cast<int64_t>(r) * c.n;
-        const int off = static_cast<int>(reinterpret_cast<uintptr_t>(a) & 15);
-        const int lim = off + c.n;  // the row occupies bytes [off, lim) from the aligned address below
-        const bool live = c.g < g1 && r < c.n;
-#pragma unroll
-        for (int j = 0; j < 5; ++j) {
-            const int v0 = 2048 * c.seg + 512 * j + 16 * lane;
-            const bool want = live && v0 < lim && (j < 4 || lane == 0);
-            x[j] = want ? __ldcs(reinterpret_cast<const uint4 *>(a - off + v0)) : make_uint4(0u, 0u, 0u, 0u);
-        }
-    };
-    Cursor c;
-    c.g = g0;
-    c.seg = 0;
-    open(c, pinst[g0]);
-    load(c, cur);
-    int ones = 0, turn = 0;
-    uint32_t bad = 0;
-    while (c.g < g1) {
-        Cursor d = c;
-        step(d);
-        load(d, nxt);
-        const int r = c.g - c.prow0;
-        uint64_t *row = c.rbits + static_cast<int64_t>(r) * c.wp;
-        if (r >= c.n) {  // padding: identity only
-            for (int w = lane; w < c.wp; w += 32) row[w] = w == (r >> 6) ? 1ull << (r & 63) : 0ull;
-        } else {
-            uint64_t *buf = buf_s[warp][turn];
-            turn ^= 1;
-            const int off = static_cast<int>(reinterpret_cast<uintptr_t>(c.E + static_cast<int64_t>(r) * c.n) & 15);
-            const int lim = off + c.n;
-#pragma unroll
-            for (int j = 0; j < 5; ++j) {
-                const int v0 = 2048 * c.seg + 512 * j + 16 * lane;
-                const uint4 x = cur[j];
-                const int lo = min(16, max(0, off - v0)), hi = min(16, max(0, lim - v0));
-                const uint32_t valid = ((1u << hi) - 1u) & ~((1u << lo) - 1u);
-                const uint32_t m = byte_lsbs(x.x) | (byte_lsbs(x.y) << 4) | (byte_lsbs(x.z) << 8) |
-                                   (byte_lsbs(x.w) << 12);
-                const uint32_t b = byte_bad(x.x) | (byte_bad(x.y) << 4) | (byte_bad(x.z) << 8) |
-                                   (byte_bad(x.w) << 12);
-                bad |= b & valid;
-                if (j < 4 || lane == 0)
-                    reinterpret_cast<uint16_t *>(buf)[32 * j + lane] = static_cast<uint16_t>(m & valid);
-            }
-            __syncwarp();  // (the other turn's buffer is written next: every lane has read it by then)
-            const uint64_t b0 = buf[lane], b1 = buf[lane + 1];
-            const uint64_t e = off ? (b0 >> off) | (b1 << (64 - off)) : b0;
-            const int w = 32 * c.seg + lane;
-            if (w < c.wp) {
-                row[w] = e | (w == (r >> 6) ? 1ull << (r & 63) : 0ull);
-                ones += __popcll(e);
-            }
-            if (32 * (c.seg + 1) >= c.wp) {
-                ones = __reduce_add_sync(kFull, ones);
-                if (lane == 0) cnt[c.row0 + r] = ones;
-                ones = 0;
-            }
-        }
-        c = d;
-#pragma unroll
-        for (int j = 0; j < 5; ++j) cur[j] = nxt[j];
+    batch_pack_kernel(const BatchInst *__restrict__ inst, const int *__restrict__ tinst, int *cnt, int *status) {
+    extern __shared__ uint64_t pack_s[];
+    __shared__ int cnt_s[kTileRows];
+    const BatchInst I = inst[tinst[blockIdx.x]];
+    const int n = I.n, wp = I.wp, R = tile_rows(n);
+    const int r0 = (static_cast<int>(blockIdx.x) - I.tile0) * R, r1 = min(I.np, r0 + R);
+    if (threadIdx.x < kTileRows) cnt_s[threadIdx.x] = 0;
+    bool bad = false;
+    if (r0 < n) {
+        pack_tile(I.E, n, wp, r0, min(r1, n), pack_s, &bad, [&](int r, int w, uint64_t e) {
+            I.rbits[static_cast<int64_t>(r) * wp + w] = e | (w == (r >> 6) ? 1ull << (r & 63) : 0ull);
+            if (e != 0ull) atomicAdd(&cnt_s[r - r0], __popcll(e));
+        });
     }
-    if (__any_sync(kFull, bad != 0) && lane == 0) atomicOr(status, ST_BAD_INPUT);
+    for (int t = max(r0, n) * wp + threadIdx.x; t < r1 * wp; t += blockDim.x) {  // padding: identity only
+        const int r = t / wp, w = t - r * wp;
+        I.rbits[t] = w == (r >> 6) ? 1ull << (r & 63) : 0ull;
+    }
+    if (bad) atomicOr(status, ST_BAD_INPUT);
+    __syncthreads();
+    for (int i = threadIdx.x; i < min(r1, n) - r0; i += blockDim.x) cnt[I.row0 + r0 + i] = cnt_s[i];
 }
 
 // Successor lists from the packed bits: eight lanes to a row, four words a lane at a time, four
@@ -926,7 +844,8 @@ dl_status solve_tc_batch(dl_ctx *ctx, Workspace &ws, cudaStream_t s, int32_t cou
     const int tm = gemm_tile_m();
     std::vector<BatchInst> inst(L);
     int64_t in_bytes = 0, mat_bytes = 0, bit_words = 0, prow = 0, row = 0, max_np = 0, max_wp = 0, tiles = 0,
-            wp_words = 0;
+            wp_words = 0, row_tiles = 0;
+    size_t tile_smem = 0;
     for (int i = 0; i < L; ++i) {
         const int32_t n = ns[live[i]];
         const int64_t np = round_up(n, 128);
@@ -936,6 +855,9 @@ dl_status solve_tc_batch(dl_ctx *ctx, Workspace &ws, cudaStream_t s, int32_t cou
         inst[i].tiles = static_cast<int32_t>(((np + tm - 1) / tm) * ((np + bn - 1) / bn));
         inst[i].prow0 = static_cast<int32_t>(std::min<int64_t>(prow, INT32_MAX));
         inst[i].row0 = static_cast<int32_t>(std::min<int64_t>(row, INT32_MAX));
+        inst[i].tile0 = static_cast<int32_t>(std::min<int64_t>(row_tiles, INT32_MAX));
+        row_tiles += (np + tile_rows(n) - 1) / tile_rows(n);
+        tile_smem = std::max(tile_smem, tile_words(n, tile_rows(n)) * 8);
         prow += np;
         row += n;
         tiles += inst[i].tiles;
@@ -979,13 +901,14 @@ dl_status solve_tc_batch(dl_ctx *ctx, Workspace &ws, cudaStream_t s, int32_t cou
     auto *dslices = static_cast<BatchSlice *>(ws.get("batch_slices", std::max<size_t>(slice_bytes, 16)));
     auto *dnslices = static_cast<int *>(ws.get("batch_nslices", sizeof(int) * L));
     auto *pinst = static_cast<int *>(ws.get("batch_pinst", sizeof(int) * total_prows));
+    auto *tinst = static_cast<int *>(ws.get("batch_tinst", sizeof(int) * row_tiles));
     auto *gcnt = static_cast<int *>(ws.get("batch_cnt", sizeof(int) * (total_rows + 1)));
     auto *gptr = static_cast<int *>(ws.get("batch_ptr", sizeof(int) * (total_rows + 1)));
     auto *scratch = static_cast<int *>(ws.get("batch_scan", sizeof(int) * 2 * (scan_blocks + 1)));
     uint8_t *staging = nullptr;
     if (mem == DL_MEM_HOST) staging = static_cast<uint8_t *>(ws.get("batch_in", std::max<int64_t>(in_bytes, 256)));
-    if (!rb || !mb || !cmask || !ctr || !state || !lists || !dinst || !dslices || !dnslices || !pinst || !gcnt ||
-        !gptr || !scratch || (mem == DL_MEM_HOST && !staging)) {
+    if (!rb || !mb || !cmask || !ctr || !state || !lists || !dinst || !dslices || !dnslices || !pinst || !tinst ||
+        !gcnt || !gptr || !scratch || (mem == DL_MEM_HOST && !staging)) {
         set_error("batch: device allocation failed (%.2f GB of bits)", 16.0 * bit_words / 1e9);
         return DL_ENOMEM;
     }
@@ -1020,9 +943,8 @@ dl_status solve_tc_batch(dl_ctx *ctx, Workspace &ws, cudaStream_t s, int32_t cou
     // 1. bits of I + E, counts and checks over all inputs, then the CSR row pointers (every
     //    call: the contents, hence the number of facts, may differ between calls)
     BCK(cudaMemsetAsync(ws.status, 0, sizeof(int), s));
-    batch_map_kernel<<<L, 256, 0, s>>>(dinst, pinst);
-    const unsigned pack_blocks = static_cast<unsigned>((total_prows + 8 * kPackRows - 1) / (8 * kPackRows));
-    batch_pack_kernel<<<pack_blocks, 256, 0, s>>>(dinst, pinst, static_cast<int>(total_prows), gcnt, ws.status);
+    batch_map_kernel<<<L, 256, 0, s>>>(dinst, pinst, tinst);
+    batch_pack_kernel<<<static_cast<unsigned>(row_tiles), 256, tile_smem, s>>>(dinst, tinst, gcnt, ws.status);
     BCK(cudaGetLastError());
     BCK(exclusive_scan_large(gcnt, static_cast<int>(total_rows), gptr, scratch, s));
     const int pre_launches = 2 + (total_rows > 64 * 1024 ? 3 : 1);

@@ -36,36 +36,56 @@ __global__ void csr_count_kernel(const uint8_t *__restrict__ E, int n, int *cnt)
     if (lane == 0) cnt[i] = c;
 }
 
-// One pass over E (warp per padded row): bits of I + E into M, successor counts, the 0/1
+// One pass over E (a CTA per tile of rows, pack_tile): bits of I + E into M, successor counts, the 0/1
 // check, ||E||_inf (max row count), nnz and the number of self-loops.
 __global__ void __launch_bounds__(256, 4)
-    csr_pack_check_kernel(const uint8_t *__restrict__ E, int n, int np, int wp, int *cnt, uint64_t *M,
+    csr_pack_check_kernel(const uint8_t *__restrict__ E, int n, int np, int wp, int R, int *cnt, uint64_t *M,
                           unsigned long long *dmax, unsigned long long *nnz, unsigned long long *diag,
                           int *status, uint64_t *colmask) {
     extern __shared__ uint64_t colmask_s[];  // the CTA's rows' facts, merged into colmask at the end
+    __shared__ int cnt_s[kTileRows], self_s;
+    uint64_t *buf = colmask_s + wp;
+    const int r0 = blockIdx.x * R, r1 = min(np, r0 + R);
     for (int w = threadIdx.x; w < wp; w += blockDim.x) colmask_s[w] = 0ull;
-    __syncthreads();
-    const int lane = threadIdx.x & 31;
-    const int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    uint64_t *row = M + static_cast<int64_t>(r) * wp;
-    if (r >= n && r < np) {  // padding: identity only
-        for (int w = lane; w < wp; w += 32) row[w] = w == (r >> 6) ? 1ull << (r & 63) : 0ull;
-    } else if (r < n) {
-        const uint8_t *a = E + static_cast<int64_t>(r) * n;
-        int c = 0;
-        bool bad = false;
-        pack_row_bits(a, n, r, wp, row, lane, c, bad, colmask_s);
-        if (lane == 0) {
-            cnt[r] = c;
-            if (bad) atomicOr(status, ST_BAD_INPUT);
-            if (c) {
-                atomicMax(dmax, static_cast<unsigned long long>(c));
-                atomicAdd(nnz, static_cast<unsigned long long>(c));
+    if (threadIdx.x < kTileRows) cnt_s[threadIdx.x] = 0;
+    if (threadIdx.x == 0) self_s = 0;
+    bool bad = false;
+    if (r0 < n) {
+        pack_tile(E, n, wp, r0, min(r1, n), buf, &bad, [&](int r, int w, uint64_t e) {
+            const bool mine = w == (r >> 6);
+            const uint64_t idb = mine ? 1ull << (r & 63) : 0ull;
+            M[static_cast<int64_t>(r) * wp + w] = e | idb;
+            if (e != 0ull) {
+                atomicAdd(&cnt_s[r - r0], __popcll(e));
+                or_shared(colmask_s + w, e);
+                if (e & idb) atomicAdd(&self_s, 1);
             }
-            if (a[r] & 1) atomicAdd(diag, 1ull);
+        });
+    }
+    for (int64_t t = static_cast<int64_t>(max(r0, n)) * wp + threadIdx.x; t < static_cast<int64_t>(r1) * wp;
+         t += blockDim.x) {  // padding: identity only
+        const int r = static_cast<int>(t / wp), w = static_cast<int>(t - static_cast<int64_t>(r) * wp);
+        M[t] = w == (r >> 6) ? 1ull << (r & 63) : 0ull;
+    }
+    bad = __syncthreads_or(bad);
+    if (threadIdx.x < 32) {
+        int top = 0, sum = 0;
+        for (int i = threadIdx.x; i < min(r1, n) - r0; i += 32) {
+            cnt[r0 + i] = cnt_s[i];
+            top = max(top, cnt_s[i]);
+            sum += cnt_s[i];
+        }
+        top = __reduce_max_sync(0xffffffffu, top);
+        sum = __reduce_add_sync(0xffffffffu, sum);
+        if (threadIdx.x == 0) {
+            if (bad) atomicOr(status, ST_BAD_INPUT);
+            if (sum) {
+                atomicMax(dmax, static_cast<unsigned long long>(top));
+                atomicAdd(nnz, static_cast<unsigned long long>(sum));
+            }
+            if (self_s) atomicAdd(diag, static_cast<unsigned long long>(self_s));
         }
     }
-    __syncthreads();
     for (int w = threadIdx.x; w < wp; w += blockDim.x)
         if (colmask_s[w] != 0ull) atomicOr(reinterpret_cast<unsigned long long *>(colmask + w), colmask_s[w]);
 }
@@ -179,21 +199,19 @@ __global__ void __launch_bounds__(256)
     fill_row_from_bits(M + static_cast<int64_t>(r) * wp, wp, r, ptr[r], ptr[r + 1], col, lane);
 }
 
-// Bits of E alone (no identity; rows >= n zero), the 0/1 check; warp per padded row.
+// Bits of E alone (no identity; rows >= n zero), the 0/1 check; a CTA per tile of rows.
 __global__ void __launch_bounds__(256, 4)
-    pack_bits_kernel(const uint8_t *__restrict__ E, int n, int np, int wp, uint64_t *M, int *status) {
-    const int lane = threadIdx.x & 31;
-    const int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (r >= np) return;
-    uint64_t *row = M + static_cast<int64_t>(r) * wp;
-    if (r >= n) {
-        for (int w = lane; w < wp; w += 32) row[w] = 0ull;
-        return;
-    }
-    int c = 0;
+    pack_bits_kernel(const uint8_t *__restrict__ E, int n, int np, int wp, int R, uint64_t *M, int *status) {
+    extern __shared__ uint64_t pack_s[];
+    const int r0 = blockIdx.x * R, r1 = min(np, r0 + R);
     bool bad = false;
-    pack_row_bits(E + static_cast<int64_t>(r) * n, n, r, wp, row, lane, c, bad, nullptr, false);
-    if (lane == 0 && bad) atomicOr(status, ST_BAD_INPUT);
+    if (r0 < n)
+        pack_tile(E, n, wp, r0, min(r1, n), pack_s, &bad,
+                  [&](int r, int w, uint64_t e) { M[static_cast<int64_t>(r) * wp + w] = e; });
+    for (int64_t t = static_cast<int64_t>(max(r0, n)) * wp + threadIdx.x; t < static_cast<int64_t>(r1) * wp;
+         t += blockDim.x)
+        M[t] = 0ull;
+    if (bad) atomicOr(status, ST_BAD_INPUT);
 }
 
 // Exclusive scan in one CTA: each thread holds 16 consecutive counts in registers, a warp
@@ -433,13 +451,22 @@ cudaError_t csr_build(const uint8_t *E, int n, int *cnt, int *ptr, cudaStream_t 
     return cudaGetLastError();
 }
 
+// Shared memory beyond 48 KB (rows of more than 190 000 columns) is asked for.
+template <class Kernel>
+static cudaError_t tile_smem(Kernel kernel, size_t smem) {
+    if (smem <= 48 * 1024) return cudaSuccess;
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+}
+
 cudaError_t csr_pack_checked(const uint8_t *E, int n, int np, int64_t wp, int *cnt, int *ptr, uint64_t *M,
                              unsigned long long *dmax, unsigned long long *nnz, unsigned long long *diag, int *status,
                              uint64_t *colmask, cudaStream_t s) {
     if (wp > 6144) return cudaErrorInvalidValue;  // the CTA's column mask lives in shared memory
-    const size_t smem = static_cast<size_t>(wp) * sizeof(uint64_t);
-    csr_pack_check_kernel<<<static_cast<unsigned>((np + 7) / 8), 256, smem, s>>>(
-        E, n, np, static_cast<int>(wp), cnt, M, dmax, nnz, diag, status, colmask);
+    const int R = tile_rows(n, n <= kTileSmallN ? kTileBytesSmall : kTileBytes);
+    const size_t smem = (static_cast<size_t>(wp) + tile_words(n, R)) * sizeof(uint64_t);
+    if (const cudaError_t e = tile_smem(csr_pack_check_kernel, smem)) return e;
+    csr_pack_check_kernel<<<static_cast<unsigned>((np + R - 1) / R), 256, smem, s>>>(
+        E, n, np, static_cast<int>(wp), R, cnt, M, dmax, nnz, diag, status, colmask);
     return launch_programmatic(exclusive_scan_kernel, dim3(1), dim3(1024), 0, s, static_cast<const int *>(cnt), n, ptr);
 }
 
@@ -461,7 +488,11 @@ cudaError_t unpack_bits_u8(const uint64_t *Eb, int n, uint8_t *E, int *status, c
 }
 
 cudaError_t pack_bits(const uint8_t *E, int n, int np, int64_t wp, uint64_t *M, int *status, cudaStream_t s) {
-    pack_bits_kernel<<<static_cast<unsigned>((np + 7) / 8), 256, 0, s>>>(E, n, np, static_cast<int>(wp), M, status);
+    const int R = tile_rows(n, n <= kTileSmallN ? kTileBytesSmall : kTileBytes);
+    const size_t smem = tile_words(n, R) * sizeof(uint64_t);
+    if (const cudaError_t e = tile_smem(pack_bits_kernel, smem)) return e;
+    pack_bits_kernel<<<static_cast<unsigned>((np + R - 1) / R), 256, smem, s>>>(E, n, np, static_cast<int>(wp), R, M,
+                                                                                status);
     return cudaGetLastError();
 }
 

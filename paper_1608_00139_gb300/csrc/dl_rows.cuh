@@ -203,6 +203,26 @@ __device__ __forceinline__ uint32_t byte_bad(uint32_t x) {
     return byte_lsbs(((t + 0x7F7F7F7Fu) | t) >> 7);
 }
 
+// Sixteen bytes that are 0 or 1 as 16 bits, byte b -> bit b, in five operations: a product with a
+// multiplier of four powers of two gathers a word's bytes in its top four bits (no lower sum
+// carries), a second word's land above them.  Any byte that is neither 0 nor 1 is left in `bad`, and
+// the bits are then of no use.
+__device__ __forceinline__ uint32_t pack16(const uint4 &x, uint32_t &bad) {
+    bad |= (x.x | x.y | x.z | x.w) & 0xFEFEFEFEu;
+    const uint32_t lo = x.x * 0x01020408u + x.y * 0x10204080u, hi = x.z * 0x01020408u + x.w * 0x10204080u;
+    return __byte_perm(lo, hi, 0x73) & 0xFFFFu;
+}
+// The bytes of x outside [lo, hi) cleared.
+__device__ __forceinline__ uint4 keep_bytes(const uint4 &x, int lo, int hi) {
+    auto word = [&](uint32_t v, int at) {
+        const int a = min(4, max(0, lo - at)), b = min(4, max(0, hi - at));
+        const uint32_t below_b = b == 4 ? 0xFFFFFFFFu : (1u << (8 * b)) - 1u;
+        const uint32_t below_a = a == 4 ? 0xFFFFFFFFu : (1u << (8 * a)) - 1u;
+        return v & below_b & ~below_a;
+    };
+    return make_uint4(word(x.x, 0), word(x.y, 4), word(x.z, 8), word(x.w, 12));
+}
+
 // *word |= e on shared memory, as 32-bit operations on the halves that have bits (a 64-bit one is a loop
 // of compare and swap).
 __device__ __forceinline__ void or_shared(uint64_t *word, uint64_t e) {
@@ -212,92 +232,68 @@ __device__ __forceinline__ void or_shared(uint64_t *word, uint64_t e) {
     if (hi != 0u) atomicOr(h + 1, hi);
 }
 
-// One warp packs row r of a 0/1 byte matrix (the n bytes at a, any alignment) into wp 64-bit
-// words at `row`, plus the identity bit r.  The row is read as aligned 16-byte chunks: lane
-// L of segment s holds the 64 bytes that start 64 (32 s + L) bytes after the aligned address
-// below a, and each model word is two of those 64-bit groups shifted by the misalignment.
-// Bytes outside the row are masked off (they are never counted or checked).  Every lane
-// returns the row's count of ones (without the identity) and whether a byte was not 0/1.
-// With colmask (shared memory, wp words) the row's facts are also ORed into it; without
-// identity the bit r is not added.
-__device__ __forceinline__ void pack_row_bits(const uint8_t *a, int n, int r, int wp, uint64_t *row, int lane,
-                                              int &count, bool &bad_byte, uint64_t *colmask = nullptr,
-                                              bool identity = true) {
-    const int idw = identity ? r >> 6 : -1;
-    const uint64_t idb = 1ull << (r & 63);
-    const int off = static_cast<int>(reinterpret_cast<uintptr_t>(a) & 15);
-    const uint8_t *base = a - off;
-    const int lim = off + n;  // the row occupies bytes [off, lim) from base
-    const int nseg = wp / 32 + 1;
-    uint32_t bad = 0;
-    int c = 0;
-    uint64_t carry = 0;
-    auto shifted = [off](uint64_t lo, uint64_t hi) { return off ? (lo >> off) | (hi << (64 - off)) : lo; };
-    // the next segment's chunks are loaded before this one is processed (two in flight)
-    uint4 cur[4];
-    auto load = [&](int sg, uint4 (&x)[4]) {
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int v0 = 64 * (32 * sg + lane) + 16 * j;
-            x[j] = v0 < lim ? *reinterpret_cast<const uint4 *>(base + v0) : make_uint4(0u, 0u, 0u, 0u);
-        }
-    };
-    load(0, cur);
-    for (int sg = 0; sg < nseg; ++sg) {
-        const int u = 32 * sg + lane;
-        uint4 nx[4] = {};
-        if (sg + 1 < nseg) load(sg + 1, nx);
-        uint64_t vw = 0;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int v0 = 64 * u + 16 * j;
-            if (v0 < lim) {
-                const uint4 x = cur[j];
-                const int lo = max(0, off - v0), hi = min(16, lim - v0);
-                const uint32_t valid = ((1u << hi) - 1u) & ~((1u << lo) - 1u);
-                const uint32_t m = byte_lsbs(x.x) | (byte_lsbs(x.y) << 4) | (byte_lsbs(x.z) << 8) |
-                                   (byte_lsbs(x.w) << 12);
-                const uint32_t b = byte_bad(x.x) | (byte_bad(x.y) << 4) | (byte_bad(x.z) << 8) |
-                                   (byte_bad(x.w) << 12);
-                vw |= static_cast<uint64_t>(m & valid) << (16 * j);
-                bad |= b & valid;
-            }
-        }
-        c += __popcll(vw);
-        const uint64_t nxt = __shfl_down_sync(0xffffffffu, vw, 1);
-        const uint64_t first = __shfl_sync(0xffffffffu, vw, 0);
-        auto put = [&](int w, uint64_t e) {  // e: the facts of word w
-            row[w] = e | (w == idw ? idb : 0ull);
-            if (colmask != nullptr && e != 0ull) or_shared(colmask + w, e);
-        };
-        if (sg > 0 && lane == 31) {
-            const int w = 32 * (sg - 1) + 31;
-            if (w < wp) put(w, shifted(carry, first));
-        }
-        if (lane < 31) {
-            const int w = 32 * sg + lane;
-            if (w < wp) put(w, shifted(vw, nxt));
-        }
-        carry = vw;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) cur[j] = nx[j];
-    }
-    if (lane == 31) {
-        const int w = 32 * (nseg - 1) + 31;
-        if (w < wp) {
-            const uint64_t e = shifted(carry, 0ull);
-            row[w] = e | (w == idw ? idb : 0ull);
-            if (colmask != nullptr && e != 0ull) or_shared(colmask + w, e);
-        }
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        c += __shfl_xor_sync(0xffffffffu, c, o);
-        bad |= __shfl_xor_sync(0xffffffffu, bad, o);
-    }
-    count = c;
-    bad_byte = bad != 0;
+// The bits of the rows [r0, r1) of an n x n 0/1 byte matrix (any alignment) by one CTA.  The rows are
+// one run of bytes, so they are read as such: coalesced 16-byte pieces, eight in flight a thread, packed
+// to a run of bits in `buf` (tile_words words of shared memory), from which word w of row r is read at
+// its bit offset and handed to put(r, w, facts).  Bound by the read: what a row costs beyond its bytes (a
+// warp to a row, pieces at the row's own misalignment) took more issue slots than the 6 operations a
+// piece, TILE_NOTE.  A byte that is neither 0 nor 1 sets *bad for some thread; bytes outside the matrix
+// are cleared (only the first and the last row's pieces can hold any).  Ends with the CTA's threads in
+// their put calls: no barrier behind them.
+constexpr int kTileBytes = 32768;       // a tile where there are many
+constexpr int kTileBytesSmall = 8192;   // and of one matrix of at most kTileSmallN rows (512 tiles at 2048)
+constexpr int kTileSmallN = 4096;
+constexpr int kTileRows = 64;
+__host__ __device__ inline int tile_rows(int64_t n, int bytes = kTileBytes) {
+    const int64_t r = n > 0 ? bytes / n : kTileRows;
+    return static_cast<int>(r < 1 ? 1 : r > kTileRows ? kTileRows : r);
 }
+__host__ __device__ inline size_t tile_words(int64_t n, int rows) {
+    return static_cast<size_t>((rows * n + 15 + 127) / 64 + 1);
+}
+
+template <class Put>
+__device__ __forceinline__ void pack_tile(const uint8_t *__restrict__ E, int n, int wp, int r0, int r1, uint64_t *buf,
+                                          bool *bad, Put put) {
+    constexpr int kFly = 8;
+    const uint8_t *a = E + static_cast<int64_t>(r0) * n;
+    const int off = static_cast<int>(reinterpret_cast<uintptr_t>(a) & 15);
+    const int lim = off + (r1 - r0) * n;  // the rows are the bytes [off, lim) from the aligned address below
+    const uint4 *src = reinterpret_cast<const uint4 *>(a - off);
+    const int pieces = (lim + 15) >> 4;
+    const bool edge = r0 == 0 || r1 == n;
+    uint32_t odd = 0;
+    for (int p0 = threadIdx.x; p0 < pieces; p0 += kFly * blockDim.x) {
+        uint4 x[kFly];
+#pragma unroll
+        for (int j = 0; j < kFly; ++j) {
+            const int p = p0 + j * blockDim.x;
+            x[j] = p < pieces ? __ldg(src + p) : make_uint4(0u, 0u, 0u, 0u);
+        }
+#pragma unroll
+        for (int j = 0; j < kFly; ++j) {
+            const int p = p0 + j * blockDim.x;
+            if (p >= pieces) break;
+            if (edge && (16 * p < off || 16 * p + 16 > lim)) x[j] = keep_bytes(x[j], off - 16 * p, lim - 16 * p);
+            reinterpret_cast<uint16_t *>(buf)[p] = static_cast<uint16_t>(pack16(x[j], odd));
+        }
+    }
+    *bad = odd != 0;
+    __syncthreads();
+    for (int t = threadIdx.x; t < (r1 - r0) * wp; t += blockDim.x) {
+        const int i = t / wp, w = t - i * wp;
+        const int left = n - 64 * w;  // columns from this word on
+        uint64_t e = 0ull;
+        if (left > 0) {
+            const int at = off + i * n + 64 * w, sh = at & 63;
+            e = buf[at >> 6] >> sh;
+            if (sh) e |= buf[(at >> 6) + 1] << (64 - sh);
+            if (left < 64) e &= (1ull << left) - 1ull;
+        }
+        put(r0 + i, w, e);
+    }
+}
+
 
 // One warp writes the successor list of row r into col[pos0 .. pos1) from its packed bits
 // (I + E: the identity bit belongs to E only when the row holds pos1 - pos0 ones).
