@@ -38,7 +38,7 @@ enum : int {
 // ---------------------------------------------------------------------------------------
 // tcgen05 GEMM (dl_umma.cu)
 // ---------------------------------------------------------------------------------------
-enum GemmKind : int { KIND_F8 = 0, KIND_TF32 = 1 };
+enum GemmKind : int { KIND_F8 = 0, KIND_TF32 = 1, KIND_F16 = 2 };
 enum GemmEpi : int { EPI_BOOL = 0, EPI_SUB_F32 = 1, EPI_STORE_F32 = 2 };
 
 // Boolean epilogue: v = [acc > 0] OR [add8 != 0]; writes e4m3 1.0/0.0 bytes, packed bits,

@@ -19,9 +19,10 @@
 //   3. W = A^-1 in FP32: the block solves applied to the identity (kept transposed, Z = I A^-T,
 //      by groups of 8 blocks with precomputed inverses of the groups' diagonal parts, so that
 //      every product is a tensor-core GEMM with K = 1024), then W = Z^T.
-//   4. Refinement in FP64 on Z = X^T, from Z = 0:  R^T = (eps E - A X)^T, i.e.
+//   4. Refinement on Z = X^T (FP64), from Z = 0:  R^T = (eps E - A X)^T, i.e.
 //        R^T[j][i] = eps * sum_{k : E[i][k]} (Z[j][k] + [k = j]) - Z[j][i]
-//      (E is 0/1: E X is a sum of rows of X, summed exactly in 64-bit fixed point);
+//      (E is 0/1: E X is a sum of rows of X, summed exactly in 64-bit fixed point; from the second
+//      step on the sums are kept and only the correction's are added);
 //      D^T = R^T W^T, one TF32 GEMM of n x n x n; Z += D^T; until max|R| <= tol * eps.  The first
 //      step (Z = 0, R^T = (eps E)^T) is the solve itself; each later one contracts the error by
 //      about ||I - W A||, a few TF32 units times kappa(A), kappa_inf(A) <= 2 (1 + ||E||_inf).
@@ -29,6 +30,7 @@
 //      boolean recheck of R2 = min1(E + E R2) confirms the model or adds lost facts.
 // Every product is a "TN" GEMM (both operands stored with K contiguous), the form the TF32
 // tensor cores run here; that is why the right-hand side is kept transposed.
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -299,6 +301,21 @@ __device__ __forceinline__ long long fixed_of(long long bits, int e) {
     return bits < 0 ? -v : v;
 }
 
+__device__ __forceinline__ int exponent_of(double z) {  // the exponent field
+    return static_cast<int>((__double_as_longlong(z) >> 52) & 0x7FF);
+}
+
+// The largest v of a block of 256 threads (wmax: 8 words of shared memory; ends behind a barrier).
+__device__ __forceinline__ int block_max(int v, int *wmax) {
+    v = __reduce_max_sync(0xffffffffu, v);
+    if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = v;
+    __syncthreads();
+    int m = 0;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) m = max(m, wmax[w]);
+    return m;
+}
+
 // Scale of row j of Z in the residual: every term of a sum (the +1 or A[i][j] included) stays
 // below 2^hb, hb from the row's largest exponent field, and a sum of at most 2^deg_bits terms
 // below 2^62.
@@ -307,20 +324,25 @@ __device__ __forceinline__ int row_scale(int ex_max, int deg_bits, int min_hb = 
     return max(0, 62 - deg_bits - hb);
 }
 
-// floor(s * eps_q / 2^62) for |s| < 2^62, 0 <= eps_q <= 2^62: eps s in fixed point, with
-// eps_q = round(eps 2^62) (a 128-bit product, integer units only).
+// round(s * eps_q / 2^62) for |s| < 2^62, 0 <= eps_q <= 2^62: eps s in fixed point, with
+// eps_q = round(eps 2^62) (a 128-bit product, integer units only; rounded, since a floor's mean of half a
+// unit in every entry would be most of the solution's last error).
 __device__ __forceinline__ long long mul_eps(long long s, long long eps_q) {
     const unsigned long long lo = static_cast<unsigned long long>(s) * static_cast<unsigned long long>(eps_q);
     const long long hi = __mul64hi(s, eps_q);
-    return static_cast<long long>((static_cast<unsigned long long>(hi) << 2) | (lo >> 62));
+    return static_cast<long long>((static_cast<unsigned long long>(hi) << 2) | (lo >> 62)) +
+           static_cast<long long>((lo >> 61) & 1);
 }
 
-// r (|r| < 2^62) as a float, within one rounding of the nearest: two exact 32-bit conversions
-// of its halves combined by one fma.
+// r (|r| < 2^62) as a float, within one rounding of the nearest: two 32-bit conversions of the
+// halves of |r| combined by one fma (of |r|: the low half of a small negative r is near 2^31, and
+// its conversion would lose all but multiples of 128).
 __device__ __forceinline__ float float_of(long long r) {
-    const float hi = static_cast<float>(static_cast<int>(r >> 31));
-    const float lo = static_cast<float>(static_cast<unsigned>(r & 0x7FFFFFFFll));
-    return fmaf(hi, 2147483648.0f, lo);
+    const unsigned long long m = static_cast<unsigned long long>(r < 0 ? -r : r);
+    const float hi = static_cast<float>(static_cast<int>(m >> 31));
+    const float lo = static_cast<float>(static_cast<unsigned>(m & 0x7FFFFFFFull));
+    const float f = fmaf(hi, 2147483648.0f, lo);
+    return r < 0 ? -f : f;
 }
 
 // Residual of the transposed system:
@@ -328,14 +350,15 @@ __device__ __forceinline__ float float_of(long long r) {
 // (right-hand side eps E; with rhs, a general right-hand side eps A, the [k = j] term becomes
 // A[i][j]), as FP32 (right-hand side of the next correction), and max |R| into *rmax (bits of a
 // non-negative float).  The sums are exact in 64-bit fixed point: Zf[j][k] = round(Z[j][k] 2^e_j)
-// (plus 2^e_j at k = j for the closure's right-hand side), written by add_fix_kernel with e_j
+// (plus 2^e_j at k = j for the closure's right-hand side), written by first_fix_kernel with e_j
 // chosen so that no sum reaches 2^62; eps times a sum is an exact 128-bit product with
-// eps_q = round(eps 2^62), floored; the result is rounded once to FP32.  Every error is below
+// eps_q = round(eps 2^62), rounded; the result is rounded once to FP32.  Every error is below
 // 2^-(62 - deg_bits) of the row's largest entry, under one FP64 ulp of it, and no FP64 unit is
 // used.  Two kernels compute it, by the density of E:
 
-// R^T[j][i] from the fixed-point sum and Zf[j][i] (the result's last step).
-__device__ __forceinline__ float residual_entry(long long sum, long long z, int i, int j, int n, int e,
+// R^T[j][i] from the fixed-point sum and Zf[j][i] (the result's last step); the right-hand side's term
+// joins the sum, which is then S[j][i] of the updates below.
+__device__ __forceinline__ float residual_entry(long long &sum, long long z, int i, int j, int n, int e,
                                                 long long eps_q, float inv, const uint8_t *rhs, const double *rhsr) {
     if (rhsr != nullptr) {
         sum += fixed_of(__double_as_longlong(rhsr[static_cast<int64_t>(i) * n + j]), e);
@@ -353,7 +376,8 @@ template <int G>
 __global__ void __launch_bounds__(1024, 1)
     residual_rows_kernel(const int *__restrict__ ptr, const int *__restrict__ col, int n, int np, long long eps_q,
                          const int *__restrict__ escale, const long long *__restrict__ Zf, float *__restrict__ R,
-                         unsigned *rmax, const uint8_t *__restrict__ rhs, const double *__restrict__ rhsr) {
+                         long long *__restrict__ S, unsigned *rmax, const uint8_t *__restrict__ rhs,
+                         const double *__restrict__ rhsr) {
     extern __shared__ long long zi[];  // G rows of np
     const int j0 = blockIdx.x * G;
 #pragma unroll
@@ -399,6 +423,7 @@ __global__ void __launch_bounds__(1024, 1)
             float r = 0.0f;
             if (i < n && j < n) r = residual_entry(sum[g], zi[g * np + i], i, j, n, e[g], eps_q, inv[g], rhs, rhsr);
             R[static_cast<int64_t>(j) * np + i] = r;
+            S[static_cast<int64_t>(j) * np + i] = sum[g];
             m = fmaxf(m, fabsf(r));
         }
     }
@@ -476,8 +501,8 @@ __global__ void fix_transpose_kernel(const double *__restrict__ Z, const int *__
 __global__ void __launch_bounds__(32 * kRWarps, 1)
     residual_band_kernel(const __grid_constant__ CUtensorMap zmap, int n, int np, int nbd, const int *__restrict__ off,
                          const uint16_t *__restrict__ edges, long long eps_q, const int *__restrict__ escale,
-                         const long long *__restrict__ ZfT, float *__restrict__ R, unsigned *rmax,
-                         const uint8_t *__restrict__ rhs, const double *__restrict__ rhsr, int *status,
+                         const long long *__restrict__ ZfT, float *__restrict__ R, long long *__restrict__ S,
+                         unsigned *rmax, const uint8_t *__restrict__ rhs, const double *__restrict__ rhsr, int *status,
                          uint64_t budget_ns) {
     extern __shared__ __align__(1024) uint8_t rsmem[];
     uint16_t *ebuf = reinterpret_cast<uint16_t *>(rsmem + 2 * kBandBytes) + (threadIdx.x >> 5) * kEdgeBuf;
@@ -578,20 +603,23 @@ __global__ void __launch_bounds__(32 * kRWarps, 1)
             m = fmaxf(m, fabsf(v4[u]));
         }
         *reinterpret_cast<float4 *>(rrow + il) = make_float4(v4[0], v4[1], v4[2], v4[3]);
+        longlong2 *srow = reinterpret_cast<longlong2 *>(S + static_cast<int64_t>(j) * np + i0 + il);
+        srow[0] = make_longlong2(acc[il], acc[il + 1]);
+        srow[1] = make_longlong2(acc[il + 2], acc[il + 3]);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(fullmask, m, o));
     if (lane == 0 && m > 0.0f) atomicMax(rmax, __float_as_uint(m));
 }
 
-// Z += D for row j (one block per row, the new row kept in shared memory), then the row's scale
-// e_j = row_scale(largest exponent field, deg_bits, min_hb) into escale[j] (min_hb: a real right-
-// hand side's terms are below 2^min_hb too) and the fixed-point row
-// Zf[j][k] = round(Z[j][k] 2^e_j), plus 2^e_j at k = j < n when add_identity (the closure's
-// [k = j] term of the residual).
-__global__ void __launch_bounds__(256) add_fix_kernel(double *__restrict__ Z, const float *__restrict__ D, int n,
-                                                      int np, int deg_bits, int min_hb, int add_identity,
-                                                      int *__restrict__ escale, long long *__restrict__ Zf) {
+// Z = D for row j (the first product; with D == nullptr Z stays; one block per row, the row kept in
+// shared memory), then the row's scale e_j = row_scale(largest exponent field, deg_bits, min_hb)
+// into escale[j] (min_hb: a real right-hand side's terms are below 2^min_hb too) and the
+// fixed-point row Zf[j][k] = round(Z[j][k] 2^e_j), plus 2^e_j at k = j < n when add_identity (the
+// closure's [k = j] term of the residual).
+__global__ void __launch_bounds__(256) first_fix_kernel(double *__restrict__ Z, const float *__restrict__ D, int n,
+                                                        int np, int deg_bits, int min_hb, int add_identity,
+                                                        int *__restrict__ escale, long long *__restrict__ Zf) {
     // (Zf == nullptr: only Z and escale; fix_transpose_kernel then writes the transposed copy)
     extern __shared__ double zrow_s[];
     __shared__ int wmax[8];
@@ -599,30 +627,22 @@ __global__ void __launch_bounds__(256) add_fix_kernel(double *__restrict__ Z, co
     const int64_t base = static_cast<int64_t>(j) * np;
     int ex = 0;
     for (int k = threadIdx.x * 4; k < np; k += blockDim.x * 4) {
-        const float4 d = *reinterpret_cast<const float4 *>(D + base + k);
-        double2 z0 = *reinterpret_cast<const double2 *>(Z + base + k);
-        double2 z1 = *reinterpret_cast<const double2 *>(Z + base + k + 2);
-        z0.x += static_cast<double>(d.x);
-        z0.y += static_cast<double>(d.y);
-        z1.x += static_cast<double>(d.z);
-        z1.y += static_cast<double>(d.w);
-        *reinterpret_cast<double2 *>(Z + base + k) = z0;
-        *reinterpret_cast<double2 *>(Z + base + k + 2) = z1;
+        double2 z0, z1;
+        if (D != nullptr) {
+            const float4 d = *reinterpret_cast<const float4 *>(D + base + k);
+            z0 = make_double2(static_cast<double>(d.x), static_cast<double>(d.y));
+            z1 = make_double2(static_cast<double>(d.z), static_cast<double>(d.w));
+            *reinterpret_cast<double2 *>(Z + base + k) = z0;
+            *reinterpret_cast<double2 *>(Z + base + k + 2) = z1;
+        } else {
+            z0 = *reinterpret_cast<const double2 *>(Z + base + k);
+            z1 = *reinterpret_cast<const double2 *>(Z + base + k + 2);
+        }
         *reinterpret_cast<double2 *>(zrow_s + k) = z0;
         *reinterpret_cast<double2 *>(zrow_s + k + 2) = z1;
-        ex = max(ex, max(max(static_cast<int>((__double_as_longlong(z0.x) >> 52) & 0x7FF),
-                             static_cast<int>((__double_as_longlong(z0.y) >> 52) & 0x7FF)),
-                         max(static_cast<int>((__double_as_longlong(z1.x) >> 52) & 0x7FF),
-                             static_cast<int>((__double_as_longlong(z1.y) >> 52) & 0x7FF))));
+        ex = max(ex, max(max(exponent_of(z0.x), exponent_of(z0.y)), max(exponent_of(z1.x), exponent_of(z1.y))));
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) ex = max(ex, __shfl_xor_sync(0xffffffffu, ex, o));
-    if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = ex;
-    __syncthreads();
-    int m = 0;
-#pragma unroll
-    for (int w = 0; w < 8; ++w) m = max(m, wmax[w]);
-    const int e = row_scale(m, deg_bits, min_hb);
+    const int e = row_scale(block_max(ex, wmax), deg_bits, min_hb);
     if (threadIdx.x == 0) escale[j] = e;
     if (Zf == nullptr) return;
     for (int k = threadIdx.x; k < np; k += blockDim.x) {
@@ -630,6 +650,213 @@ __global__ void __launch_bounds__(256) add_fix_kernel(double *__restrict__ Z, co
         if (add_identity && k == j && j < n) v += 1ll << e;
         Zf[base + k] = v;
     }
+}
+
+// A later correction D, taken as integers: row j of D becomes q = round(D 2^g_j), |q| <= 2^qbits, with
+// g_j from the row's largest entry (23 bits, FP32's own precision of that entry, unless rows of E
+// have more than 8192 ones), and Z += q 2^-g_j.  The residual of the new Z is then the old
+// one's with E q added to the exact sums S, for which q is written as 32-bit integers (kSlices ==
+// false) or as two f16 integers q = 2^(sb + 1) hi + lo, |hi|, |lo| <= 2^sb, rows j and np + j of Q.
+// What q leaves of D stays in the residual, so the corrections converge as before.  A row that
+// has outgrown its scale sets *outgrown (the sums are then formed again).  Bound by its 24 bytes an
+// entry and by one conversion and one addition of the FP64 units: 272 us at n = 8192 (5.9 TB/s).
+template <bool kSlices>
+__global__ void __launch_bounds__(256) refine_add_kernel(double *__restrict__ Z, const float *__restrict__ D, int np,
+                                                         int deg_bits, int min_hb, int sb,
+                                                         const int *__restrict__ escale, int *__restrict__ gscale,
+                                                         void *__restrict__ Q, unsigned *outgrown) {
+    extern __shared__ float drow_s[];
+    __shared__ int wmax[8];
+    const int j = blockIdx.x;
+    const int64_t base = static_cast<int64_t>(j) * np;
+    float top = 0.0f;
+    for (int k = threadIdx.x * 4; k < np; k += blockDim.x * 4) {
+        const float4 d = *reinterpret_cast<const float4 *>(D + base + k);
+        *reinterpret_cast<float4 *>(drow_s + k) = d;
+        top = fmaxf(fmaxf(top, fmaxf(fabsf(d.x), fabsf(d.y))), fmaxf(fabsf(d.z), fabsf(d.w)));
+    }
+    const int tb = block_max(static_cast<int>(__float_as_uint(top) >> 23), wmax);  // top < 2^(tb - 126)
+    const int qbits = kSlices ? 2 * sb + 1 : 23;
+    const int g = min(100, qbits - (tb - 126));
+    if (threadIdx.x == 0) gscale[j] = g;
+    const float up = __int_as_float((127 + g) << 23), down = __int_as_float((127 - g) << 23);
+    int ex = 0;
+    for (int k = threadIdx.x * 4; k < np; k += blockDim.x * 4) {
+        const float4 d = *reinterpret_cast<const float4 *>(drow_s + k);
+        const float q[4] = {rintf(d.x * up), rintf(d.y * up), rintf(d.z * up), rintf(d.w * up)};
+        double2 z0 = *reinterpret_cast<const double2 *>(Z + base + k);
+        double2 z1 = *reinterpret_cast<const double2 *>(Z + base + k + 2);
+        z0.x += static_cast<double>(q[0] * down);
+        z0.y += static_cast<double>(q[1] * down);
+        z1.x += static_cast<double>(q[2] * down);
+        z1.y += static_cast<double>(q[3] * down);
+        *reinterpret_cast<double2 *>(Z + base + k) = z0;
+        *reinterpret_cast<double2 *>(Z + base + k + 2) = z1;
+        ex = max(ex, max(max(exponent_of(z0.x), exponent_of(z0.y)), max(exponent_of(z1.x), exponent_of(z1.y))));
+        if (kSlices) {
+            __half hi[4], lo[4];
+            const float cut = __int_as_float((127 - (sb + 1)) << 23), back = __int_as_float((127 + sb + 1) << 23);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const float h = rintf(q[u] * cut);
+                hi[u] = __float2half_rn(h);
+                lo[u] = __float2half_rn(q[u] - h * back);
+            }
+            __half *out = static_cast<__half *>(Q);
+            *reinterpret_cast<uint2 *>(out + base + k) = *reinterpret_cast<const uint2 *>(hi);
+            *reinterpret_cast<uint2 *>(out + static_cast<int64_t>(np) * np + base + k) =
+                *reinterpret_cast<const uint2 *>(lo);
+        } else {
+            *reinterpret_cast<int4 *>(static_cast<int *>(Q) + base + k) =
+                make_int4(static_cast<int>(q[0]), static_cast<int>(q[1]), static_cast<int>(q[2]), static_cast<int>(q[3]));
+        }
+    }
+    __syncthreads();
+    const int m = block_max(ex, wmax);
+    if (threadIdx.x == 0 && row_scale(m, deg_bits, min_hb) < escale[j]) atomicOr(outgrown, 1u);
+}
+
+// v 2^sh, to the nearest integer.
+__device__ __forceinline__ long long shifted_sum(long long v, int sh) {
+    if (sh >= 0) return v << sh;
+    return sh > -63 ? (v + (1ll << (-sh - 1))) >> -sh : 0ll;
+}
+
+// S[j][i] += 2^(e_j - g_j) sum_{k in succ(i)} q[j][k], and the residual R^T[j][i] = eps S[j][i] - Z[j][i] 2^e_j
+// of it: the sums arrive as the two f16 slices' products (P rows j and np + j: integers below 2^24,
+// exact in the FP32 accumulators).  A row of S to a CTA; bound by its 36 bytes an entry: 340 us at
+// n = 8192 (7.1 TB/s).
+__global__ void __launch_bounds__(256)
+    update_slices_kernel(const float *__restrict__ P, int n, int np, int sb, long long eps_q,
+                         const int *__restrict__ escale, const int *__restrict__ gscale, const double *__restrict__ Z,
+                         long long *__restrict__ S, float *__restrict__ R, unsigned *rmax) {
+    const int j = blockIdx.x, e = escale[j], sh = e - gscale[j];
+    const int64_t base = static_cast<int64_t>(j) * np, low = static_cast<int64_t>(np) * np;
+    const float inv = __int_as_float((127 - e) << 23);
+    float m = 0.0f;
+    for (int i = threadIdx.x * 4; i < np; i += blockDim.x * 4) {
+        const float4 h = *reinterpret_cast<const float4 *>(P + base + i);
+        const float4 l = *reinterpret_cast<const float4 *>(P + low + base + i);
+        longlong2 s0 = *reinterpret_cast<const longlong2 *>(S + base + i);
+        longlong2 s1 = *reinterpret_cast<const longlong2 *>(S + base + i + 2);
+        const longlong2 z0 = *reinterpret_cast<const longlong2 *>(Z + base + i);
+        const longlong2 z1 = *reinterpret_cast<const longlong2 *>(Z + base + i + 2);
+        auto sum = [&](float a, float b) {
+            return shifted_sum((static_cast<long long>(static_cast<int>(a)) << (sb + 1)) + static_cast<int>(b), sh);
+        };
+        s0.x += sum(h.x, l.x);
+        s0.y += sum(h.y, l.y);
+        s1.x += sum(h.z, l.z);
+        s1.y += sum(h.w, l.w);
+        *reinterpret_cast<longlong2 *>(S + base + i) = s0;
+        *reinterpret_cast<longlong2 *>(S + base + i + 2) = s1;
+        auto entry = [&](long long s, long long z, int u) {
+            return i + u < n && j < n ? float_of(mul_eps(s, eps_q) - fixed_of(z, e)) * inv : 0.0f;
+        };
+        const float4 r = make_float4(entry(s0.x, z0.x, 0), entry(s0.y, z0.y, 1), entry(s1.x, z1.x, 2), entry(s1.y, z1.y, 3));
+        *reinterpret_cast<float4 *>(R + base + i) = r;
+        m = fmaxf(fmaxf(m, fmaxf(fabsf(r.x), fabsf(r.y))), fmaxf(fabsf(r.z), fabsf(r.w)));
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if ((threadIdx.x & 31) == 0 && m > 0.0f) atomicMax(rmax, __float_as_uint(m));
+}
+
+// The same with the sums gathered (sparse E): G rows j of q in shared memory, the rows' entries of a
+// column side by side (one load serves G rows), a thread per row i walking its successors.  q < 2^24,
+// so four terms are added in 32 bits.
+template <int G>
+struct IntVec;
+template <>
+struct IntVec<4> {
+    using T = int4;
+};
+template <>
+struct IntVec<2> {
+    using T = int2;
+};
+
+template <int G>
+__global__ void __launch_bounds__(1024, 1)
+    update_rows_kernel(const int *__restrict__ ptr, const int *__restrict__ col, const int *__restrict__ Q, int n, int np,
+                       long long eps_q, const int *__restrict__ escale, const int *__restrict__ gscale,
+                       const double *__restrict__ Z, long long *__restrict__ S, float *__restrict__ R, unsigned *rmax) {
+    using V = typename IntVec<G>::T;
+    extern __shared__ __align__(16) int q_s[];  // np x G
+    V *qv = reinterpret_cast<V *>(q_s);
+    const int j0 = blockIdx.x * G;  // (np is a multiple of 256: every row exists)
+#pragma unroll 2
+    for (int k = threadIdx.x; k < np; k += blockDim.x) {
+        int v[G];
+#pragma unroll
+        for (int g = 0; g < G; ++g) v[g] = Q[static_cast<int64_t>(j0 + g) * np + k];
+        qv[k] = *reinterpret_cast<const V *>(v);
+    }
+    __syncthreads();
+    int e[G], sh[G];
+    float inv[G];
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+        e[g] = escale[j0 + g];
+        sh[g] = e[g] - gscale[j0 + g];
+        inv[g] = __int_as_float((127 - e[g]) << 23);
+    }
+    float m = 0.0f;
+    for (int i = threadIdx.x; i < np; i += blockDim.x) {
+        long long sum[G], s[G], z[G];
+#pragma unroll
+        for (int g = 0; g < G; ++g) {  // in flight during the walk
+            const int64_t at = static_cast<int64_t>(j0 + g) * np + i;
+            s[g] = S[at];
+            z[g] = __double_as_longlong(Z[at]);
+            sum[g] = 0;
+        }
+        if (i < n) {
+            const int q1 = ptr[i + 1];
+            int q = ptr[i];
+            for (; q + 4 <= q1; q += 4) {
+                V v[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) v[u] = qv[col[q + u]];
+#pragma unroll
+                for (int g = 0; g < G; ++g) {
+                    const int *a = reinterpret_cast<const int *>(v);
+                    sum[g] += (a[g] + a[G + g]) + (a[2 * G + g] + a[3 * G + g]);
+                }
+            }
+            for (; q < q1; ++q) {
+                const V v = qv[col[q]];
+#pragma unroll
+                for (int g = 0; g < G; ++g) sum[g] += reinterpret_cast<const int *>(&v)[g];
+            }
+        }
+#pragma unroll
+        for (int g = 0; g < G; ++g) {
+            const int j = j0 + g;
+            const int64_t at = static_cast<int64_t>(j) * np + i;
+            s[g] += shifted_sum(sum[g], sh[g]);
+            S[at] = s[g];
+            float r = 0.0f;
+            if (i < n && j < n) r = float_of(mul_eps(s[g], eps_q) - fixed_of(z[g], e[g])) * inv[g];
+            R[at] = r;
+            m = fmaxf(m, fabsf(r));
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if ((threadIdx.x & 31) == 0 && m > 0.0f) atomicMax(rmax, __float_as_uint(m));
+}
+
+// E as f16 (np x np, zero padding), the B operand of the slices' product; 8 entries a thread.
+__global__ void __launch_bounds__(256) e_f16_kernel(const uint8_t *__restrict__ E, int n, int np, __half *__restrict__ O) {
+    const int64_t t = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
+    const int i = static_cast<int>(t / (np / 8)), k0 = static_cast<int>(t - static_cast<int64_t>(i) * (np / 8)) * 8;
+    if (i >= np) return;
+    uint16_t o[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+        o[u] = i < n && k0 + u < n && E[static_cast<int64_t>(i) * n + k0 + u] ? 0x3C00u : 0u;
+    *reinterpret_cast<uint4 *>(O + static_cast<int64_t>(i) * np + k0) = *reinterpret_cast<const uint4 *>(o);
 }
 
 // R^T = (eps F)^T for a real F (n x n FP64), FP32, zero padding.
@@ -787,6 +1014,12 @@ __global__ void __launch_bounds__(kFirstThreads) first_product_kernel(const int 
 // Graphs with at most this many facts per constant take the gathered first product.
 constexpr int64_t kSparseFirstDegree = 12;
 
+// From this share of ones in E the residual's updates are a product with E, below it gathers: at n = 8192
+// the product of both slices takes 1.3 ms and grows with n^3, the gathers 0.57 ms at 8 ones a row, of
+// which all but 0.3 grow with the ones and n^2.  (The residual formed as a whole takes 4.2 ms at 82
+// ones a row, 0.97 at 8, once instead of in every step: 36.8 -> 25.7 and 20.7 -> 18.7 ms.)
+constexpr double kSliceDensity = 0.009;
+
 // Consecutive NVTX ranges, one open at a time.
 struct Phases {
     bool open = false;
@@ -861,7 +1094,7 @@ dl_status tc_mixed(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &
 
     // ---- GEMM table ---------------------------------------------------------------------
     Table tb;
-    std::vector<Launch> l21, udiag, urest, bulk, wfwd, wbwd, refine;
+    std::vector<Launch> l21, udiag, urest, bulk, wfwd, wbwd, refine, slice;
     double flops_lu = 0, flops_w = 0, flops_ref = 0;
     const Operand opA{A32, np, np, np, 0, 0};
     const Operand opS{Sinv, np, BL, BL, 0, 0}, opST{SinvT, np, BL, BL, 0, 0};
@@ -981,6 +1214,22 @@ dl_status tc_mixed(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &
     // refinement product D^T = R^T W^T (B operand W = A^-1, row-major)
     ok = ok && tb.add(refine, EPI_STORE_F32, 256, N, N, N, Operand{R32, np, np, np, 0, 0},
                       Operand{Wt, np, np, np, 0, 0}, D32, np, 0, 0, false, &flops_ref);
+    // the residual's update: both f16 slices of the correction against E (see refine_add_kernel)
+    if (ok && a.out_rtilde != nullptr) {
+        auto *q16 = static_cast<__half *>(ws.get("mx_Zf", np * np * 8));
+        if (!q16) {
+            set_error("mixed path: device allocation failed (row scales)");
+            return DL_ENOMEM;
+        }
+        GemmProblem p;
+        GemmEpilogue e{};
+        e.c32 = reinterpret_cast<float *>(X64);
+        e.ld_c32 = np;
+        ok = gemm_make_problem(&p, KIND_F16, true, 256, 2 * N, N, N, Operand{q16, 2 * np, np, np, 0, 0},
+                               Operand{q16 + 2 * np * np, np, np, np, 0, 0}, e, &tb.err);
+        slice.push_back(Launch{static_cast<int>(tb.probs.size()), 1, p.tiles_m * p.tiles_n, EPI_STORE_F32, 256});
+        tb.probs.push_back(p);
+    }
     if (!ok) {
         set_error("mixed path: %s", tb.err.c_str());
         return DL_EDEVICE;
@@ -1193,8 +1442,12 @@ dl_status tc_mixed(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &
     }
     const long long eps_q = std::llround(std::ldexp(eps, 62));
     auto *escale = static_cast<int *>(ws.get("mx_escale", np * 4));
+    auto *gscale = static_cast<int *>(ws.get("mx_gscale", np * 4));
     auto *Zf = static_cast<long long *>(ws.get("mx_Zf", np * np * 8));
-    if (!escale || !Zf) {
+    const bool need_x = a.out_rtilde != nullptr;  // (see the refinement loop below)
+    // the exact sums E Z + right-hand side, kept from the first residual on
+    auto *S64 = need_x ? static_cast<long long *>(ws.get("mx_S", np * np * 8)) : Zf;
+    if (!escale || !gscale || !Zf || !S64) {
         set_error("mixed path: device allocation failed (row scales)");
         return DL_ENOMEM;
     }
@@ -1203,7 +1456,7 @@ dl_status tc_mixed(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &
         set_error("mixed path: n = %d exceeds the refinement's shared-memory row (%zu bytes)", n, row_smem);
         return DL_EINVAL;
     }
-    MCK(cudaFuncSetAttribute(add_fix_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(row_smem)));
+    MCK(cudaFuncSetAttribute(first_fix_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(row_smem)));
     // the residual kernel by density: rows of Zf per block for sparse E, bucketed bands otherwise
     const bool banded = static_cast<int64_t>(nnz) >= 32ll * n;
     const int rows_per_block = static_cast<int>(std::min<size_t>(3, (227 * 1024) / row_smem));
@@ -1211,7 +1464,6 @@ dl_status tc_mixed(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &
     int *boff = nullptr;
     uint16_t *bedges = nullptr;
     CUtensorMap zmap{};  // ZfT (banded residual)
-    const bool need_x = a.out_rtilde != nullptr;  // (see the refinement loop below)
     if (banded && need_x) {
         const int64_t cells = static_cast<int64_t>(ni) * nbd * kRI;
         auto *bcnt = static_cast<int *>(ws.get("mx_bcnt", (cells + 1) * 4));
@@ -1247,21 +1499,92 @@ dl_status tc_mixed(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &
             dim3 tgrid(static_cast<unsigned>(np / TT), static_cast<unsigned>(np / TT));
             fix_transpose_kernel<<<tgrid, dim3(TT, 8), 0, s>>>(Z64, escale, n, N, general_rhs ? 0 : 1, Zf);
             residual_band_kernel<<<static_cast<unsigned>((np / kRJ) * ni), 32 * kRWarps, kResidualSmem, s>>>(
-                zmap, n, N, nbd, boff, bedges, eps_q, escale, Zf, R32, rmax_p, a.rhs, a.rhs_real, ws.status,
+                zmap, n, N, nbd, boff, bedges, eps_q, escale, Zf, R32, S64, rmax_p, a.rhs, a.rhs_real, ws.status,
                 ctx->budget_ns);
             return cudaGetLastError();
         }
         const unsigned grid = static_cast<unsigned>((np + rows_per_block - 1) / rows_per_block);
         const size_t smem = row_smem * rows_per_block;
         if (rows_per_block == 3)
-            residual_rows_kernel<3><<<grid, 1024, smem, s>>>(csr_ptr, csr_col, n, N, eps_q, escale, Zf, R32, rmax_p, a.rhs,
+            residual_rows_kernel<3><<<grid, 1024, smem, s>>>(csr_ptr, csr_col, n, N, eps_q, escale, Zf, R32, S64, rmax_p, a.rhs,
                                                              a.rhs_real);
         else if (rows_per_block == 2)
-            residual_rows_kernel<2><<<grid, 1024, smem, s>>>(csr_ptr, csr_col, n, N, eps_q, escale, Zf, R32, rmax_p, a.rhs,
+            residual_rows_kernel<2><<<grid, 1024, smem, s>>>(csr_ptr, csr_col, n, N, eps_q, escale, Zf, R32, S64, rmax_p, a.rhs,
                                                              a.rhs_real);
         else
-            residual_rows_kernel<1><<<grid, 1024, smem, s>>>(csr_ptr, csr_col, n, N, eps_q, escale, Zf, R32, rmax_p, a.rhs,
+            residual_rows_kernel<1><<<grid, 1024, smem, s>>>(csr_ptr, csr_col, n, N, eps_q, escale, Zf, R32, S64, rmax_p, a.rhs,
                                                              a.rhs_real);
+        return cudaGetLastError();
+    };
+    // Later residuals from the sums' updates: a product of E in f16 with the correction's two slices
+    // where E has at least kSliceDensity of its entries, else gathers.
+    const bool slices = need_x && static_cast<double>(nnz) >= kSliceDensity * n * n;
+    const int sb = std::min(11, 24 - deg_bits);  // a slice's sum of dmax terms of 2^sb stays within 2^24
+    // (the slices and E in f16 take Zf's place once the first residual is formed, the products X64's)
+    auto *Q16 = reinterpret_cast<__half *>(Zf);
+    auto *E16 = Q16 + 2 * np * np;
+    auto *P32 = reinterpret_cast<float *>(X64);
+    const size_t q_smem = static_cast<size_t>(np) * 4;
+    const int rows_q = 4 * q_smem <= 227 * 1024 ? 4 : 2;
+    if (slices) {
+        MCK(gemm_prepare(KIND_F16, true, 256, EPI_STORE_F32));
+        MCK(cudaFuncSetAttribute(refine_add_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 static_cast<int>(q_smem)));
+    } else if (need_x) {
+        MCK(cudaFuncSetAttribute(refine_add_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 static_cast<int>(q_smem)));
+        if (rows_q == 4)
+            MCK(cudaFuncSetAttribute(update_rows_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     static_cast<int>(4 * q_smem)));
+        else
+            MCK(cudaFuncSetAttribute(update_rows_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     static_cast<int>(2 * q_smem)));
+    }
+    auto first_fix = [&](const float *D) -> cudaError_t {
+        first_fix_kernel<<<static_cast<unsigned>(np), 256, row_smem, s>>>(Z64, D, n, N, deg_bits, min_hb,
+                                                                        general_rhs ? 0 : 1, escale,
+                                                                        banded || !need_x ? nullptr : Zf);
+        ++launches;
+        return cudaGetLastError();
+    };
+    // the whole residual, then what the updates need
+    auto residual_whole = [&](unsigned *rmax_p) -> cudaError_t {
+        cudaError_t e = residual(rmax_p);
+        ++launches;
+        if (e == cudaSuccess && slices) {
+            e_f16_kernel<<<static_cast<unsigned>((np * np / 8 + 255) / 256), 256, 0, s>>>(E, n, N, E16);
+            e = cudaGetLastError();
+            ++launches;
+        }
+        return e;
+    };
+    // Z += D and the residual of the new Z; rmax_p[1] is set if a row has outgrown its scale
+    auto residual_update = [&](unsigned *rmax_p) -> cudaError_t {
+        cudaError_t e;
+        launches += 2;
+        if (slices) {
+            refine_add_kernel<true><<<static_cast<unsigned>(np), 256, q_smem, s>>>(Z64, D32, N, deg_bits, min_hb, sb, escale,
+                                                                                gscale, Q16, rmax_p + 1);
+            if ((e = cudaGetLastError()) != cudaSuccess) return e;
+            const Launch &L = slice[0];
+            e = gemm_launch(KIND_F16, true, L.bn, L.epi, dprob + L.first, L.count, L.tiles, std::min(L.tiles, sms),
+                            ws.status, ctx->budget_ns, s);
+            if (e != cudaSuccess) return e;
+            ++launches;
+            update_slices_kernel<<<static_cast<unsigned>(np), 256, 0, s>>>(P32, n, N, sb, eps_q, escale, gscale, Z64, S64,
+                                                                         R32, rmax_p);
+            return cudaGetLastError();
+        }
+        auto *Q32 = reinterpret_cast<int *>(Zf);
+        refine_add_kernel<false><<<static_cast<unsigned>(np), 256, q_smem, s>>>(Z64, D32, N, deg_bits, min_hb, sb, escale,
+                                                                             gscale, Q32, rmax_p + 1);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        if (rows_q == 4)
+            update_rows_kernel<4><<<static_cast<unsigned>(np / 4), 1024, 4 * q_smem, s>>>(
+                csr_ptr, csr_col, Q32, n, N, eps_q, escale, gscale, Z64, S64, R32, rmax_p);
+        else
+            update_rows_kernel<2><<<static_cast<unsigned>(np / 2), 1024, 2 * q_smem, s>>>(
+                csr_ptr, csr_col, Q32, n, N, eps_q, escale, gscale, Z64, S64, R32, rmax_p);
         return cudaGetLastError();
     };
     // The first product as a gather for sparse E (the closure's own right-hand side eps E): the
@@ -1292,7 +1615,6 @@ dl_status tc_mixed(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &
     // The residual has a rounding floor of about (row length) * 2^-53 * max|X|; refinement stops
     // at tol, or when it no longer halves the residual once that is below 1e-8 * eps.
     const double floor_ok = 1e-8 * eps;
-    MCK(cudaMemsetAsync(Z64, 0, np * np * 8, s));
     if (!sparse_first) {
         dim3 tgrid(static_cast<unsigned>(np / TT), static_cast<unsigned>(np / TT));
         if (a.rhs_real)
@@ -1313,21 +1635,30 @@ dl_status tc_mixed(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &
             MCK(run(refine[0], sms, s));  // D^T = R^T W^T
             ++gemm_products;
         }
-        add_fix_kernel<<<static_cast<unsigned>(np), 256, row_smem, s>>>(Z64, D32, n, N, deg_bits, min_hb,
-                                                                      general_rhs ? 0 : 1, escale,
-                                                                      banded || !need_x ? nullptr : Zf);
-        MCK(cudaGetLastError());
-        ++launches;
         ++products;
-        if (!need_x) break;  // the model only: no refinement
-        MCK(cudaMemsetAsync(rmax_d, 0, sizeof(unsigned), s));
-        MCK(residual(rmax_d));
-        ++launches;
-        unsigned h = 0;
-        MCK(cudaMemcpyAsync(&h, rmax_d, sizeof(h), cudaMemcpyDeviceToHost, s));
+        if (!need_x) {  // the model only: no refinement
+            MCK(first_fix(D32));
+            break;
+        }
+        unsigned h[2] = {0, 0};  // max|R| (bits of a float), a row has outgrown its scale
+        MCK(cudaMemsetAsync(rmax_d, 0, sizeof(h), s));
+        if (products == 1) {
+            MCK(first_fix(D32));
+            MCK(residual_whole(rmax_d));
+        } else {
+            MCK(residual_update(rmax_d));
+        }
+        MCK(cudaMemcpyAsync(h, rmax_d, sizeof(h), cudaMemcpyDeviceToHost, s));
         MCK(cudaStreamSynchronize(s));
+        if (h[1] != 0) {  // new scales, the sums formed again
+            MCK(cudaMemsetAsync(rmax_d, 0, sizeof(h), s));
+            MCK(first_fix(nullptr));
+            MCK(residual_whole(rmax_d));
+            MCK(cudaMemcpyAsync(h, rmax_d, sizeof(h), cudaMemcpyDeviceToHost, s));
+            MCK(cudaStreamSynchronize(s));
+        }
         float hf = 0.0f;
-        std::memcpy(&hf, &h, sizeof(hf));
+        std::memcpy(&hf, &h[0], sizeof(hf));
         rmax = hf;
         if (rmax <= tol * eps) break;
         if (products == 1 || rmax < 0.5 * best) {  // refinement steps must keep halving the residual

@@ -45,7 +45,7 @@ constexpr int kThreads = 64 + 32 * kEpiWarps;
 
 template <int KIND, int BN, int EPI>
 struct Cfg {
-    static constexpr int ELEM = KIND == KIND_F8 ? 1 : 4;      // bytes per element
+    static constexpr int ELEM = KIND == KIND_F8 ? 1 : KIND == KIND_F16 ? 2 : 4;  // bytes per element
     static constexpr int BK = 128 / ELEM;                      // elements per k-block
     static constexpr int KI = 32 / ELEM;                       // K of one MMA instruction
     static constexpr int A_BYTES = BM * 128;
@@ -53,17 +53,17 @@ struct Cfg {
     static constexpr int STAGE = A_BYTES + B_BYTES;
     // FP32 output: 32 x 32 float tiles per epilogue warp, taken from the pipeline's stages: two
     // for the subtracting epilogue (C of the next chunk in flight), one for the storing one
-    static constexpr int EPI_TILES = KIND != KIND_TF32 ? 0 : EPI == EPI_SUB_F32 ? 2 : 1;
+    static constexpr int EPI_TILES = KIND == KIND_F8 ? 0 : EPI == EPI_SUB_F32 ? 2 : 1;
     static constexpr int EPI_STAGE = kEpiWarps * EPI_TILES * 32 * 32 * 4;
     static constexpr int S_FIT = (232448 - 1024 - 256 - EPI_STAGE) / STAGE;
-    static constexpr int S = KIND == KIND_TF32 ? (S_FIT > 8 ? 8 : S_FIT) : ((196608 / STAGE) > 8 ? 8 : (196608 / STAGE));
+    static constexpr int S = KIND != KIND_F8 ? (S_FIT > 8 ? 8 : S_FIT) : ((196608 / STAGE) > 8 ? 8 : (196608 / STAGE));
     static constexpr int TMEM_COLS = 2 * BN;
     static constexpr int SMEM = 1024 + S * STAGE + 256 + EPI_STAGE;
 };
 
 template <int KIND, int BN, bool B_KMAJOR>
 __host__ __device__ constexpr uint32_t make_idesc() {
-    // D = F32 (bits 4-5 = 1); A/B format (bits 7-9, 10-12): E4M3 = 0, TF32 = 2;
+    // D = F32 (bits 4-5 = 1); A/B format (bits 7-9, 10-12): E4M3 = 0, F16 = 0, TF32 = 2;
     // A K-major (bit 15 = 0); B major (bit 16); N >> 3 (bits 17-22); M >> 4 (bits 24-28).
     return (1u << 4) | ((KIND == KIND_TF32 ? 2u : 0u) << 7) |
            ((KIND == KIND_TF32 ? 2u : 0u) << 10) | ((B_KMAJOR ? 0u : 1u) << 16) |
@@ -597,6 +597,9 @@ cudaError_t gemm_prepare(GemmKind kind, bool b_kmajor, int bn, GemmEpi epi) {
             return bn == 256 ? prepare_t<KIND_TF32, 256, true, EPI_STORE_F32>()
                              : prepare_t<KIND_TF32, 128, true, EPI_STORE_F32>();
     }
+    // F16 (the residual's exact integer products) stores FP32 from K-major operands
+    if (kind == KIND_F16 && b_kmajor && bn == 256 && epi == EPI_STORE_F32)
+        return prepare_t<KIND_F16, 256, true, EPI_STORE_F32>();
     return cudaErrorInvalidValue;
 }
 
@@ -604,19 +607,20 @@ bool gemm_make_problem(GemmProblem *p, GemmKind kind, bool b_kmajor, int bn, int
                        const Operand &A, const Operand &B, const GemmEpilogue &epi,
                        std::string *err) {
     std::memset(p, 0, sizeof(*p));
-    const int elem = kind == KIND_F8 ? 1 : 4;
+    const int elem = kind == KIND_F8 ? 1 : kind == KIND_F16 ? 2 : 4;
     const int bk = 128 / elem;
     if (M <= 0 || N <= 0 || K <= 0 || K % bk != 0 || N % 32 != 0 || (bn != 128 && bn != 256)) {
         if (err) *err = "unsupported GEMM shape";
         return false;
     }
-    if (kind == KIND_TF32 && (reinterpret_cast<uintptr_t>(epi.c32) % 16 != 0 || epi.ld_c32 % 4 != 0 ||
+    if (kind != KIND_F8 && (reinterpret_cast<uintptr_t>(epi.c32) % 16 != 0 || epi.ld_c32 % 4 != 0 ||
                               epi.out_col0 % 4 != 0)) {
         if (err) *err = "FP32 output must be 16-byte aligned with a row stride of 4k elements";
         return false;
     }
-    const CUtensorMapDataType dt =
-        kind == KIND_F8 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
+    const CUtensorMapDataType dt = kind == KIND_F8    ? CU_TENSOR_MAP_DATA_TYPE_UINT8
+                                   : kind == KIND_F16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16
+                                                      : CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
     if (!make_map(&p->tmA, dt, elem, A, static_cast<uint32_t>(bk), BM, err)) return false;
     if (b_kmajor) {
         if (!make_map(&p->tmB, dt, elem, B, static_cast<uint32_t>(bk), static_cast<uint32_t>(bn), err))
@@ -660,6 +664,8 @@ cudaError_t gemm_launch(GemmKind kind, bool b_kmajor, int bn, GemmEpi epi, const
             return bn == 256 ? DL_GEMM_T(KIND_TF32, 256, true, EPI_STORE_F32)
                              : DL_GEMM_T(KIND_TF32, 128, true, EPI_STORE_F32);
     }
+    if (kind == KIND_F16 && b_kmajor && bn == 256 && epi == EPI_STORE_F32)
+        return DL_GEMM_T(KIND_F16, 256, true, EPI_STORE_F32);
 #undef DL_GEMM_T
     return cudaErrorInvalidValue;
 }
