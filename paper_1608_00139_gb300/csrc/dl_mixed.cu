@@ -359,11 +359,12 @@ __device__ __forceinline__ float float_of(long long r) {
 // R^T[j][i] from the fixed-point sum and Zf[j][i] (the result's last step); the right-hand side's term
 // joins the sum, which is then S[j][i] of the updates below.
 __device__ __forceinline__ float residual_entry(long long &sum, long long z, int i, int j, int n, int e,
-                                                long long eps_q, float inv, const uint8_t *rhs, const double *rhsr) {
+                                                long long eps_q, float inv, const uint8_t *rhs, const double *rhsr,
+                                                bool rhs_transposed = false) {
     if (rhsr != nullptr) {
         sum += fixed_of(__double_as_longlong(rhsr[static_cast<int64_t>(i) * n + j]), e);
     } else if (rhs != nullptr) {
-        if (rhs[static_cast<int64_t>(i) * n + j]) sum += 1ll << e;
+        if (rhs[rhs_transposed ? static_cast<int64_t>(j) * n + i : static_cast<int64_t>(i) * n + j]) sum += 1ll << e;
     } else if (i == j) {
         z -= 1ll << e;  // Zf carries the [k = j] term
     }
@@ -371,12 +372,13 @@ __device__ __forceinline__ float residual_entry(long long &sum, long long z, int
 }
 
 // (1) Sparse E: G rows j of Zf per block in shared memory, a thread per row i walking its
-// successors (few gathers per row; Zf is read once).
+// successors (few gathers per row; Zf is read once).  rhs_t is A^T (the threads of a warp read 32
+// entries of a row of it; A's own entries, one in each of 32 rows, took half of the kernel's 0.97 ms).
 template <int G>
 __global__ void __launch_bounds__(1024, 1)
     residual_rows_kernel(const int *__restrict__ ptr, const int *__restrict__ col, int n, int np, long long eps_q,
                          const int *__restrict__ escale, const long long *__restrict__ Zf, float *__restrict__ R,
-                         long long *__restrict__ S, unsigned *rmax, const uint8_t *__restrict__ rhs,
+                         long long *__restrict__ S, unsigned *rmax, const uint8_t *__restrict__ rhs_t,
                          const double *__restrict__ rhsr) {
     extern __shared__ long long zi[];  // G rows of np
     const int j0 = blockIdx.x * G;
@@ -421,7 +423,8 @@ __global__ void __launch_bounds__(1024, 1)
             const int j = j0 + g;
             if (j >= np) break;
             float r = 0.0f;
-            if (i < n && j < n) r = residual_entry(sum[g], zi[g * np + i], i, j, n, e[g], eps_q, inv[g], rhs, rhsr);
+            if (i < n && j < n)
+                r = residual_entry(sum[g], zi[g * np + i], i, j, n, e[g], eps_q, inv[g], rhs_t, rhsr, true);
             R[static_cast<int64_t>(j) * np + i] = r;
             S[static_cast<int64_t>(j) * np + i] = sum[g];
             m = fmaxf(m, fabsf(r));
@@ -978,10 +981,10 @@ dl_status mixed_streams(Workspace &ws) {
 
 }  // namespace
 
-// The first product of the refinement when E is sparse: with Z = 0 the residual is R = eps E, and
-// D^T = R^T W^T has rows  D^T[j][:] = eps * sum_{k : E[k][j] = 1} W^T[k][:]  (rows of W^T, row-major
-// in WT, gathered over the predecessors of j from the CSR of E^T): nnz(E) rows read instead of an
-// n^3 product.  Rows j >= n are zero; columns i >= n come out zero (W's padded rows are identity
+// The first product of the refinement when the right-hand side A (the closure's: E) is sparse: with
+// Z = 0 the residual is R = eps A, and D^T = R^T W^T has rows
+// D^T[j][:] = eps * sum_{k : A[k][j] = 1} W^T[k][:]  (rows of W^T, row-major in WT, gathered over the
+// predecessors of j from the CSR of A^T): nnz(A) rows read instead of an n^3 product.  Rows j >= n are zero; columns i >= n come out zero (W's padded rows are identity
 // rows).
 constexpr int kFirstThreads = 256;
 
@@ -1011,7 +1014,7 @@ __global__ void __launch_bounds__(kFirstThreads) first_product_kernel(const int 
     }
 }
 
-// Graphs with at most this many facts per constant take the gathered first product.
+// Right-hand sides with at most this many facts per constant take the gathered first product.
 constexpr int64_t kSparseFirstDegree = 12;
 
 // From this share of ones in E the residual's updates are a product with E, below it gathers: at n = 8192
@@ -1494,6 +1497,7 @@ dl_status tc_mixed(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &
         MCK(cudaFuncSetAttribute(residual_rows_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
         MCK(cudaFuncSetAttribute(residual_rows_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     }
+    const uint8_t *rhs_t = nullptr;  // A^T, set below for the general right-hand side
     auto residual = [&](unsigned *rmax_p) -> cudaError_t {
         if (banded) {
             dim3 tgrid(static_cast<unsigned>(np / TT), static_cast<unsigned>(np / TT));
@@ -1506,13 +1510,13 @@ dl_status tc_mixed(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &
         const unsigned grid = static_cast<unsigned>((np + rows_per_block - 1) / rows_per_block);
         const size_t smem = row_smem * rows_per_block;
         if (rows_per_block == 3)
-            residual_rows_kernel<3><<<grid, 1024, smem, s>>>(csr_ptr, csr_col, n, N, eps_q, escale, Zf, R32, S64, rmax_p, a.rhs,
+            residual_rows_kernel<3><<<grid, 1024, smem, s>>>(csr_ptr, csr_col, n, N, eps_q, escale, Zf, R32, S64, rmax_p, rhs_t,
                                                              a.rhs_real);
         else if (rows_per_block == 2)
-            residual_rows_kernel<2><<<grid, 1024, smem, s>>>(csr_ptr, csr_col, n, N, eps_q, escale, Zf, R32, S64, rmax_p, a.rhs,
+            residual_rows_kernel<2><<<grid, 1024, smem, s>>>(csr_ptr, csr_col, n, N, eps_q, escale, Zf, R32, S64, rmax_p, rhs_t,
                                                              a.rhs_real);
         else
-            residual_rows_kernel<1><<<grid, 1024, smem, s>>>(csr_ptr, csr_col, n, N, eps_q, escale, Zf, R32, S64, rmax_p, a.rhs,
+            residual_rows_kernel<1><<<grid, 1024, smem, s>>>(csr_ptr, csr_col, n, N, eps_q, escale, Zf, R32, S64, rmax_p, rhs_t,
                                                              a.rhs_real);
         return cudaGetLastError();
     };
@@ -1587,23 +1591,38 @@ dl_status tc_mixed(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &
                 csr_ptr, csr_col, Q32, n, N, eps_q, escale, gscale, Z64, S64, R32, rmax_p);
         return cudaGetLastError();
     };
-    // The first product as a gather for sparse E (the closure's own right-hand side eps E): the
-    // CSR of E^T from a transposed byte copy of E.
-    const bool sparse_first = !general_rhs && static_cast<int64_t>(nnz) <= kSparseFirstDegree * n;
+    // The first product as a gather for a sparse right-hand side eps A (the closure's: eps E), from the
+    // CSR of A^T (from a transposed byte copy).
+    const uint8_t *rhs_bytes = a.rhs_real ? nullptr : a.rhs ? a.rhs : E;
+    bool sparse_first = rhs_bytes && (a.rhs || static_cast<int64_t>(nnz) <= kSparseFirstDegree * n);
     int *pptr = nullptr, *pcol = nullptr;
     if (sparse_first) {
-        auto *Et = static_cast<uint8_t *>(ws.get("mx_Et", static_cast<size_t>(n) * n));
+        auto *At = static_cast<uint8_t *>(ws.get("mx_Et", static_cast<size_t>(n) * n));
         auto *pcnt = static_cast<int *>(ws.get("mx_pcnt", (np + 1) * 4));
         pptr = static_cast<int *>(ws.get("mx_pptr", (np + 1) * 4));
-        pcol = static_cast<int *>(ws.get("mx_pcol", static_cast<size_t>(std::max(nnz, 1)) * 4));
-        if (!Et || !pcnt || !pptr || !pcol) {
-            set_error("mixed path: device allocation failed (CSR of E^T)");
+        if (!At || !pcnt || !pptr) {
+            set_error("mixed path: device allocation failed (CSR of the right-hand side)");
             return DL_ENOMEM;
         }
-        MCK(transpose(E, n, n, n, Et, n, s));
-        MCK(csr_build(Et, n, pcnt, pptr, s));
-        MCK(csr_fill(Et, n, pptr, pcol, s));
+        MCK(transpose(rhs_bytes, n, n, n, At, n, s));
+        MCK(csr_build(At, n, pcnt, pptr, s));
         launches += 3;
+        int facts = nnz;
+        if (a.rhs) {
+            MCK(cudaMemcpyAsync(&facts, pptr + n, sizeof(int), cudaMemcpyDeviceToHost, s));
+            MCK(cudaStreamSynchronize(s));
+            sparse_first = static_cast<int64_t>(facts) <= kSparseFirstDegree * n;
+            rhs_t = At;
+        }
+        if (sparse_first) {
+            pcol = static_cast<int *>(ws.get("mx_pcol", static_cast<size_t>(std::max(facts, 1)) * 4));
+            if (!pcol) {
+                set_error("mixed path: device allocation failed (CSR of the right-hand side)");
+                return DL_ENOMEM;
+            }
+            MCK(csr_fill(At, n, pptr, pcol, s));
+            ++launches;
+        }
     }
     // Without an R~ output only the model is wanted: X > 0 after the solve is already exact where
     // it is positive (A is an M-matrix and every quantity of the factorisation keeps its sign, so
