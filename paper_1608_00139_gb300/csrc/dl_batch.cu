@@ -56,6 +56,7 @@ struct BatchInst {
     int32_t prow0;  // first padded row in the order of all instances
     int32_t row0;   // first real row in the order of all instances
     int32_t tile0;  // first tile of rows of the packing, in the order of all instances
+    int32_t slices; // column slices (0: the instance is too large for them)
 };
 
 // Per-instance counters (arrays of `count` entries) and the active-instance counter.
@@ -384,10 +385,12 @@ __global__ void __launch_bounds__(kSliceThreads)
 
 // After the slices: an instance all of whose slices are done is done, the others start over as
 // active ones (from the bits their unfinished slices wrote back).
-__global__ void batch_settle_kernel(const int *__restrict__ nslices, int L, BatchCounters c, int *open) {
+__global__ void batch_settle_kernel(const BatchInst *__restrict__ inst, int L, BatchCounters c, const int *status,
+                                    int *open) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k == 0) open[1] = *status;
     if (k >= L) return;
-    const int want = nslices[k];
+    const int want = inst[k].slices;
     if (want > 0 && c.chg[k] == static_cast<unsigned long long>(want)) {
         c.state[k] = B_DONE;
     } else {
@@ -880,28 +883,22 @@ dl_status solve_tc_batch(dl_ctx *ctx, Workspace &ws, cudaStream_t s, int32_t cou
         return DL_EINVAL;
     }
     const int scan_blocks = static_cast<int>((total_rows + 1023) / 1024);
-    // the columns of every instance of up to kSliceRows constants, the slices with the most work first
-    std::vector<BatchSlice> slices;
-    std::vector<int32_t> nslices(L, 0);
+    // the columns of every instance of up to kSliceRows constants, in slices
+    size_t nslices = 0;
     for (int i = 0; i < L; ++i) {
-        if (inst[i].n > kSliceRows) continue;
-        const int W = slice_words(inst[i].n);
-        for (int w0 = 0; w0 < inst[i].wp; w0 += W, ++nslices[i])
-            slices.push_back(BatchSlice{i, w0, std::min(W, inst[i].wp - w0)});
+        inst[i].slices = inst[i].n > kSliceRows ? 0 : (inst[i].wp + slice_words(inst[i].n) - 1) / slice_words(inst[i].n);
+        nslices += inst[i].slices;
     }
-    std::stable_sort(slices.begin(), slices.end(), [&](const BatchSlice &a, const BatchSlice &b) {
-        return static_cast<int64_t>(a.nw) * inst[a.k].n > static_cast<int64_t>(b.nw) * inst[b.k].n;
-    });
-    const size_t slice_bytes = slices.size() * sizeof(BatchSlice);
     auto *rb = static_cast<uint64_t *>(ws.get("batch_rbits", bit_words * 8));
     auto *mb = static_cast<uint64_t *>(ws.get("batch_mbits", bit_words * 8));
     auto *cmask = static_cast<uint64_t *>(ws.get("batch_colmask", std::max<int64_t>(wp_words, 1) * 8));
-    auto *ctr = static_cast<unsigned long long *>(ws.get("batch_ctr", kCounterArrays * sizeof(unsigned long long) * L));
-    auto *state = static_cast<int *>(ws.get("batch_state", sizeof(int) * (L + 1)));  // and whether any is open
+    // counters, states, whether any instance is open and the status word, read back together
+    const size_t result_bytes = kCounterArrays * sizeof(unsigned long long) * L + sizeof(int) * (L + 2);
+    auto *ctr = static_cast<unsigned long long *>(ws.get("batch_ctr", result_bytes));
+    int *state = ctr ? reinterpret_cast<int *>(ctr + kCounterArrays * static_cast<size_t>(L)) : nullptr;
     auto *lists = static_cast<int *>(ws.get("batch_list", sizeof(int) * (8 + 3 * (L + 1) + 2 + 2 * L + 1)));
     auto *dinst = static_cast<BatchInst *>(ws.get("batch_inst", sizeof(BatchInst) * L));
-    auto *dslices = static_cast<BatchSlice *>(ws.get("batch_slices", std::max<size_t>(slice_bytes, 16)));
-    auto *dnslices = static_cast<int *>(ws.get("batch_nslices", sizeof(int) * L));
+    auto *dslices = static_cast<BatchSlice *>(ws.get("batch_slices", std::max<size_t>(nslices, 1) * sizeof(BatchSlice)));
     auto *pinst = static_cast<int *>(ws.get("batch_pinst", sizeof(int) * total_prows));
     auto *tinst = static_cast<int *>(ws.get("batch_tinst", sizeof(int) * row_tiles));
     auto *gcnt = static_cast<int *>(ws.get("batch_cnt", sizeof(int) * (total_rows + 1)));
@@ -909,7 +906,7 @@ dl_status solve_tc_batch(dl_ctx *ctx, Workspace &ws, cudaStream_t s, int32_t cou
     auto *scratch = static_cast<int *>(ws.get("batch_scan", sizeof(int) * 2 * (scan_blocks + 1)));
     uint8_t *staging = nullptr;
     if (mem == DL_MEM_HOST) staging = static_cast<uint8_t *>(ws.get("batch_in", std::max<int64_t>(in_bytes, 256)));
-    if (!rb || !mb || !cmask || !ctr || !state || !lists || !dinst || !dslices || !dnslices || !pinst || !tinst ||
+    if (!rb || !mb || !cmask || !ctr || !lists || !dinst || !dslices || !pinst || !tinst ||
         !gcnt || !gptr || !scratch || (mem == DL_MEM_HOST && !staging)) {
         set_error("batch: device allocation failed (%.2f GB of bits)", 16.0 * bit_words / 1e9);
         return DL_ENOMEM;
@@ -939,8 +936,6 @@ dl_status solve_tc_batch(dl_ctx *ctx, Workspace &ws, cudaStream_t s, int32_t cou
         bo += np * (np / 64);
     }
     BCK(cudaMemcpyAsync(dinst, inst.data(), sizeof(BatchInst) * L, cudaMemcpyHostToDevice, s));
-    BCK(cudaMemcpyAsync(dnslices, nslices.data(), sizeof(int) * L, cudaMemcpyHostToDevice, s));
-    if (slice_bytes) BCK(cudaMemcpyAsync(dslices, slices.data(), slice_bytes, cudaMemcpyHostToDevice, s));
 
     // 1. bits of I + E, counts and checks over all inputs, then the CSR row pointers (every
     //    call: the contents, hence the number of facts, may differ between calls)
@@ -949,6 +944,18 @@ dl_status solve_tc_batch(dl_ctx *ctx, Workspace &ws, cudaStream_t s, int32_t cou
     batch_pack_kernel<<<static_cast<unsigned>(row_tiles), 256, tile_smem, s>>>(dinst, tinst, gcnt, ws.status);
     BCK(cudaGetLastError());
     BCK(exclusive_scan_large(gcnt, static_cast<int>(total_rows), gptr, scratch, s));
+    // (the slices with the most work first; listed while the inputs are packed)
+    std::vector<BatchSlice> slices;
+    slices.reserve(nslices);
+    for (int i = 0; i < L; ++i) {
+        const int W = slice_words(inst[i].n);
+        for (int q = 0; q < inst[i].slices; ++q)
+            slices.push_back(BatchSlice{i, q * W, std::min(W, inst[i].wp - q * W)});
+    }
+    std::stable_sort(slices.begin(), slices.end(), [&](const BatchSlice &x, const BatchSlice &y) {
+        return static_cast<int64_t>(x.nw) * inst[x.k].n > static_cast<int64_t>(y.nw) * inst[y.k].n;
+    });
+    if (nslices) BCK(cudaMemcpyAsync(dslices, slices.data(), nslices * sizeof(BatchSlice), cudaMemcpyHostToDevice, s));
     const int pre_launches = 2 + (total_rows > 64 * 1024 ? 3 : 1);
     int nnz_total = 0, hst = 0;
     BCK(cudaMemcpyAsync(&nnz_total, gptr + total_rows, sizeof(int), cudaMemcpyDeviceToHost, s));
@@ -965,8 +972,7 @@ dl_status solve_tc_batch(dl_ctx *ctx, Workspace &ws, cudaStream_t s, int32_t cou
     }
 
     // 2. the successor lists, then every instance's column slices
-    BCK(cudaMemsetAsync(state, 0, sizeof(int) * (L + 1), s));
-    BCK(cudaMemsetAsync(ctr, 0, kCounterArrays * sizeof(unsigned long long) * L, s));
+    BCK(cudaMemsetAsync(ctr, 0, result_bytes, s));
     const unsigned fill_blocks = static_cast<unsigned>((total_prows + 8 * kFillRows - 1) / (8 * kFillRows));
     batch_fill_kernel<<<fill_blocks, 256, 0, s>>>(dinst, pinst, static_cast<int>(total_prows), gptr, gcol);
     int launches = pre_launches + 2;
@@ -976,16 +982,12 @@ dl_status solve_tc_batch(dl_ctx *ctx, Workspace &ws, cudaStream_t s, int32_t cou
             dinst, dslices, gptr, gcol, bc, ws.status);
         ++launches;
     }
-    batch_settle_kernel<<<(L + 255) / 256, 256, 0, s>>>(dnslices, L, bc, state + L);
+    batch_settle_kernel<<<(L + 255) / 256, 256, 0, s>>>(dinst, L, bc, ws.status, state + L);
     BCK(cudaGetLastError());
-    std::vector<int> hstate(L + 1);
-    std::vector<unsigned long long> hctr(kCounterArrays * static_cast<size_t>(L));
+    std::vector<unsigned long long> hctr(result_bytes / sizeof(unsigned long long) + 1);
+    const int *hstate = reinterpret_cast<const int *>(hctr.data() + kCounterArrays * static_cast<size_t>(L));
     auto read_back = [&]() -> cudaError_t {
-        cudaError_t e = cudaMemcpyAsync(hstate.data(), state, sizeof(int) * (L + 1), cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(hctr.data(), ctr, sizeof(unsigned long long) * kCounterArrays * L,
-                                cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(&hst, ws.status, sizeof(int), cudaMemcpyDeviceToHost, s);
+        const cudaError_t e = cudaMemcpyAsync(hctr.data(), ctr, result_bytes, cudaMemcpyDeviceToHost, s);
         return e == cudaSuccess ? cudaStreamSynchronize(s) : e;
     };
     BCK(cudaEventRecord(ev1, s));
@@ -1005,7 +1007,9 @@ dl_status solve_tc_batch(dl_ctx *ctx, Workspace &ws, cudaStream_t s, int32_t cou
                                   cudaMemcpyDeviceToHost, s));
         }
     }
+    hst = hstate[L + 1];
     if (mem == DL_MEM_HOST || hstate[L] != 0) {
+        BCK(cudaMemcpyAsync(&hst, ws.status, sizeof(int), cudaMemcpyDeviceToHost, s));
         BCK(cudaEventRecord(ev1, s));
         BCK(read_back());
     }
