@@ -65,8 +65,11 @@ struct Factor {
 };
 
 // The byte matrices a program's runs work on, kept between them (cudaMalloc and cudaFree of a dozen
-// matrices took 0.9 of a run's 1.4 ms at n = 2048); as many as the largest run needed, freed with the
-// program.  A program's calls are serialised by its context.
+// matrices took 0.9 of a run's 1.4 ms at n = 2048); as many as the largest run needed, up to kStoreBytes
+// in all between runs (larger matrices cost more than their allocation does), freed with the program.  A
+// program's calls are serialised by its context.
+constexpr size_t kStoreBytes = size_t{1} << 30;
+
 struct MatrixStore {
     struct Block {
         void *p;
@@ -352,6 +355,13 @@ struct Pool {
     Pool(const Pool &) = delete;
     ~Pool() {
         for (size_t k : taken) store.blocks[k].used = false;
+        size_t held = 0;
+        for (const auto &b : store.blocks) held += b.bytes;
+        while (held > kStoreBytes && !store.blocks.back().used) {  // (blocks in use keep their places)
+            held -= store.blocks.back().bytes;
+            cudaFree(store.blocks.back().p);
+            store.blocks.pop_back();
+        }
     }
     uint8_t *alloc(size_t bytes) {
         bytes = std::max<size_t>(bytes, 16);
