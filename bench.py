@@ -331,7 +331,7 @@ def bench_batch(ctx, torch, reps: int = 10) -> dict:
         flat[int(o):int(o) + e.size] = e.reshape(-1)
     dev = torch.from_numpy(flat).cuda()
     torch.cuda.synchronize()
-    ctx.tc_batch_flat(dev, ns, offsets)  # captures the graph
+    ctx.tc_batch_flat(dev, ns, offsets)  # sizes the work space
     t0 = time.perf_counter()
     for _ in range(reps):
         _, _, st = ctx.tc_batch_flat(dev, ns, offsets)

@@ -394,13 +394,14 @@ DL_API dl_status dl_program_describe(const dl_program *prog, char *buf, size_t c
  * dl_tc_closure gives (eps <= 0, thr = 0; the program of Sec. 3).  ns[k], Es[k], out_bits[k]
  * describe problem k; all live in `mem`.  Every problem follows the DL_PATH_AUTO scheme:
  * one packing pass over all inputs builds one CSR over all problems' rows (one host read
- * sizes it), then a captured CUDA graph runs problems of at most 1024 padded rows to their
- * fixpoint in shared memory (one CTA each), batched in-place Iteration sweeps (Sec. 7.1) over
+ * sizes it); the columns of every problem of at most 4096 constants are closed in slices in
+ * shared memory (one CTA each).  Problems with a slice still changing after 64 sweeps, and
+ * larger ones, go on in a captured CUDA graph: batched in-place Iteration sweeps (Sec. 7.1) over
  * the rows of every problem still changing, and rounds of one persistent grouped FP8
  * tensor-core squaring launch over exactly the problems still active, each followed by more
  * sweeps; a problem leaves the active lists when a sweep changes nothing, and its model and
  * certificate are written then.  A second captured graph with further rounds runs only if a
- * problem is still active after the first.  Every decision is taken on the device.
+ * problem is still active after the first.
  * stats (optional, one for the whole batch): iters = squaring rounds launched.
  */
 DL_API dl_status dl_tc_batch(dl_ctx *ctx, int32_t count, const int32_t *ns, const uint8_t *const *Es,
