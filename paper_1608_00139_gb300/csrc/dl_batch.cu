@@ -242,7 +242,7 @@ __device__ __forceinline__ void or2(ulonglong2 &a, const ulonglong2 &b) {
 }
 
 // The sweeps and the model of one slice (see above); Col: uint16_t (shared) or int (global).
-template <class Col>
+template <int kMaxSweeps, class Col>
 __device__ __forceinline__ void close_slice(const BatchInst &I, int k, int w0, int nw, ulonglong2 *M, const int *rp,
                                             uint8_t *stamp, const Col *__restrict__ col, ulonglong2 cm, int G,
                                             BatchCounters c, int *status, unsigned *ones_s) {
@@ -257,7 +257,7 @@ __device__ __forceinline__ void close_slice(const BatchInst &I, int k, int w0, i
     };
     int t = 1;
     bool conv = false;
-    for (; t <= kSliceSweeps; ++t) {
+    for (; t <= kMaxSweeps; ++t) {
         bool ch = false;
         for (int r = r0; r < n && lv; r += dr) {
             ulonglong2 acc = M[r * nv + l];
@@ -288,7 +288,7 @@ __device__ __forceinline__ void close_slice(const BatchInst &I, int k, int w0, i
             break;
         }
     }
-    if (threadIdx.x == 0) atomicMax(&c.sweeps[k], static_cast<unsigned long long>(min(t, kSliceSweeps)));
+    if (threadIdx.x == 0) atomicMax(&c.sweeps[k], static_cast<unsigned long long>(min(t, kMaxSweeps)));
     if (!conv) {
         for (int r = r0; r < n && lv; r += dr)
             *reinterpret_cast<ulonglong2 *>(I.rbits + static_cast<int64_t>(r) * I.wp + wl) = M[r * nv + l];
@@ -331,14 +331,12 @@ __device__ __forceinline__ void close_slice(const BatchInst &I, int k, int w0, i
     }
 }
 
-__global__ void __launch_bounds__(kSliceThreads)
-    batch_slice_kernel(const BatchInst *__restrict__ inst, const BatchSlice *__restrict__ slices,
-                       const int *__restrict__ ptr, const int *__restrict__ col, BatchCounters c, int *status) {
+template <int kMaxSweeps>
+__device__ __forceinline__ void run_slice(const BatchInst I, const BatchSlice S, const int *__restrict__ ptr,
+                                          const int *__restrict__ col, const BatchCounters c, int *status) {
     extern __shared__ __align__(16) unsigned char slice_smem[];
     __shared__ uint64_t cm_s[16];
     __shared__ unsigned ones_s;
-    const BatchSlice S = slices[blockIdx.x];
-    const BatchInst I = inst[S.k];
     const int n = I.n, nv = S.nw >> 1;
     auto *M = reinterpret_cast<ulonglong2 *>(slice_smem);  // n x nv
     auto *rp = reinterpret_cast<int *>(M + n * nv);        // n + 1 row pointers
@@ -379,8 +377,27 @@ __global__ void __launch_bounds__(kSliceThreads)
         for (int q = threadIdx.x; q < nnz; q += kSliceThreads) scol[q] = static_cast<uint16_t>(col[base + q]);
     __syncthreads();
     if (l < nv) cm = make_ulonglong2(cm_s[2 * l], cm_s[2 * l + 1]);
-    if (fits) close_slice(I, S.k, S.w0, S.nw, M, rp, stamp, scol, cm, G, c, status, &ones_s);
-    else close_slice(I, S.k, S.w0, S.nw, M, rp, stamp, col + base, cm, G, c, status, &ones_s);
+    if (fits) close_slice<kMaxSweeps>(I, S.k, S.w0, S.nw, M, rp, stamp, scol, cm, G, c, status, &ones_s);
+    else close_slice<kMaxSweeps>(I, S.k, S.w0, S.nw, M, rp, stamp, col + base, cm, G, c, status, &ones_s);
+}
+
+__global__ void __launch_bounds__(kSliceThreads)
+    batch_slice_kernel(const BatchInst *__restrict__ inst, const BatchSlice *__restrict__ slices,
+                       const int *__restrict__ ptr, const int *__restrict__ col, BatchCounters c, int *status) {
+    const BatchSlice S = slices[blockIdx.x];
+    const BatchInst I = inst[S.k];
+    run_slice<kSliceSweeps>(I, S, ptr, col, c, status);
+}
+
+// One closure, two words to a slice: as many CTAs as there are.
+constexpr int kSingleWords = 2;
+constexpr int kSingleSweeps = 32;
+
+__global__ void __launch_bounds__(kSliceThreads)
+    single_slice_kernel(BatchInst I, const int *__restrict__ ptr, const int *__restrict__ col, BatchCounters c,
+                        int *status) {
+    const BatchSlice S{0, static_cast<int>(blockIdx.x) * kSingleWords, kSingleWords};
+    run_slice<kSingleSweeps>(I, S, ptr, col, c, status);
 }
 
 // After the slices: an instance all of whose slices are done is done, the others start over as
@@ -677,6 +694,26 @@ void launch_rows(int wpl, int grid, const BatchInst *d, const BatchList &l, cons
 }
 
 }  // namespace
+
+int close_slices_count(int n, int64_t wp) {
+    const int64_t bytes = static_cast<int64_t>(n) * (8 * kSingleWords + 5) + 16;  // M, row pointers, stamps
+    return n > 0 && n < 65536 && wp % kSingleWords == 0 && bytes <= kSliceSmem ? static_cast<int>(wp / kSingleWords) : 0;
+}
+
+cudaError_t close_slices(const int *ptr, const int *col, int n, int64_t wp, uint64_t *M, uint64_t *model,
+                         unsigned long long *counters, int *status, cudaStream_t s) {
+    BatchInst I{};
+    I.rbits = M;
+    I.mbits = model;
+    I.n = n;
+    I.wp = static_cast<int32_t>(wp);
+    const BatchCounters c{nullptr, counters, nullptr, counters + 1, nullptr, counters + 2};
+    cudaError_t e = cudaFuncSetAttribute(single_slice_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSliceSmem);
+    if (e != cudaSuccess) return e;
+    single_slice_kernel<<<static_cast<unsigned>(close_slices_count(n, wp)), kSliceThreads, kSliceSmem, s>>>(
+        I, ptr, col, c, status);
+    return cudaGetLastError();
+}
 
 // Cached schedule of the last batch (graph, the sizes and the work space it was built on).
 struct BatchPlan {

@@ -159,6 +159,13 @@ dl_status solve_transposed(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const Sol
 dl_status solve_sg_real(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &a, dl_stats *st);
 dl_status solve_compose(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &a,
                         dl_stats *st);
+// One closure by column slices in shared memory (dl_batch.cu): from bits M between I + E and the reflexive
+// closure to the model E M* (stride wp, certified; status on a failed certificate), counters[0] += slices
+// done, [1] += ones of the model, [2] = most sweeps.  A slice that still changes after 32 sweeps
+// writes its bits back to M.  close_slices_count: the slices, 0 where they do not fit.
+int close_slices_count(int n, int64_t wp);
+cudaError_t close_slices(const int *ptr, const int *col, int n, int64_t wp, uint64_t *M, uint64_t *model,
+                         unsigned long long *counters, int *status, cudaStream_t s);
 dl_status solve_tc_batch(dl_ctx *ctx, Workspace &ws, cudaStream_t s, int32_t count,
                          const int32_t *ns, const uint8_t *const *Es, dl_mem mem,
                          uint64_t *const *out_bits, dl_stats *st);

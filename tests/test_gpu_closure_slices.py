@@ -1,0 +1,39 @@
+"""Single closures that go on in column slices after the speculative sweeps: sizes around the words of
+a slice, graphs whose slices all finish, some or none, and the size where slices no longer fit.
+Models equal the oracle's bits (whole numbers: no tolerance)."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_1608_00139_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+
+def half_chain(n, seed):
+    e = inputs.er_digraph(n, 1.4 / n, seed)
+    e[:, n // 2:] = 0
+    e[n // 2:, :] = 0
+    at = np.arange(n // 2, n - 1)
+    e[at, at + 1] = 1
+    return e
+
+
+CASES = [("er", n, d) for n in (5249, 5377, 6000, 7937) for d in (1.2, 2.0)] + [
+    ("half", 6001, 0), ("er", 10700, 1.5), ("er", 10800, 1.5)]
+
+
+@pytest.mark.parametrize("kind,n,d", CASES)
+def test_sparse_closures_above_one_fact_per_row(ctx, kind, n, d):
+    oracle.set_threads(0)
+    e = half_chain(n, n) if kind == "half" else inputs.er_digraph(n, d / n, n)
+    e[n - 1, n - 1] = e[5, 5] = 1
+    ref = oracle.tc_model(e)
+    ones = int(np.unpackbits(ref.view(np.uint8)).sum())
+    dev = torch.from_numpy(e).cuda()
+    for _ in range(2):
+        out, st = ctx.tc_closure(dev)[:2]
+        assert np.array_equal(out.cpu().numpy().view(np.uint64), ref) and st["model_ones"] == ones
+    out, st = ctx.tc_closure(e)[:2]
+    assert np.array_equal(out, ref) and st["model_ones"] == ones
