@@ -704,7 +704,14 @@ cudaError_t close_slices(const int *ptr, const int *col, int n, int64_t wp, uint
                          unsigned long long *counters, int *status, cudaStream_t s) {
     BatchInst I{};
     I.rbits = M;
-    I.mbits = model;
+    // 16-byte stores where they are aligned; a caller's output need only be aligned to its 8-byte words
+    // (it has no padding words then)
+    if ((reinterpret_cast<uintptr_t>(model) & 15) == 0) {
+        I.mbits = model;
+    } else {
+        if ((n + 63) / 64 != wp) return cudaErrorInvalidValue;
+        I.out = model;
+    }
     I.n = n;
     I.wp = static_cast<int32_t>(wp);
     const BatchCounters c{nullptr, counters, nullptr, counters + 1, nullptr, counters + 2};

@@ -37,3 +37,20 @@ def test_sparse_closures_above_one_fact_per_row(ctx, kind, n, d):
         assert np.array_equal(out.cpu().numpy().view(np.uint64), ref) and st["model_ones"] == ones
     out, st = ctx.tc_closure(e)[:2]
     assert np.array_equal(out, ref) and st["model_ones"] == ones
+
+
+@pytest.mark.parametrize("n", [6081, 6144])
+def test_output_aligned_to_its_words_only(ctx, n):
+    """The model straight into a caller's output that starts 8 bytes into a buffer (rows of as many words
+    as the workspace's: n in (np - 64, np]); the words around it stay as they were."""
+    oracle.set_threads(0)
+    e = inputs.er_digraph(n, 2.0 / n, n)
+    ref = oracle.tc_model(e)
+    w = ref.shape[1]
+    buf = torch.full((n * w + 2,), -3, dtype=torch.int64, device="cuda")
+    out = buf[1:1 + n * w].view(n, w)
+    assert out.data_ptr() % 16 == 8
+    _, st = ctx.tc_closure(torch.from_numpy(e).cuda(), out=out)
+    assert np.array_equal(out.cpu().numpy().view(np.uint64), ref)
+    assert st["model_ones"] == int(np.unpackbits(ref.view(np.uint8)).sum())
+    assert int(buf[0]) == -3 and int(buf[-1]) == -3
