@@ -54,7 +54,7 @@ struct SmallState {
     int dmax[kMaxCluster];
     unsigned acc[3];                       // ... of this CTA
     unsigned probe[kMaxCluster][2], probe_acc[2];  // rows changing and ones at step kProbe
-    int dmax_s, bad_s;
+    int dmax_s, bad_s;                     // bad_s: written by thread 0 alone
 };
 
 // A 64-bit word of the shared memory of CTA `rank` at this CTA's address p.
@@ -118,7 +118,7 @@ __global__ void __launch_bounds__(kSmallThreads)
     if (tid < 32) st.colmask[tid] = 0ull;
     if (tid < 3) st.acc[tid] = 0u;
     if (tid < 2) st.probe_acc[tid] = 0u;
-    if (tid == 0) st.dmax_s = st.bad_s = 0;
+    if (tid == 0) st.dmax_s = 0;
     bool bad = false;
     uint32_t bad_kind = 0;
     // ---- the rows of E as bits ---------------------------------------------------------------
@@ -151,8 +151,9 @@ __global__ void __launch_bounds__(kSmallThreads)
         }
         bad_kind = ST_BAD_PAD;
     }
-    if (bad) st.bad_s = static_cast<int>(bad_kind);
-    __syncthreads();
+    // (the flag has one writer: a store of every thread that met a bad byte would race with its zeroing)
+    const int any_bad = __syncthreads_or(bad);
+    if (tid == 0) st.bad_s = any_bad ? static_cast<int>(bad_kind) : 0;
     // ---- M = I | E, the successor lists, the columns with a fact --------------------------------
     const int grp = lane / G, lw = lane % G, per_warp = 32 / G;
     const unsigned gmask = G == 32 ? kAll : ((1u << G) - 1u) << (grp * G);

@@ -77,3 +77,32 @@ def test_bad_input(ctx, n):
         ctx.tc_closure(e, eps=2.0)
     assert err.value.status == dl.DL_EINVAL
     assert np.array_equal(ctx.tc_closure(e)[0], oracle.tc_model(e))
+
+
+@pytest.mark.parametrize("n", [40, 128, 300, 1000])
+def test_bad_input_of_any_row_is_seen(ctx, n):
+    """One bad byte (or padding bit) in a row of every warp and CTA, many calls each: the flag is a
+    vote of the whole CTA, whichever warp runs first."""
+    e = torch.from_numpy(relation("sparse", n)).cuda()
+    packed = torch.from_numpy(oracle.pack(relation("sparse", n)).view(np.int64)).cuda()
+    for i in range(0, n, max(1, n // 40)):
+        for j in (0, n - 1):
+            was = int(e[i, j])
+            e[i, j] = 2 + i % 250
+            for _ in range(3):
+                with pytest.raises(dl.DLError) as err:
+                    ctx.tc_closure(e)
+                assert err.value.status == dl.DL_EINVAL, (i, j)
+            e[i, j] = was
+        if n % 64 == 0:
+            continue  # no padding bits
+        was = int(packed[i, -1])
+        packed[i, -1] = was | -(1 << 63)
+        for _ in range(3):
+            with pytest.raises(dl.DLError) as err:
+                ctx.tc_closure_bits(packed, n)
+            assert err.value.status == dl.DL_EINVAL, i
+        packed[i, -1] = was
+    want = oracle.tc_model(relation("sparse", n))
+    assert np.array_equal(ctx.tc_closure(e)[0].cpu().numpy().view(np.uint64), want)
+    assert np.array_equal(ctx.tc_closure_bits(packed, n)[0].cpu().numpy().view(np.uint64), want)
