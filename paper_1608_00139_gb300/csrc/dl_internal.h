@@ -35,6 +35,20 @@ enum : int {
     ST_BAD_PAD = 128,          // a bit-packed input row had a bit at a column >= n
 };
 
+// Lets a kernel be launched with all the dynamic shared memory that a block can have beside its static one.
+// The limit belongs to the kernel, and the contexts and serving slots of a process share it: set to one
+// call's need, it could be lowered between another thread's setting and its launch, which then fails.  So
+// it is only ever set to this one value.
+template <class Kernel>
+inline cudaError_t allow_all_smem(Kernel *kernel) {
+    constexpr int kBlockSmem = 232448;  // 227 KB
+    cudaFuncAttributes at;
+    const cudaError_t e = cudaFuncGetAttributes(&at, kernel);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                kBlockSmem - static_cast<int>(at.sharedSizeBytes));
+}
+
 // ---------------------------------------------------------------------------------------
 // tcgen05 GEMM (dl_umma.cu)
 // ---------------------------------------------------------------------------------------

@@ -1459,7 +1459,7 @@ dl_status tc_mixed(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &
         set_error("mixed path: n = %d exceeds the refinement's shared-memory row (%zu bytes)", n, row_smem);
         return DL_EINVAL;
     }
-    MCK(cudaFuncSetAttribute(first_fix_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(row_smem)));
+    MCK(allow_all_smem(first_fix_kernel));
     // the residual kernel by density: rows of Zf per block for sparse E, bucketed bands otherwise
     const bool banded = static_cast<int64_t>(nnz) >= 32ll * n;
     const int rows_per_block = static_cast<int>(std::min<size_t>(3, (227 * 1024) / row_smem));
@@ -1492,10 +1492,9 @@ dl_status tc_mixed(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &
             return DL_EDEVICE;
         }
     } else {
-        const int smem = static_cast<int>(row_smem * rows_per_block);
-        MCK(cudaFuncSetAttribute(residual_rows_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        MCK(cudaFuncSetAttribute(residual_rows_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        MCK(cudaFuncSetAttribute(residual_rows_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        MCK(allow_all_smem(residual_rows_kernel<1>));
+        MCK(allow_all_smem(residual_rows_kernel<2>));
+        MCK(allow_all_smem(residual_rows_kernel<3>));
     }
     const uint8_t *rhs_t = nullptr;  // A^T, set below for the general right-hand side
     auto residual = [&](unsigned *rmax_p) -> cudaError_t {
@@ -1532,17 +1531,10 @@ dl_status tc_mixed(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &
     const int rows_q = 4 * q_smem <= 227 * 1024 ? 4 : 2;
     if (slices) {
         MCK(gemm_prepare(KIND_F16, true, 256, EPI_STORE_F32));
-        MCK(cudaFuncSetAttribute(refine_add_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 static_cast<int>(q_smem)));
+        MCK(allow_all_smem(refine_add_kernel<true>));
     } else if (need_x) {
-        MCK(cudaFuncSetAttribute(refine_add_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 static_cast<int>(q_smem)));
-        if (rows_q == 4)
-            MCK(cudaFuncSetAttribute(update_rows_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     static_cast<int>(4 * q_smem)));
-        else
-            MCK(cudaFuncSetAttribute(update_rows_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     static_cast<int>(2 * q_smem)));
+        MCK(allow_all_smem(refine_add_kernel<false>));
+        MCK(rows_q == 4 ? allow_all_smem(update_rows_kernel<4>) : allow_all_smem(update_rows_kernel<2>));
     }
     auto first_fix = [&](const float *D) -> cudaError_t {
         first_fix_kernel<<<static_cast<unsigned>(np), 256, row_smem, s>>>(Z64, D, n, N, deg_bits, min_hb,

@@ -499,22 +499,19 @@ cudaError_t sg_real_step(const int *ptr, const int *col, int n, int np, double e
                          double *U, double *Xn, float *R, unsigned long long *dmax, bool fused, cudaStream_t s) {
     const size_t smem = sizeof(double) * static_cast<size_t>(np);
     if (fused && np <= 4096) {
-        cudaError_t e = cudaFuncSetAttribute(sg_fused_kernel<512, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             static_cast<int>(smem));
+        cudaError_t e = allow_all_smem(sg_fused_kernel<512, 8>);
         if (e != cudaSuccess) return e;
         sg_fused_kernel<512, 8><<<static_cast<unsigned>(np), 512, smem, s>>>(ptr, col, n, np, eps, B, X, Xn, R, dmax);
         return cudaGetLastError();
     }
     if (fused) {
-        cudaError_t e = cudaFuncSetAttribute(sg_fused_kernel<1024, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             static_cast<int>(smem));
+        cudaError_t e = allow_all_smem(sg_fused_kernel<1024, 16>);
         if (e != cudaSuccess) return e;
         sg_fused_kernel<1024, 16><<<static_cast<unsigned>(np), 1024, smem, s>>>(ptr, col, n, np, eps, B, X, Xn, R,
                                                                                dmax);
         return cudaGetLastError();
     }
-    cudaError_t e = cudaFuncSetAttribute(sg_xpt_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(smem));
+    cudaError_t e = allow_all_smem(sg_xpt_kernel);
     if (e != cudaSuccess) return e;
     sg_xpt_kernel<<<static_cast<unsigned>(np), 256, smem, s>>>(ptr, col, n, np, X, U);
     dim3 grid(static_cast<unsigned>((np + 255) / 256), static_cast<unsigned>(np));
@@ -567,8 +564,7 @@ cudaError_t trans_local(const int *ptr, const int *col, int n, int np, T eps, co
     if (row * g > limit) return cudaErrorInvalidValue;
     auto launch = [&](auto *kernel) -> cudaError_t {
         const size_t smem = row * g;
-        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   static_cast<int>(smem));
+        const cudaError_t e = allow_all_smem(kernel);
         if (e != cudaSuccess) return e;
         kernel<<<static_cast<unsigned>(np / g), 512, smem, s>>>(ptr, col, n, np, eps, X, RT, Y, skip);
         return cudaGetLastError();
@@ -638,8 +634,7 @@ cudaError_t trans_last_step(const int *ptr, const int *col, int n, int np, doubl
 cudaError_t trans_finish(const int *rank, int n, int np, int64_t wp, const double *X, double *out, uint64_t *bits,
                          cudaStream_t s) {
     const size_t smem = static_cast<size_t>(n) * sizeof(double);
-    const cudaError_t e = cudaFuncSetAttribute(trans_finish_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               static_cast<int>(smem));
+    const cudaError_t e = allow_all_smem(trans_finish_kernel);
     if (e != cudaSuccess) return e;
     trans_finish_kernel<<<static_cast<unsigned>(n), 512, smem, s>>>(rank, n, np, static_cast<int>(wp), X, out,
                                                                     reinterpret_cast<uint32_t *>(bits));

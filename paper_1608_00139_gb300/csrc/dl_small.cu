@@ -371,6 +371,9 @@ __global__ void __launch_bounds__(kSmallThreads)
     }
 }
 
+// (within the 48 KB that every kernel may have: no limit to raise)
+static_assert(2 * 128 * 16 * 8 + 128 * (kListCap + 1) * 2 + sizeof(SmallState) + 16 <= 48 * 1024, "n = 1024: R = 128, w = 16");
+
 template <int C>
 cudaError_t launch_small(const uint8_t *E, const uint64_t *Eb, int n, int logR, uint64_t *out, SmallClosure *result,
                          cudaStream_t s) {
@@ -379,9 +382,6 @@ cudaError_t launch_small(const uint8_t *E, const uint64_t *Eb, int n, int logR, 
     while (G < w) G <<= 1;
     const size_t smem = static_cast<size_t>(2 * R * w) * 8 + static_cast<size_t>(R) * (kListCap + 1) * 2 +
                         sizeof(SmallState) + 16;
-    cudaError_t e = cudaFuncSetAttribute(closure_small_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(smem));
-    if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(C);
     cfg.blockDim = dim3(kSmallThreads);
