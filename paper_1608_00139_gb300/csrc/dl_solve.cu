@@ -442,8 +442,7 @@ dl_status tc_small(Workspace &ws, cudaStream_t s, const SolveArgs &a, dl_stats *
     tm.mark(1);
     CK(closure_small(E, Eb, n, model, r, s));
     tm.mark(2);
-    if (a.mem != DL_MEM_DEVICE) CK(cudaMemcpyAsync(a.out_bits, model, out_bytes, cudaMemcpyDeviceToHost, s));
-    tm.mark(3);
+    if (a.mem == DL_MEM_DEVICE) tm.mark(3);
     CK(cudaStreamSynchronize(s));
     if ((rc = status_error(r->status))) return rc;
     double eps = 0;
@@ -452,6 +451,11 @@ dl_status tc_small(Workspace &ws, cudaStream_t s, const SolveArgs &a, dl_stats *
     if (r->violations != 0) {
         set_error("internal: converged closure failed its certificate");
         return DL_EDEVICE;
+    }
+    if (a.mem != DL_MEM_DEVICE) {  // (host memory is written only by a call that succeeds)
+        CK(cudaMemcpyAsync(a.out_bits, model, out_bytes, cudaMemcpyDeviceToHost, s));
+        tm.mark(3);
+        CK(cudaStreamSynchronize(s));
     }
     if (st) {
         st->path_used = DL_PATH_AUTO;

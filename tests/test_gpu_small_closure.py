@@ -106,3 +106,35 @@ def test_bad_input_of_any_row_is_seen(ctx, n):
     want = oracle.tc_model(relation("sparse", n))
     assert np.array_equal(ctx.tc_closure(e)[0].cpu().numpy().view(np.uint64), want)
     assert np.array_equal(ctx.tc_closure_bits(packed, n)[0].cpu().numpy().view(np.uint64), want)
+
+
+@pytest.mark.parametrize("n", [100, 300, 1000])
+def test_refused_calls_leave_host_memory_alone(ctx, n):
+    """Bad bytes, padding bits and eps: the caller's output is as it was (an earlier query's model is in
+    the workspace)."""
+    good = relation("sparse", n)
+    ctx.tc_closure(good)
+    out = np.full((n, dl.words(n)), 0x5A5A5A5A5A5A5A5A, np.uint64)
+    before = out.copy()
+    bad = good.copy()
+    bad[n // 2, n - 1] = 2
+    padded = oracle.pack(good).copy()
+    padded[n - 1, -1] |= np.uint64(1) << np.uint64(63)
+    for call in (lambda: ctx.tc_closure(bad, out=out), lambda: ctx.tc_closure_bits(padded, n, out=out),
+                 lambda: ctx.tc_closure(good, eps=2.0, out=out)):
+        with pytest.raises(dl.DLError) as err:
+            call()
+        assert err.value.status == dl.DL_EINVAL
+        assert np.array_equal(out, before)
+    ctx.tc_closure(good, out=out)
+    assert np.array_equal(out, oracle.tc_model(good))
+
+
+@pytest.mark.parametrize("kind,n", [("sparse", 300), ("chain", 512), ("chain", 1000)])
+def test_packed_host_rows_in_place(ctx, kind, n):
+    """The output over the input, also where a long path is handed to the general route."""
+    e = relation(kind, n)
+    ctx.tc_closure(relation("dense", n))
+    rows = oracle.pack(e).copy()
+    ctx.tc_closure_bits(rows, n, out=rows)
+    assert np.array_equal(rows, oracle.tc_model(e))
