@@ -451,10 +451,14 @@ cudaError_t csr_build(const uint8_t *E, int n, int *cnt, int *ptr, cudaStream_t 
     return cudaGetLastError();
 }
 
-// Shared memory beyond 48 KB (rows of more than 190 000 columns) is asked for.
+// Shared memory beyond 48 KB, the kernels' static part (less than kTileStatic) included, is asked for: rows of
+// more than some 192 000 columns.
+constexpr size_t kTileStatic = 1024;
+static_assert(sizeof(int) * (kTileRows + 1) <= kTileStatic, "csr_pack_check_kernel's counts");
+
 template <class Kernel>
 static cudaError_t tile_smem(Kernel kernel, size_t smem) {
-    if (smem <= 48 * 1024) return cudaSuccess;
+    if (smem + kTileStatic <= 48 * 1024) return cudaSuccess;
     return allow_all_smem(kernel);
 }
 
