@@ -471,6 +471,7 @@ cudaError_t csr_pack_checked(const uint8_t *E, int n, int np, int64_t wp, int *c
     if (const cudaError_t e = tile_smem(csr_pack_check_kernel, smem)) return e;
     csr_pack_check_kernel<<<static_cast<unsigned>((np + R - 1) / R), 256, smem, s>>>(
         E, n, np, static_cast<int>(wp), R, cnt, M, dmax, nnz, diag, status, colmask);
+    if (const cudaError_t e = cudaGetLastError()) return e;  // (nothing may follow on counts that were not written)
     return launch_programmatic(exclusive_scan_kernel, dim3(1), dim3(1024), 0, s, static_cast<const int *>(cnt), n, ptr);
 }
 
@@ -481,6 +482,7 @@ cudaError_t bits_ingest_checked(const uint64_t *Eb, int n, int np, int64_t wp, i
     const size_t smem = static_cast<size_t>(wp) * sizeof(uint64_t);
     bits_ingest_check_kernel<<<static_cast<unsigned>((np + 7) / 8), 256, smem, s>>>(
         Eb, n, np, static_cast<int>(wp), cnt, M, dmax, nnz, diag, status, colmask);
+    if (const cudaError_t e = cudaGetLastError()) return e;
     return launch_programmatic(exclusive_scan_kernel, dim3(1), dim3(1024), 0, s, static_cast<const int *>(cnt), n, ptr);
 }
 
