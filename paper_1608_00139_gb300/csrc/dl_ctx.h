@@ -29,6 +29,7 @@ struct Workspace {
     struct Buf {
         void *p = nullptr;
         size_t bytes = 0;
+        bool spare = false;  // may be freed when another buffer finds no room
     };
     std::map<std::string, Buf> bufs;
     void *host_pinned = nullptr;  // small pinned staging for scalars and GEMM tables
@@ -62,6 +63,9 @@ struct Workspace {
     void release();
     // device buffer of at least `bytes` (contents undefined); nullptr on failure
     void *get(const std::string &name, size_t bytes);
+    // Buffer `name` is not needed until it is got again: a get() that finds no room may free it.
+    void spare(const std::string &name);
+    bool drop_spares();  // frees them; whether there were any
     // bytes held by buffer `name` (0 if it does not exist)
     size_t capacity(const std::string &name) const;
     size_t footprint() const;

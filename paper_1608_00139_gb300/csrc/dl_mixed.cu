@@ -372,14 +372,15 @@ __device__ __forceinline__ float residual_entry(long long &sum, long long z, int
 }
 
 // (1) Sparse E: G rows j of Zf per block in shared memory, a thread per row i walking its
-// successors (few gathers per row; Zf is read once).  rhs_t is A^T (the threads of a warp read 32
-// entries of a row of it; A's own entries, one in each of 32 rows, took half of the kernel's 0.97 ms).
+// successors (few gathers per row; Zf is read once).  rhs is A^T with rhs_transposed (the threads of a warp
+// read 32 entries of a row of it; A's own entries, one in each of 32 rows, took half of the kernel's 0.97
+// ms; they are read where there was no room for A^T).  S (optional): the sums.
 template <int G>
 __global__ void __launch_bounds__(1024, 1)
     residual_rows_kernel(const int *__restrict__ ptr, const int *__restrict__ col, int n, int np, long long eps_q,
                          const int *__restrict__ escale, const long long *__restrict__ Zf, float *__restrict__ R,
-                         long long *__restrict__ S, unsigned *rmax, const uint8_t *__restrict__ rhs_t,
-                         const double *__restrict__ rhsr) {
+                         long long *__restrict__ S, unsigned *rmax, const uint8_t *__restrict__ rhs,
+                         bool rhs_transposed, const double *__restrict__ rhsr) {
     extern __shared__ long long zi[];  // G rows of np
     const int j0 = blockIdx.x * G;
 #pragma unroll
@@ -424,9 +425,9 @@ __global__ void __launch_bounds__(1024, 1)
             if (j >= np) break;
             float r = 0.0f;
             if (i < n && j < n)
-                r = residual_entry(sum[g], zi[g * np + i], i, j, n, e[g], eps_q, inv[g], rhs_t, rhsr, true);
+                r = residual_entry(sum[g], zi[g * np + i], i, j, n, e[g], eps_q, inv[g], rhs, rhsr, rhs_transposed);
             R[static_cast<int64_t>(j) * np + i] = r;
-            S[static_cast<int64_t>(j) * np + i] = sum[g];
+            if (S != nullptr) S[static_cast<int64_t>(j) * np + i] = sum[g];
             m = fmaxf(m, fabsf(r));
         }
     }
@@ -606,6 +607,7 @@ __global__ void __launch_bounds__(32 * kRWarps, 1)
             m = fmaxf(m, fabsf(v4[u]));
         }
         *reinterpret_cast<float4 *>(rrow + il) = make_float4(v4[0], v4[1], v4[2], v4[3]);
+        if (S == nullptr) continue;
         longlong2 *srow = reinterpret_cast<longlong2 *>(S + static_cast<int64_t>(j) * np + i0 + il);
         srow[0] = make_longlong2(acc[il], acc[il + 1]);
         srow[1] = make_longlong2(acc[il + 2], acc[il + 3]);
@@ -615,13 +617,13 @@ __global__ void __launch_bounds__(32 * kRWarps, 1)
     if (lane == 0 && m > 0.0f) atomicMax(rmax, __float_as_uint(m));
 }
 
-// Z = D for row j (the first product; with D == nullptr Z stays; one block per row, the row kept in
-// shared memory), then the row's scale e_j = row_scale(largest exponent field, deg_bits, min_hb)
+// Z = D for row j (the first product; with add Z += D, with D == nullptr Z stays; one block per row, the row
+// kept in shared memory), then the row's scale e_j = row_scale(largest exponent field, deg_bits, min_hb)
 // into escale[j] (min_hb: a real right-hand side's terms are below 2^min_hb too) and the
 // fixed-point row Zf[j][k] = round(Z[j][k] 2^e_j), plus 2^e_j at k = j < n when add_identity (the
 // closure's [k = j] term of the residual).
-__global__ void __launch_bounds__(256) first_fix_kernel(double *__restrict__ Z, const float *__restrict__ D, int n,
-                                                        int np, int deg_bits, int min_hb, int add_identity,
+__global__ void __launch_bounds__(256) first_fix_kernel(double *__restrict__ Z, const float *__restrict__ D, bool add,
+                                                        int n, int np, int deg_bits, int min_hb, int add_identity,
                                                         int *__restrict__ escale, long long *__restrict__ Zf) {
     // (Zf == nullptr: only Z and escale; fix_transpose_kernel then writes the transposed copy)
     extern __shared__ double zrow_s[];
@@ -635,6 +637,12 @@ __global__ void __launch_bounds__(256) first_fix_kernel(double *__restrict__ Z, 
             const float4 d = *reinterpret_cast<const float4 *>(D + base + k);
             z0 = make_double2(static_cast<double>(d.x), static_cast<double>(d.y));
             z1 = make_double2(static_cast<double>(d.z), static_cast<double>(d.w));
+            if (add) {
+                const double2 a0 = *reinterpret_cast<const double2 *>(Z + base + k);
+                const double2 a1 = *reinterpret_cast<const double2 *>(Z + base + k + 2);
+                z0 = make_double2(a0.x + z0.x, a0.y + z0.y);
+                z1 = make_double2(a1.x + z1.x, a1.y + z1.y);
+            }
             *reinterpret_cast<double2 *>(Z + base + k) = z0;
             *reinterpret_cast<double2 *>(Z + base + k + 2) = z1;
         } else {
@@ -1448,9 +1456,9 @@ dl_status tc_mixed(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &
     auto *gscale = static_cast<int *>(ws.get("mx_gscale", np * 4));
     auto *Zf = static_cast<long long *>(ws.get("mx_Zf", np * np * 8));
     const bool need_x = a.out_rtilde != nullptr;  // (see the refinement loop below)
-    // the exact sums E Z + right-hand side, kept from the first residual on
-    auto *S64 = need_x ? static_cast<long long *>(ws.get("mx_S", np * np * 8)) : Zf;
-    if (!escale || !gscale || !Zf || !S64) {
+    // the exact sums E Z + right-hand side, kept from the first residual on (allocated last, below)
+    long long *S64 = nullptr;
+    if (!escale || !gscale || !Zf) {
         set_error("mixed path: device allocation failed (row scales)");
         return DL_ENOMEM;
     }
@@ -1496,7 +1504,7 @@ dl_status tc_mixed(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &
         MCK(allow_all_smem(residual_rows_kernel<2>));
         MCK(allow_all_smem(residual_rows_kernel<3>));
     }
-    const uint8_t *rhs_t = nullptr;  // A^T, set below for the general right-hand side
+    const uint8_t *rhs_t = nullptr;  // A^T, set below for the general right-hand side (if there is room)
     auto residual = [&](unsigned *rmax_p) -> cudaError_t {
         if (banded) {
             dim3 tgrid(static_cast<unsigned>(np / TT), static_cast<unsigned>(np / TT));
@@ -1509,19 +1517,20 @@ dl_status tc_mixed(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &
         const unsigned grid = static_cast<unsigned>((np + rows_per_block - 1) / rows_per_block);
         const size_t smem = row_smem * rows_per_block;
         if (rows_per_block == 3)
-            residual_rows_kernel<3><<<grid, 1024, smem, s>>>(csr_ptr, csr_col, n, N, eps_q, escale, Zf, R32, S64, rmax_p, rhs_t,
-                                                             a.rhs_real);
+            residual_rows_kernel<3><<<grid, 1024, smem, s>>>(csr_ptr, csr_col, n, N, eps_q, escale, Zf, R32, S64, rmax_p,
+                                                             rhs_t ? rhs_t : a.rhs, rhs_t != nullptr, a.rhs_real);
         else if (rows_per_block == 2)
-            residual_rows_kernel<2><<<grid, 1024, smem, s>>>(csr_ptr, csr_col, n, N, eps_q, escale, Zf, R32, S64, rmax_p, rhs_t,
-                                                             a.rhs_real);
+            residual_rows_kernel<2><<<grid, 1024, smem, s>>>(csr_ptr, csr_col, n, N, eps_q, escale, Zf, R32, S64, rmax_p,
+                                                             rhs_t ? rhs_t : a.rhs, rhs_t != nullptr, a.rhs_real);
         else
-            residual_rows_kernel<1><<<grid, 1024, smem, s>>>(csr_ptr, csr_col, n, N, eps_q, escale, Zf, R32, S64, rmax_p, rhs_t,
-                                                             a.rhs_real);
+            residual_rows_kernel<1><<<grid, 1024, smem, s>>>(csr_ptr, csr_col, n, N, eps_q, escale, Zf, R32, S64, rmax_p,
+                                                             rhs_t ? rhs_t : a.rhs, rhs_t != nullptr, a.rhs_real);
         return cudaGetLastError();
     };
     // Later residuals from the sums' updates: a product of E in f16 with the correction's two slices
     // where E has at least kSliceDensity of its entries, else gathers.
-    const bool slices = need_x && static_cast<double>(nnz) >= kSliceDensity * n * n;
+    // Without room for the sums (8 np^2 bytes) every residual is formed as a whole.
+    bool slices = need_x && static_cast<double>(nnz) >= kSliceDensity * n * n;
     const int sb = std::min(11, 24 - deg_bits);  // a slice's sum of dmax terms of 2^sb stays within 2^24
     // (the slices and E in f16 take Zf's place once the first residual is formed, the products X64's)
     auto *Q16 = reinterpret_cast<__half *>(Zf);
@@ -1536,8 +1545,8 @@ dl_status tc_mixed(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &
         MCK(allow_all_smem(refine_add_kernel<false>));
         MCK(rows_q == 4 ? allow_all_smem(update_rows_kernel<4>) : allow_all_smem(update_rows_kernel<2>));
     }
-    auto first_fix = [&](const float *D) -> cudaError_t {
-        first_fix_kernel<<<static_cast<unsigned>(np), 256, row_smem, s>>>(Z64, D, n, N, deg_bits, min_hb,
+    auto first_fix = [&](const float *D, bool add) -> cudaError_t {
+        first_fix_kernel<<<static_cast<unsigned>(np), 256, row_smem, s>>>(Z64, D, add, n, N, deg_bits, min_hb,
                                                                         general_rhs ? 0 : 1, escale,
                                                                         banded || !need_x ? nullptr : Zf);
         ++launches;
@@ -1593,14 +1602,19 @@ dl_status tc_mixed(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &
         auto *pcnt = static_cast<int *>(ws.get("mx_pcnt", (np + 1) * 4));
         pptr = static_cast<int *>(ws.get("mx_pptr", (np + 1) * 4));
         if (!At || !pcnt || !pptr) {
-            set_error("mixed path: device allocation failed (CSR of the right-hand side)");
-            return DL_ENOMEM;
+            if (!a.rhs) {
+                set_error("mixed path: device allocation failed (CSR of the right-hand side)");
+                return DL_ENOMEM;
+            }
+            sparse_first = false;  // (A itself does, with a dense first product)
         }
-        MCK(transpose(rhs_bytes, n, n, n, At, n, s));
-        MCK(csr_build(At, n, pcnt, pptr, s));
-        launches += 3;
         int facts = nnz;
-        if (a.rhs) {
+        if (sparse_first) {
+            MCK(transpose(rhs_bytes, n, n, n, At, n, s));
+            MCK(csr_build(At, n, pcnt, pptr, s));
+            launches += 3;
+        }
+        if (sparse_first && a.rhs) {
             MCK(cudaMemcpyAsync(&facts, pptr + n, sizeof(int), cudaMemcpyDeviceToHost, s));
             MCK(cudaStreamSynchronize(s));
             sparse_first = static_cast<int64_t>(facts) <= kSparseFirstDegree * n;
@@ -1608,14 +1622,20 @@ dl_status tc_mixed(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &
         }
         if (sparse_first) {
             pcol = static_cast<int *>(ws.get("mx_pcol", static_cast<size_t>(std::max(facts, 1)) * 4));
-            if (!pcol) {
+            if (pcol) {
+                MCK(csr_fill(At, n, pptr, pcol, s));
+                ++launches;
+            } else if (a.rhs) {
+                sparse_first = false;
+            } else {
                 set_error("mixed path: device allocation failed (CSR of the right-hand side)");
                 return DL_ENOMEM;
             }
-            MCK(csr_fill(At, n, pptr, pcol, s));
-            ++launches;
         }
     }
+    if (need_x) S64 = static_cast<long long *>(ws.get("mx_S", np * np * 8));
+    ws.spare("mx_S");  // (nothing is got while the loop below runs; what follows may have the room)
+    slices = slices && S64 != nullptr;
     // Without an R~ output only the model is wanted: X > 0 after the solve is already exact where
     // it is positive (A is an M-matrix and every quantity of the factorisation keeps its sign, so
     // no entry cancels to a spurious value), entries lost to underflow land in the guard band, and
@@ -1648,13 +1668,13 @@ dl_status tc_mixed(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &
         }
         ++products;
         if (!need_x) {  // the model only: no refinement
-            MCK(first_fix(D32));
+            MCK(first_fix(D32, false));
             break;
         }
         unsigned h[2] = {0, 0};  // max|R| (bits of a float), a row has outgrown its scale
         MCK(cudaMemsetAsync(rmax_d, 0, sizeof(h), s));
-        if (products == 1) {
-            MCK(first_fix(D32));
+        if (products == 1 || S64 == nullptr) {
+            MCK(first_fix(D32, products > 1));
             MCK(residual_whole(rmax_d));
         } else {
             MCK(residual_update(rmax_d));
@@ -1663,7 +1683,7 @@ dl_status tc_mixed(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &
         MCK(cudaStreamSynchronize(s));
         if (h[1] != 0) {  // new scales, the sums formed again
             MCK(cudaMemsetAsync(rmax_d, 0, sizeof(h), s));
-            MCK(first_fix(nullptr));
+            MCK(first_fix(nullptr, false));
             MCK(residual_whole(rmax_d));
             MCK(cudaMemcpyAsync(h, rmax_d, sizeof(h), cudaMemcpyDeviceToHost, s));
             MCK(cudaStreamSynchronize(s));

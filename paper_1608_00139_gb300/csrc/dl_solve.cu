@@ -2613,6 +2613,7 @@ void Workspace::release() {
 
 void *Workspace::get(const std::string &name, size_t bytes) {
     Buf &b = bufs[name];
+    b.spare = false;
     if (b.p && b.bytes >= bytes) return b.p;
     // grow by at least a quarter: buffers sized by data (facts, active rows) then rarely grow
     // again, and a regrowth's cudaFree waits for the whole device
@@ -2623,13 +2624,31 @@ void *Workspace::get(const std::string &name, size_t bytes) {
         b.bytes = 0;
     }
     size_t want = (std::max(bytes, grown) + 4095) & ~static_cast<size_t>(4095);
-    if (device_alloc(&b.p, want) != cudaSuccess) {
+    cudaError_t e = device_alloc(&b.p, want);
+    if (e != cudaSuccess && drop_spares()) e = device_alloc(&b.p, want);
+    if (e != cudaSuccess) {
         cudaGetLastError();
         b.p = nullptr;
         return nullptr;
     }
     b.bytes = want;
     return b.p;
+}
+
+void Workspace::spare(const std::string &name) {
+    const auto it = bufs.find(name);
+    if (it != bufs.end()) it->second.spare = true;
+}
+
+bool Workspace::drop_spares() {
+    bool any = false;
+    for (auto &kv : bufs)
+        if (kv.second.spare && kv.second.p) {
+            cudaFree(kv.second.p);  // (waits for the device)
+            kv.second = Buf{};
+            any = true;
+        }
+    return any;
 }
 
 size_t Workspace::capacity(const std::string &name) const {
