@@ -145,6 +145,7 @@ dl_status dl_create(dl_ctx **out, int device, const dl_config *cfg) {
         return DL_ENOMEM;
     }
     ctx->device = device;
+    ctx->ws.store = &ctx->store;
     if (cfg) ctx->cfg = *cfg;
     if (ctx->cfg.wait_timeout_s > 0) ctx->budget_ns = static_cast<uint64_t>(ctx->cfg.wait_timeout_s * 1e9);
     if (set_device(ctx) != DL_OK) {
@@ -173,6 +174,7 @@ dl_status dl_destroy(dl_ctx *ctx) {
         cudaSetDevice(ctx->device);
         cudaStreamSynchronize(ctx->stream);
         ctx->ws.release();
+        ctx->store.drop(nullptr);
         if (ctx->own_stream) cudaStreamDestroy(ctx->own_stream);
     }
     delete ctx;

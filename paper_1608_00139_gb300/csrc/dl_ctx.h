@@ -6,6 +6,7 @@
 #include <cstdarg>
 #include <cstdint>
 #include <deque>
+#include <list>
 #include <map>
 #include <memory>
 #include <mutex>
@@ -23,6 +24,30 @@ void set_error(const char *fmt, ...);
 struct BatchPlan;  // cached CUDA graph of the last dl_tc_batch call (dl_batch.cu)
 void batch_plan_release(BatchPlan *p);
 
+// The byte matrices that the runs of a context's programs work on, kept between runs (cudaMalloc and
+// cudaFree of a dozen matrices took 0.9 of a run's 1.4 ms at n = 2048).  A block is its program's own and is
+// freed with it; together a context's programs keep at most kStoreBytes between runs, the longest unused
+// blocks going first (larger matrices cost more than their allocation does).  Serving threads may call
+// release_idle.
+struct MatrixStore {
+    struct Block {
+        void *p;
+        size_t bytes;
+        const void *owner;
+        bool used;
+    };
+    static constexpr size_t kStoreBytes = size_t{1} << 30;
+    std::mutex mu;
+    std::list<Block> blocks;  // the longest unused first
+
+    void *take(const void *owner, size_t bytes);  // an idle block of that size, or nullptr
+    void add(const void *owner, void *p, size_t bytes);
+    void give_back(const std::vector<void *> &ps);
+    void trim();                    // idle blocks over kStoreBytes are freed
+    bool release_idle();            // all of them are; whether there were any
+    void drop(const void *owner);   // a program's end (owner == nullptr: the context's)
+};
+
 // Grow-only device buffers, one set per execution slot (a synchronous call or one serving
 // slot), so concurrent slots never share scratch memory.
 struct Workspace {
@@ -36,6 +61,7 @@ struct Workspace {
     size_t host_bytes = 0;
     int *status = nullptr;         // device status word
     unsigned long long *scal = nullptr;  // device scalars (counters)
+    MatrixStore *store = nullptr;  // its context's
     cudaEvent_t ev[8] = {};
     static constexpr int kGemmEvents = 128;  // start/stop pairs of timed GEMM launches
     cudaEvent_t gev[kGemmEvents] = {};
@@ -65,7 +91,8 @@ struct Workspace {
     void *get(const std::string &name, size_t bytes);
     // Buffer `name` is not needed until it is got again: a get() that finds no room may free it.
     void spare(const std::string &name);
-    bool drop_spares();  // frees them; whether there were any
+    // Frees what can be done without (spare buffers, the programs' idle matrices); whether there was any.
+    bool reclaim();
     // bytes held by buffer `name` (0 if it does not exist)
     size_t capacity(const std::string &name) const;
     size_t footprint() const;
@@ -105,6 +132,7 @@ struct dl_ctx {
     uint64_t budget_ns = 2000000000ull;
     std::mutex mu;  // serialises synchronous calls
     dl::Workspace ws;
+    dl::MatrixStore store;
 
     dl::Tuning tune;  // tuned choices per size bucket (dl_tune.cu)
 

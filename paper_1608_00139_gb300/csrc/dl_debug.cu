@@ -15,6 +15,7 @@
 #include <mutex>
 #include <string>
 
+#include "dl_ctx.h"
 #include "dl_internal.h"
 
 namespace dl {
@@ -67,12 +68,17 @@ bool next_alloc_fails() {
 
 }  // namespace
 
-cudaError_t device_alloc(void **ptr, size_t bytes) {
+cudaError_t device_alloc(void **ptr, size_t bytes, Workspace *ws) {
     if (next_alloc_fails()) {
         *ptr = nullptr;
         return cudaErrorMemoryAllocation;
     }
-    return cudaMalloc(ptr, bytes);
+    cudaError_t e = cudaMalloc(ptr, bytes);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        if (ws != nullptr && ws->reclaim() && (e = cudaMalloc(ptr, bytes)) != cudaSuccess) cudaGetLastError();
+    }
+    return e;
 }
 
 cudaError_t host_pinned_alloc(void **ptr, size_t bytes) {

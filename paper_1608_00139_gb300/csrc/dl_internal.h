@@ -11,8 +11,10 @@
 namespace dl {
 
 // Every allocation of the library goes through these (dl_debug.cu): cudaMalloc / cudaMallocHost,
-// or cudaErrorMemoryAllocation when the DL_FAULT plan says this allocation fails.
-cudaError_t device_alloc(void **ptr, size_t bytes);
+// or cudaErrorMemoryAllocation when the DL_FAULT plan says this allocation fails.  Where the device has no
+// room, what ws can do without is freed first (Workspace::reclaim).
+struct Workspace;
+cudaError_t device_alloc(void **ptr, size_t bytes, Workspace *ws = nullptr);
 cudaError_t host_pinned_alloc(void **ptr, size_t bytes);
 
 // An NVTX range for the lifetime of the object (a no-op unless a profiler is attached).

@@ -64,26 +64,10 @@ struct Factor {
     bool transposed = false, negated = false;
 };
 
-// The byte matrices a program's runs work on, kept between them (cudaMalloc and cudaFree of a dozen
-// matrices took 0.9 of a run's 1.4 ms at n = 2048); as many as the largest run needed, up to kStoreBytes
-// in all between runs (larger matrices cost more than their allocation does), freed with the program.  A
-// program's calls are serialised by its context.
-constexpr size_t kStoreBytes = size_t{1} << 30;
-
-struct MatrixStore {
-    struct Block {
-        void *p;
-        size_t bytes;
-        bool used;
-    };
-    std::vector<Block> blocks;
-};
-
 }  // namespace dl
 
 struct dl_program {
     dl_ctx *ctx = nullptr;
-    dl::MatrixStore store;
     std::vector<dl::PClause> clauses;
     std::set<std::string> idb, edb;
     std::vector<std::vector<std::string>> layers;  // topological order
@@ -346,35 +330,26 @@ unsigned grid_for(int64_t count) {
     return static_cast<unsigned>(std::max<int64_t>(1, std::min<int64_t>((count / 16 + 255) / 256, 2048)));
 }
 
-// Byte matrices of one run, taken from the program's store and given back to it at the run's end (every
-// run ends with a wait for its stream, a failed one too, so the next may use them on any stream).
+// Byte matrices of one run (or one iteration of it), taken from the context's store and given back to it once
+// the run's stream is idle, so that the next run may use them on any stream.
 struct Pool {
-    MatrixStore &store;
-    std::vector<size_t> taken;
-    explicit Pool(MatrixStore &m) : store(m) {}
+    dl_program *prog;
+    cudaStream_t s;
+    std::vector<void *> taken;
+    Pool(dl_program *p, cudaStream_t stream) : prog(p), s(stream) {}
     Pool(const Pool &) = delete;
     ~Pool() {
-        for (size_t k : taken) store.blocks[k].used = false;
-        size_t held = 0;
-        for (const auto &b : store.blocks) held += b.bytes;
-        while (held > kStoreBytes && !store.blocks.back().used) {  // (blocks in use keep their places)
-            held -= store.blocks.back().bytes;
-            cudaFree(store.blocks.back().p);
-            store.blocks.pop_back();
-        }
+        cudaStreamSynchronize(s);  // (idle already unless the run has failed)
+        prog->ctx->store.give_back(taken);
     }
     uint8_t *alloc(size_t bytes) {
         bytes = std::max<size_t>(bytes, 16);
-        for (size_t k = 0; k < store.blocks.size(); ++k)
-            if (!store.blocks[k].used && store.blocks[k].bytes == bytes) {
-                store.blocks[k].used = true;
-                taken.push_back(k);
-                return static_cast<uint8_t *>(store.blocks[k].p);
-            }
-        void *p = nullptr;
-        if (device_alloc(&p, bytes) != cudaSuccess) return nullptr;
-        store.blocks.push_back(MatrixStore::Block{p, bytes, true});
-        taken.push_back(store.blocks.size() - 1);
+        void *p = prog->ctx->store.take(prog, bytes);
+        if (!p) {
+            if (device_alloc(&p, bytes, &prog->ctx->ws) != cudaSuccess) return nullptr;
+            prog->ctx->store.add(prog, p, bytes);
+        }
+        taken.push_back(p);
         return static_cast<uint8_t *>(p);
     }
 };
@@ -521,6 +496,74 @@ struct Term {
 
 }  // namespace
 
+void *MatrixStore::take(const void *owner, size_t bytes) {
+    std::lock_guard<std::mutex> lk(mu);
+    for (Block &b : blocks)
+        if (!b.used && b.owner == owner && b.bytes == bytes) {
+            b.used = true;
+            return b.p;
+        }
+    return nullptr;
+}
+
+void MatrixStore::add(const void *owner, void *p, size_t bytes) {
+    std::lock_guard<std::mutex> lk(mu);
+    blocks.push_back(Block{p, bytes, owner, true});
+}
+
+void MatrixStore::give_back(const std::vector<void *> &ps) {
+    std::lock_guard<std::mutex> lk(mu);
+    for (void *p : ps)
+        for (auto it = blocks.begin(); it != blocks.end(); ++it)
+            if (it->p == p) {
+                it->used = false;
+                blocks.splice(blocks.end(), blocks, it);
+                break;
+            }
+}
+
+void MatrixStore::trim() {
+    std::lock_guard<std::mutex> lk(mu);
+    size_t held = 0;
+    for (const Block &b : blocks) held += b.bytes;
+    for (auto it = blocks.begin(); it != blocks.end() && held > kStoreBytes;) {
+        if (it->used) {
+            ++it;
+            continue;
+        }
+        held -= it->bytes;
+        cudaFree(it->p);
+        it = blocks.erase(it);
+    }
+}
+
+bool MatrixStore::release_idle() {
+    std::lock_guard<std::mutex> lk(mu);
+    bool any = false;
+    for (auto it = blocks.begin(); it != blocks.end();) {
+        if (it->used) {
+            ++it;
+            continue;
+        }
+        cudaFree(it->p);  // (waits for the device)
+        it = blocks.erase(it);
+        any = true;
+    }
+    return any;
+}
+
+void MatrixStore::drop(const void *owner) {
+    std::lock_guard<std::mutex> lk(mu);
+    for (auto it = blocks.begin(); it != blocks.end();) {
+        if (owner != nullptr && it->owner != owner) {
+            ++it;
+            continue;
+        }
+        cudaFree(it->p);
+        it = blocks.erase(it);
+    }
+}
+
 dl_status program_create(dl_ctx *ctx, const char *text, dl_program **out) {
     auto *p = new (std::nothrow) dl_program;
     if (!p) {
@@ -578,7 +621,7 @@ dl_status program_create(dl_ctx *ctx, const char *text, dl_program **out) {
 void program_destroy(dl_program *p) {
     if (!p) return;
     for (auto &kv : p->rel) cudaFree(kv.second);
-    for (auto &b : p->store.blocks) cudaFree(b.p);
+    p->ctx->store.drop(p);
     delete p;
 }
 
@@ -593,7 +636,7 @@ dl_status program_set(dl_program *p, cudaStream_t s, const char *pred, int32_t n
     }
     const size_t bytes = static_cast<size_t>(n) * n;
     uint8_t *&d = p->rel[pred];
-    if (!d && device_alloc(reinterpret_cast<void **>(&d), std::max<size_t>(bytes, 16)) != cudaSuccess) {
+    if (!d && device_alloc(reinterpret_cast<void **>(&d), std::max<size_t>(bytes, 16), &p->ctx->ws) != cudaSuccess) {
         d = nullptr;
         p->rel.erase(pred);
         set_error("program: device allocation failed");
@@ -619,7 +662,11 @@ dl_status program_run(dl_ctx *ctx, Workspace &ws, cudaStream_t s, dl_program *p,
     const int32_t n = p->n;
     const size_t nbytes = std::max<size_t>(static_cast<size_t>(n) * n, 16);
     std::ostringstream plan;
-    Pool pool(p->store);
+    struct Trim {  // (after the pool has given its matrices back)
+        MatrixStore &store;
+        ~Trim() { store.trim(); }
+    } trim{ctx->store};
+    Pool pool(p, s);
     Runner R{ctx, ws, s, n, &pool};
     dl_status rc;
     std::map<std::string, uint8_t *> model;  // this run's models (pool-owned until kept)
@@ -830,7 +877,7 @@ dl_status program_run(dl_ctx *ctx, Workspace &ws, cudaStream_t s, dl_program *p,
                         return DL_ENOTCONV;
                     }
                     {
-                        Pool inner(p->store);
+                        Pool inner(p, s);
                         R.pool = &inner;
                         for (int h = 0; h < M && !rc; ++h) {
                             if ((rc = R.copy(nxt[h], A[h]))) break;
@@ -860,8 +907,7 @@ dl_status program_run(dl_ctx *ctx, Workspace &ws, cudaStream_t s, dl_program *p,
     // keep the models (program-owned copies)
     for (auto &kv : model) {
         uint8_t *&d = p->rel[kv.first];
-        if (!d && device_alloc(reinterpret_cast<void **>(&d), nbytes) != cudaSuccess) {
-            cudaGetLastError();
+        if (!d && device_alloc(reinterpret_cast<void **>(&d), nbytes, &ctx->ws) != cudaSuccess) {
             p->rel.erase(kv.first);
             set_error("program: device allocation failed");
             return DL_ENOMEM;

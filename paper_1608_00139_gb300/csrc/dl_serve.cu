@@ -142,6 +142,7 @@ dl_status start_serving(dl_ctx *ctx) {
     const int nslots = ctx->cfg.max_slots > 0 ? ctx->cfg.max_slots : 4;
     for (int i = 0; i < nslots; ++i) {
         auto slot = std::make_unique<dl_ctx::Serve::Slot>();
+        slot->ws.store = &ctx->store;
         if (cudaStreamCreateWithFlags(&slot->stream, cudaStreamNonBlocking) != cudaSuccess) {
             set_error("serving: cudaStreamCreate failed");
             for (auto &s : sv->slots) cudaStreamDestroy(s->stream);

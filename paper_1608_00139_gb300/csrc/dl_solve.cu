@@ -2624,10 +2624,7 @@ void *Workspace::get(const std::string &name, size_t bytes) {
         b.bytes = 0;
     }
     size_t want = (std::max(bytes, grown) + 4095) & ~static_cast<size_t>(4095);
-    cudaError_t e = device_alloc(&b.p, want);
-    if (e != cudaSuccess && drop_spares()) e = device_alloc(&b.p, want);
-    if (e != cudaSuccess) {
-        cudaGetLastError();
+    if (device_alloc(&b.p, want, this) != cudaSuccess) {
         b.p = nullptr;
         return nullptr;
     }
@@ -2640,8 +2637,8 @@ void Workspace::spare(const std::string &name) {
     if (it != bufs.end()) it->second.spare = true;
 }
 
-bool Workspace::drop_spares() {
-    bool any = false;
+bool Workspace::reclaim() {
+    bool any = store != nullptr && store->release_idle();
     for (auto &kv : bufs)
         if (kv.second.spare && kv.second.p) {
             cudaFree(kv.second.p);  // (waits for the device)
