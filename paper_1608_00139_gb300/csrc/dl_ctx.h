@@ -78,8 +78,15 @@ struct Workspace {
     int mx_graph_launches = 0;
     BatchPlan *batch_plan = nullptr;
     bool last_heavy = false;  // the last closure on this workspace had rows of > 256 successors
-    bool last_wide = false;   // ... and a model of more than 256 facts per row (no walks next time)
-    int layer_skips = 0;      // same-generation calls left before layers are looked for again
+    // what the last relation that a route did not suit looked like: size, longest row, facts
+    struct Shape {
+        int64_t n = 0;
+        unsigned long long dmax = 0, nnz = 0;
+        bool is(int64_t n_, unsigned long long d, unsigned long long f) const { return n == n_ && dmax == d && nnz == f; }
+    };
+    Shape wide;           // a closure with heavy rows and more than 256 facts per row (no walks for it)
+    Shape unlayered;      // a same-generation relation without short layers,
+    int layer_skips = 0;  // ... not looked for again in this many calls with one of that shape
     bool last_rows_closed = false;  // ... was closed by the Iteration on single rows alone
     bool last_dense = false;        // ... had more than two facts per row (no single-row Iteration)
     int last_spec_sweeps = 0;       // ... settled in its speculative phase after this many

@@ -668,8 +668,10 @@ dl_status tc_auto(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &a
     };
     // rows of more than 256 successors: the model by walks over the successor lists, which a closure of
     // few facts per row (a citation-like DAG) needs no more than (n = 16384: 2.05 ms by sweeps, 0.36 ms);
-    // given up on the device when it is not, and not tried after a heavy closure that was wide
-    if (!spec && !dense && dmax > 256 && wp <= 256 && !ws.last_wide) {
+    // given up on the device when it is not, and not tried again for a relation as the last one that was wide
+    // (size, longest row and facts; 39 us for nothing each time)
+    if (!spec && !dense && dmax > 256 && wp <= 256 &&
+        !ws.wide.is(n, dmax, static_cast<unsigned long long>(nnz))) {
         auto *open_rows = static_cast<int *>(ws.get("g_open", (np + 1) * 4));
         NEED(open_rows);
         auto *counters = reinterpret_cast<unsigned *>(ws.scal + SC_OPEN);
@@ -800,7 +802,8 @@ dl_status tc_auto(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &a
         set_error("internal: converged closure failed its certificate");
         return DL_EDEVICE;
     }
-    if (ws.last_heavy) ws.last_wide = host_scal(ws)[SC_ONES] > 256ull * static_cast<unsigned long long>(n);
+    if (dmax > 256 && host_scal(ws)[SC_ONES] > 256ull * static_cast<unsigned long long>(n))
+        ws.wide = {n, dmax, static_cast<unsigned long long>(nnz)};
     if (!direct && (rc = write_bits(s, mbits, wp, a.out_bits, n, a.mem))) return rc;
     tm.mark(3);
     if ((rc = finish(ws, s))) return rc;
@@ -1081,11 +1084,15 @@ void layers_read(Workspace &ws, Layers *ly) {
 // When P is acyclic in few layers of short parent lists (a forest, a shallow DAG), the rows are
 // formed layer by layer instead, each once, from the final rows of its parents (sg_level):
 // forest N = 4096, 17 layers, one call: 0.85 ms by the doubling, 0.21 ms here.
-// Otherwise, and unless iterate is set, it returns at once.
+// Otherwise, and unless iterate is set, it returns at once.  The search for layers costs some 30 us, a
+// tenth of a small doubling: it is left out in the kLayerSkips calls after one that found none, for a
+// relation of the same size, longest row and facts (unless look_now: it is known to be another one).
 // Returns with *done = false (and nothing written) if the rows are too wide or the
 // iterations exceed the budget: the doubling below then solves the problem.
+constexpr int kLayerSkips = 7;
+
 dl_status sg_iteration(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &a, dl_stats *st, bool *done,
-                       bool iterate = true, const uint64_t *seed = nullptr, bool *layered = nullptr) {
+                       bool iterate = true, const uint64_t *seed = nullptr, bool look_now = false) {
     (void)ctx;
     *done = false;
     const int32_t n = a.n;
@@ -1128,18 +1135,27 @@ dl_status sg_iteration(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveAr
         ++launches;
     }
     Layers ly;
-    if (!a.no_layers && !seed && dag_levels_fit(n)) {
-        if ((rc = layers_enqueue(ws, s, X, n, wp, ptr, &ly))) return rc;
-        launches += 2;
-    }
+    bool look = !a.no_layers && !seed && dag_levels_fit(n);
+    const bool defer = look && !look_now && ws.layer_skips > 0 && ws.unlayered.n == n;  // until the facts are counted
+    if (look && !defer && (rc = layers_enqueue(ws, s, X, n, wp, ptr, &ly))) return rc;
     if ((rc = read_scalars(ws, s)) || (rc = read_status(ws))) return rc;
+    if (defer && ws.unlayered.is(n, host_scal(ws)[SC_DMAX], host_scal(ws)[SC_NNZ])) {
+        --ws.layer_skips;
+        look = false;
+    } else if (defer) {
+        if ((rc = layers_enqueue(ws, s, X, n, wp, ptr, &ly)) || (rc = read_scalars(ws, s))) return rc;
+    }
+    if (look) launches += 2;
     layers_read(ws, &ly);
-    if (layered) *layered = ly.levels() > 0;
     const double dmax = static_cast<double>(host_scal(ws)[SC_DMAX]);
     double eps = 0;
     if ((rc = choose_eps(a.eps, 1.0 / (1.0 + dmax * dmax), "Sec. 7.2 (1/(1+||P||^2))", &eps))) return rc;
     const bool sym = seed == nullptr && (Bm == nullptr || host_scal(ws)[SC_CQ] == 0);
     const int64_t nnz = static_cast<int64_t>(host_scal(ws)[SC_NNZ]);
+    if (look && ly.levels() == 0) {
+        ws.unlayered = {n, host_scal(ws)[SC_DMAX], host_scal(ws)[SC_NNZ]};
+        ws.layer_skips = kLayerSkips;
+    }
     if (!iterate && ly.levels() == 0) return DL_OK;
     auto *col = ly.filled ? ly.col : static_cast<int *>(ws.get("g_col", static_cast<size_t>(std::max<int64_t>(nnz, 1)) * 4));
     NEED(col);
@@ -1214,7 +1230,8 @@ dl_status sg_iteration(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveAr
     return DL_OK;
 }
 
-dl_status sg_doubling(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &a, dl_stats *st);
+dl_status sg_doubling(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &a, dl_stats *st,
+                      bool *other = nullptr);
 
 dl_status solve_sg(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &a, dl_stats *st) {
     if (a.thr != 0.0) {
@@ -1233,26 +1250,20 @@ dl_status solve_sg(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &
     // Layers, where P has them, are cheaper than either (and found by the same preparation).
     const int tuned_iteration = tuned(ctx, np).sg_iteration;  // measured crossover, when tuned
     const bool iterate = tuned_iteration >= 0 ? tuned_iteration == 1 : np >= 6144;
-    // (not looked for in the next kLayerSkips calls of a workspace whose last search found none: it costs
-    // some 30 us, a tenth of a small doubling)
-    constexpr int kLayerSkips = 7;
-    SolveArgs b = a;
-    if (!b.no_layers && ws.layer_skips > 0) {
-        --ws.layer_skips;
-        b.no_layers = true;
-    }
-    if (a.path == DL_PATH_AUTO && (iterate || !b.no_layers)) {
-        bool done = false, layered = false;
-        const dl_status rc = sg_iteration(ctx, ws, s, b, st, &done, iterate, nullptr, &layered);
-        if (!b.no_layers && !layered) ws.layer_skips = kLayerSkips;
-        if (rc != DL_OK || done) return rc;
+    if (a.path == DL_PATH_AUTO && (iterate || !a.no_layers)) {
+        dl_status rc;
+        bool done = false, other = false;
+        if (!iterate && ws.layer_skips > 0 && ws.unlayered.n == a.n)  // no layers if it is of the last one's shape
+            if ((rc = sg_doubling(ctx, ws, s, a, st, &other)) || !other) return rc;
+        if ((rc = sg_iteration(ctx, ws, s, a, st, &done, iterate, nullptr, other)) || done) return rc;
     }
     return sg_doubling(ctx, ws, s, a, st);
 }
 
 // Same generation by boolean doubling on the tensor cores: S_{2m} = min1(S_m + Q_m S_m Q_m^T),
-// Q_{2m} = min1(Q_m^2), from S_1 = B, Q_1 = P.
-dl_status sg_doubling(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &a, dl_stats *st) {
+// Q_{2m} = min1(Q_m^2), from S_1 = B, Q_1 = P.  With other: for a relation of the shape of the last one without
+// layers only; any other is left alone, and *other set, as soon as its facts are counted.
+dl_status sg_doubling(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &a, dl_stats *st, bool *other) {
     const int32_t n = a.n;
     const int64_t np = round_up(std::max<int64_t>(n, 1), 256);
     const int64_t wp = np / 64;
@@ -1281,6 +1292,11 @@ dl_status sg_doubling(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArg
     }
     tm.mark(1);
     if ((rc = read_scalars(ws, s)) || (rc = read_status(ws))) return rc;
+    if (other) {
+        *other = !ws.unlayered.is(n, host_scal(ws)[SC_DMAX], host_scal(ws)[SC_NNZ]);
+        if (*other) return DL_OK;
+        --ws.layer_skips;
+    }
     const double dmax = static_cast<double>(host_scal(ws)[SC_DMAX]);
     double eps = 0;
     if ((rc = choose_eps(a.eps, 1.0 / (1.0 + dmax * dmax), "Sec. 7.2 (1/(1+||P||^2))", &eps))) return rc;
