@@ -676,9 +676,7 @@ dl_status tc_auto(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &a
         NEED(open_rows);
         auto *counters = reinterpret_cast<unsigned *>(ws.scal + SC_OPEN);
         CK(cudaMemsetAsync(counters, 0, 2 * sizeof(unsigned long long), s));
-        sc.start();
         CK(reach_rows(ptr, col, n, wp, model, open_rows, counters, s));
-        sc.stop();
         launches += 2;
         if ((rc = read_scalars(ws, s))) return rc;
         const auto *h = reinterpret_cast<const unsigned *>(host_scal(ws) + SC_OPEN);
@@ -715,13 +713,10 @@ dl_status tc_auto(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &a
     if (spec && !converged && t_sq > 100e-6 && close_slices_count(n, wp) > 0) {
         const int slices = close_slices_count(n, wp);
         CK(cudaMemsetAsync(vslot, 0, 3 * sizeof(unsigned long long), s));
-        sc.start();
-        CK(close_slices(ptr, col, n, wp, rbits, model, vslot, ws.status, s));
-        sc.stop();
+        CK(close_slices(ptr, col, n, wp, rbits, model, vslot, ws.status, s));  // (its sweeps are not through memory)
         ++launches;
         if ((rc = read_scalars(ws, s)) || (rc = read_status(ws))) return rc;
         const int ran = static_cast<int>(host_scal(ws)[34]);
-        sc.account(ran + 1, sweep_min_bytes);
         sweeps += ran;
         if (host_scal(ws)[32] == static_cast<unsigned long long>(slices)) {
             host_scal(ws)[SC_ONES] = host_scal(ws)[33];

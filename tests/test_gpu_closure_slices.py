@@ -54,3 +54,19 @@ def test_output_aligned_to_its_words_only(ctx, n):
     assert np.array_equal(out.cpu().numpy().view(np.uint64), ref)
     assert st["model_ones"] == int(np.unpackbits(ref.view(np.uint8)).sum())
     assert int(buf[0]) == -3 and int(buf[-1]) == -3
+
+
+def test_sweep_counters_hold_sweeps_through_memory_only(ctx):
+    """The steps that a slice takes in shared memory, and the walks of hub rows, are no sweep launches."""
+    oracle.set_threads(0)
+    n = 6000
+    dev = torch.from_numpy(inputs.er_digraph(n, 2.5 / n, 1)).cuda()
+    for _ in range(2):
+        _, st = ctx.tc_closure(dev)
+        assert 0 < st["sweep_launches"] < st["gpu_launches"] and st["recheck_sweeps"] > st["sweep_launches"]
+    dag = inputs.pa_dag(3000, 3000)
+    assert dag.sum(axis=1).max() > 256
+    for _ in range(2):  # (the second call walks from the start)
+        bits, st = ctx.tc_closure(dag)
+        assert np.array_equal(bits, oracle.tc_model(dag))
+    assert st["sweep_launches"] == 0 and st["ms_sweep"] == 0 and st["sweep_bytes"] == 0
