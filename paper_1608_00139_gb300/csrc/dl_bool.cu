@@ -412,6 +412,8 @@ __global__ void __launch_bounds__(256)
 //      row whose frontier outgrows kReachFront or whose paths are longer than kReachSteps stays open.
 //  (2) reach_open_kernel: a CTA per open row, any frontier.  It gives all up when too many are open
 //      (the closure is not small: sweeps and squarings are for that).
+// A walk's certificate: the constants whose lists it has read are as many as its row has bits (every
+// constant reached has been expanded, so the row is closed under E, and it holds nothing unreached).
 constexpr int kReachFront = 512, kReachSteps = 64, kReachLight = 16;
 
 // The successors of the constants nodes[0 .. cnt), 32 per turn from `first` on by `stride`: visit(j) for
@@ -439,10 +441,11 @@ __device__ __forceinline__ void expand_nodes(const int *__restrict__ ptr, const 
     }
 }
 
-// counters[0] = open rows, [1] = rows given up, [2] = ones of the rows written.
+// counters[0] = open rows, [1] = rows given up, [2] = ones of the rows written; *violations += rows that fail
+// their certificate.
 __global__ void __launch_bounds__(256)
     reach_rows_kernel(const int *__restrict__ ptr, const int *__restrict__ col, int n, int wp, uint64_t *__restrict__ out,
-                      int *__restrict__ open_rows, unsigned *counters) {
+                      int *__restrict__ open_rows, unsigned *counters, unsigned long long *violations) {
     extern __shared__ uint64_t reach_s[];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     // per warp: the row's bits, two frontiers, the next frontier's length
@@ -458,6 +461,7 @@ __global__ void __launch_bounds__(256)
     for (int w = lane; w < wp; w += 32) bits[w] = 0ull;
     if (lane == 0) front[0] = static_cast<uint16_t>(i);
     int cnt = 1, cur = 0, steps = 0;
+    unsigned expanded = 0;  // constants reached whose lists have been read
     bool closed = true;
     __syncwarp();
     while (cnt > 0) {
@@ -479,6 +483,7 @@ __global__ void __launch_bounds__(256)
         cnt = *next_cnt;
         __syncwarp();  // every lane has read the count before lane 0 clears it
         cur ^= 1;
+        expanded += cnt;  // (by the next turn, or the row stays open)
     }
     if (!closed) {
         if (lane == 0) open_rows[atomicAdd(counters, 1u)] = i;
@@ -491,15 +496,17 @@ __global__ void __launch_bounds__(256)
     }
     ones = __reduce_add_sync(0xffffffffu, ones);
     if (lane == 0 && ones) atomicAdd(reinterpret_cast<unsigned long long *>(counters + 2), static_cast<unsigned long long>(ones));
+    if (lane == 0 && ones != expanded) atomicAdd(violations, 1ull);
 }
 
 __global__ void __launch_bounds__(256)
     reach_open_kernel(const int *__restrict__ ptr, const int *__restrict__ col, int n, int wp, uint64_t *__restrict__ out,
-                      const int *__restrict__ open_rows, unsigned *counters) {
+                      const int *__restrict__ open_rows, unsigned *counters, unsigned long long *violations) {
     extern __shared__ uint64_t reach_s[];
     uint64_t *bits = reach_s, *done = bits + wp;              // reached; reached and expanded
     uint16_t *list = reinterpret_cast<uint16_t *>(done + wp);  // the step's constants (at most n)
     __shared__ int cnt_s;
+    __shared__ unsigned ones_s;
     const unsigned open = counters[0];
     if (open > static_cast<unsigned>(n) / 8) {
         if (blockIdx.x == 0 && threadIdx.x == 0) counters[1] = open;
@@ -512,9 +519,11 @@ __global__ void __launch_bounds__(256)
         if (threadIdx.x == 0) {
             list[0] = static_cast<uint16_t>(i);
             cnt_s = 1;
+            ones_s = 0u;
         }
         __syncthreads();
         int cnt = 1, steps = 0;
+        unsigned expanded = 0;
         while (cnt > 0 && steps < 2 * kReachSteps) {
             ++steps;
             expand_nodes(ptr, col, list, cnt, 32 * warp, static_cast<int>(blockDim.x), [&](int j) {
@@ -534,6 +543,7 @@ __global__ void __launch_bounds__(256)
             }
             __syncthreads();
             cnt = cnt_s;
+            expanded += cnt;
         }
         unsigned ones = 0;
         for (int w = threadIdx.x; w < wp; w += blockDim.x) {
@@ -541,9 +551,13 @@ __global__ void __launch_bounds__(256)
             ones += __popcll(bits[w]);
         }
         ones = __reduce_add_sync(0xffffffffu, ones);
-        if (lane == 0 && ones)
-            atomicAdd(reinterpret_cast<unsigned long long *>(counters + 2), static_cast<unsigned long long>(ones));
-        if (threadIdx.x == 0 && cnt > 0) atomicAdd(counters + 1, 1u);  // a path too long for the walk
+        if (lane == 0 && ones) atomicAdd(&ones_s, ones);
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            atomicAdd(reinterpret_cast<unsigned long long *>(counters + 2), static_cast<unsigned long long>(ones_s));
+            if (cnt > 0) atomicAdd(counters + 1, 1u);  // a path too long for the walk
+            else if (ones_s != expanded) atomicAdd(violations, 1ull);
+        }
         __syncthreads();
     }
 }
@@ -862,15 +876,15 @@ cudaError_t row_iteration(const int *ptr, const int *col, int n, int64_t wp, uin
 }
 
 cudaError_t reach_rows(const int *ptr, const int *col, int n, int64_t wp, uint64_t *out, int *open_rows,
-                       unsigned *counters, cudaStream_t s) {
+                       unsigned *counters, unsigned long long *violations, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
     if (wp > 256) return cudaErrorInvalidValue;  // 16-bit names of constants, rows in shared memory
     const size_t smem = 8 * (static_cast<size_t>(wp) + kReachFront / 2 + 1) * sizeof(uint64_t);
     reach_rows_kernel<<<static_cast<unsigned>((n + 7) / 8), 256, smem, s>>>(ptr, col, n, static_cast<int>(wp), out,
-                                                                          open_rows, counters);
+                                                                          open_rows, counters, violations);
     const size_t smem_open = static_cast<size_t>(wp) * 2 * sizeof(uint64_t) + static_cast<size_t>(wp) * 64 * sizeof(uint16_t);
     reach_open_kernel<<<static_cast<unsigned>(num_sms() * 4), 256, smem_open, s>>>(ptr, col, n, static_cast<int>(wp),
-                                                                                 out, open_rows, counters);
+                                                                                 out, open_rows, counters, violations);
     return cudaGetLastError();
 }
 

@@ -191,9 +191,10 @@ cudaError_t row_iteration(const int *ptr, const int *col, int n, int64_t wp, uin
 // Rows i < n of the model (what paths of one edge or more reach from i) by breadth-first walks over the
 // CSR, wp <= 256 words per row.  counters (zeroed by the caller): [0] rows that needed the second, CTA-wide
 // walk, [1] rows given up (out is then incomplete), [2], [3] the ones of the rows written (64 bits).
-// open_rows: n ints of scratch.
+// open_rows: n ints of scratch.  *violations += rows that fail their certificate (not every constant
+// reached has been expanded).
 cudaError_t reach_rows(const int *ptr, const int *col, int n, int64_t wp, uint64_t *out, int *open_rows,
-                       unsigned *counters, cudaStream_t s);
+                       unsigned *counters, unsigned long long *violations, cudaStream_t s);
 // Bit-matrix helpers for same generation (np x np bits, wp = np / 64 words per row).
 // dst = src^T (np a multiple of 64; dst distinct from src); nothing if *skip == 0.
 cudaError_t bits_transpose(const uint64_t *src, uint64_t *dst, int np, int64_t wp, const unsigned long long *skip,

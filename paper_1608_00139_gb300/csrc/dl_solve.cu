@@ -676,13 +676,12 @@ dl_status tc_auto(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &a
         NEED(open_rows);
         auto *counters = reinterpret_cast<unsigned *>(ws.scal + SC_OPEN);
         CK(cudaMemsetAsync(counters, 0, 2 * sizeof(unsigned long long), s));
-        CK(reach_rows(ptr, col, n, wp, model, open_rows, counters, s));
+        CK(reach_rows(ptr, col, n, wp, model, open_rows, counters, ws.scal + SC_VIOL, s));  // (SC_VIOL is 0 still)
         launches += 2;
         if ((rc = read_scalars(ws, s))) return rc;
         const auto *h = reinterpret_cast<const unsigned *>(host_scal(ws) + SC_OPEN);
         if (h[1] == 0) {
             host_scal(ws)[SC_ONES] = host_scal(ws)[SC_OPEN + 1];
-            host_scal(ws)[SC_VIOL] = 0;
             converged = emitted = true;
         }
     }
