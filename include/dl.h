@@ -291,7 +291,8 @@ DL_API dl_status dl_sg_real(dl_ctx *ctx, int32_t n, const uint8_t *P, const uint
  * refine_tol * eps (DL_ENOTCONV after 100000 steps); DL_PATH_AUTO at n <= 16384 sums the series in
  * FP32 for the corrections of an FP64 iterate until its FP64 residual is at most refine_tol * eps
  * (relations on which that is slow take the FP64 series); stats->guard_flagged counts the 64-bit bit
- * words where R~2 > 0 differs from the model (nonzero only under FP64 underflow).
+ * words where R~2 > 0 differs from the model: entries that underflowed, or so deep that the series
+ * stopped above them.
  * Paths: DL_PATH_AUTO (model; R~2 if out_rtilde is not NULL), DL_PATH_FP64 (model and the series,
  * out_rtilde optional), DL_PATH_BOOL_FP8 (model only: a non-NULL out_rtilde returns DL_EINVAL);
  * DL_PATH_MIXED returns DL_ENOTIMPL.  thr must be 0.

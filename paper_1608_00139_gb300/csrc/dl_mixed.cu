@@ -1025,10 +1025,17 @@ __global__ void __launch_bounds__(kFirstThreads) first_product_kernel(const int 
 // Right-hand sides with at most this many facts per constant take the gathered first product.
 constexpr int64_t kSparseFirstDegree = 12;
 
-// From this share of ones in E the residual's updates are a product with E, below it gathers: at n = 8192
-// the product of both slices takes 1.3 ms and grows with n^3, the gathers 0.57 ms at 8 ones a row, of
-// which all but 0.3 grow with the ones and n^2.  (The residual formed as a whole takes 4.2 ms at 82
-// ones a row, 0.97 at 8, once instead of in every step: 36.8 -> 25.7 and 20.7 -> 18.7 ms.)
+// From this share of ones in E the residual's updates are a product with E, below it gathers.  The product of
+// both slices grows with n^3 (1.3 ms at n = 8192, and 0.34 for the sums), the gathers with the ones and n.  The
+// refinement of a solve with R~, all updates by products / all by gathers, ms by ones a row:
+//   n = 8192   8: 14.7 / 10.5   16: 16.2 / 13.1   32: 18.6 / 18.4   48: 18.9 / 22.4   64: 19.2 / 25.6   80: 19.4 / 28.9
+//   n = 4096   8: 2.70 / 2.28   16: 2.97 / 2.80   24: 3.10 / 3.23   32: 3.30 / 3.81   64: 3.42 / 5.26
+//   n = 2048   8: 0.68 / 0.64   16: 0.71 / 0.74   32: 0.79 / 1.02   64: 0.85 / 1.44
+//   n = 1000   8: 0.35 / 0.30   24: 0.37 / 0.36   32: 0.38 / 0.39   64: 0.51 / 0.63
+// so the two cross near 32, 20, 14 and 28 ones a row (0.4, 0.5, 0.7 and 2.8 %): the line suits n = 2048, and
+// costs up to 0.05 ms at n = 1000 (products from 9 ones a row) and, from 32 to 73 ones a row, 6 ms at n = 8192
+// (gathers).  Formed as a whole in every step, as without room for the sums, the residual takes 4.2 ms at 82
+// ones a row and 0.97 at 8.
 constexpr double kSliceDensity = 0.009;
 
 // Consecutive NVTX ranges, one open at a time.

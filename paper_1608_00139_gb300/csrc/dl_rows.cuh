@@ -237,9 +237,9 @@ __device__ __forceinline__ void or_shared(uint64_t *word, uint64_t e) {
 // to a run of bits in `buf` (tile_words words of shared memory), from which word w of row r is read at
 // its bit offset and handed to put(r, w, facts).  Bound by the read: what a row costs beyond its bytes (a
 // warp to a row, pieces at the row's own misalignment) took more issue slots than the 6 operations a
-// piece (1.43 GB of rows of about 1 KB: 547 us with a warp to a row, 304 us so).  A byte that is neither 0 nor 1 sets *bad for some thread; bytes outside the matrix
-// are cleared (only the first and the last row's pieces can hold any).  Ends with the CTA's threads in
-// their put calls: no barrier behind them.
+// piece (1.43 GB of rows of about 1 KB: 547 us with a warp to a row, 304 us so).  A byte that is neither 0
+// nor 1 sets *bad for some thread; bytes outside the matrix are cleared (only the first and the last row's
+// pieces can hold any).  Ends with the CTA's threads in their put calls: no barrier behind them.
 constexpr int kTileBytes = 32768;       // a tile where there are many
 constexpr int kTileBytesSmall = 8192;   // and of one matrix of at most kTileSmallN rows (512 tiles at 2048)
 constexpr int kTileSmallN = 4096;
@@ -293,7 +293,6 @@ __device__ __forceinline__ void pack_tile(const uint8_t *__restrict__ E, int n, 
         put(r0 + i, w, e);
     }
 }
-
 
 // One warp writes the successor list of row r into col[pos0 .. pos1) from its packed bits
 // (I + E: the identity bit belongs to E only when the row holds pos1 - pos0 ones).

@@ -80,7 +80,7 @@ __device__ __forceinline__ void cluster_barrier() {
 
 // The 16 columns 16 q .. + 16 of a row of E bytes: their low bits, and *bad for other bytes.  Any
 // alignment: the one or two aligned 16-byte chunks that hold them (no other chunk is touched).
-__device__ __forceinline__ uint32_t pack16(const uint8_t *row, int n, int q, bool *bad) {
+__device__ __forceinline__ uint32_t pack16_at(const uint8_t *row, int n, int q, bool *bad) {
     const int c0 = 16 * q;
     if (c0 >= n) return 0u;
     const int m = min(16, n - c0);  // columns that exist
@@ -130,7 +130,7 @@ __global__ void __launch_bounds__(kSmallThreads)
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 const int t = t0 + u * kSmallThreads;
-                v[u] = t < items ? pack16(E + static_cast<int64_t>(row0 + t / (4 * w)) * n, n, t % (4 * w), &bad) : 0u;
+                v[u] = t < items ? pack16_at(E + static_cast<int64_t>(row0 + t / (4 * w)) * n, n, t % (4 * w), &bad) : 0u;
             }
 #pragma unroll
             for (int u = 0; u < 4; ++u) {

@@ -2393,7 +2393,7 @@ dl_status trans_real_first(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const Sol
 // corrections of an FP64 iterate whose FP64 residual decides (an FP64 step is bound by the two FP64
 // lanes of an SM, an FP32 one by its bytes); relations whose series is slow fall back to FP64.  The
 // positive entries are compared with the model (guard_flagged counts the bit words where they
-// differ: only underflow can make them).
+// differ: entries that underflowed, or that the series stopped above).
 dl_status solve_transposed(dl_ctx *ctx, Workspace &ws, cudaStream_t s, const SolveArgs &a, dl_stats *st) {
     if (a.thr != 0.0) {
         set_error("thr must be 0: the model is R~ > 0 (Theorem 2)");
